@@ -5,8 +5,8 @@
 // logits[r, v] = sum_h hidden[r, h] * weight[v, h] is a dense contraction: bf16 operands on the tcgen05 tensor cores, f32
 // accumulators in tensor memory.  One persistent CTA per SM walks over 128-token tiles of the vocabulary (tile = CTA index,
 // + grid size, ...): every weight tile leaves HBM once and meets all rows (up to 256: two 128-row accumulators side by
-// side on one weight stream); the hidden states (a few MB) are re-read from L2.  Roles: warp 0 requests tiles by TMA
-// (64-element K slices, 128-byte swizzle, a ring of 192 KB cut into 4 to 12 stages), warp 1 issues the products and commits them to the
+// side on one weight stream); the hidden states (a few MB) are re-read from L2.  Roles: warps 0 and 6 request weight
+// and hidden-state tiles by TMA (64-element K slices, 128-byte swizzle, a ring of 192 KB cut into 4 to 12 stages), warp 1 issues the products and commits them to the
 // ring's "empty" barriers and to the accumulator's "full" barrier, warps 2-5 read a finished accumulator (one row per
 // thread), keep the running (maximum, first token that reaches it) per row across the CTA's tiles while the next tile's
 // products fill the other accumulator.  A second small kernel merges the CTAs' candidates per row (greater logit, then
@@ -28,8 +28,9 @@ using namespace tcp;
 constexpr int kLmBM = 128;        // rows per accumulator (tensor-memory lanes)
 constexpr int kLmBK = 64;         // hidden elements per stage (one 128-byte swizzled row)
 constexpr int kLmTileBytes = kLmBM * kLmBK * 2;  // 16 KB: one 128 x 64 bf16 operand tile
-constexpr int kLmThreads = 192;   // producer warp, issuer warp, four epilogue warps
+constexpr int kLmThreads = 224;   // weight producer, issuer, four epilogue warps, hidden-state producer
 constexpr int kLmRowsPerLaunch = 2 * kLmBM;
+constexpr int kLmMaxParts = 160;  // CTAs of a launch: one per SM, at most this many
 
 // Vocabulary entries per tile: a launch-time choice (a multiple of 32), so that the tiles spread evenly over the CTAs
 // (V = 32000 on 148 SMs: 143 tiles of 224 instead of 250 of 128 in two uneven rounds).  Two row tiles leave room for 128.
@@ -51,9 +52,9 @@ struct LmParams {
     int a_rows;      // rows of a hidden-state box (a multiple of 32, <= 128): 26 rows need not move 128
     int stages;      // ring stages of a_rows * NM + bn rows of 128 bytes each
     int k_steps;     // H / 64
-    float* part_v;   // [grid][256][KT] the CTAs' best logits per row, best first
-    int32_t* part_t; // [grid][256][KT] and their tokens
-    int32_t* status; // one word (may be null): S4C_SEQ_TIMEOUT is OR-ed in when a wait was given up
+    float* part_v;   // [256][kLmMaxParts][KT] per row the CTAs' best logits, best first
+    int32_t* part_t; // [256][kLmMaxParts][KT] and their tokens
+    int32_t* gave_up; // [kLmMaxParts]: 1 where the CTA gave up a wait
 };
 
 template <int NM, int KT>
@@ -76,19 +77,17 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
     volatile int* tail = reinterpret_cast<volatile int*>(gen + Cfg::kRingBytes + Cfg::kBars * 8);
     volatile int* tmem_slot = tail;       // written by tcgen05.alloc
     volatile int* dead = tail + 1;        // a wait was given up
-    volatile int* issued_s = tail + 2;    // stage fills the producer has requested
-    auto sA = [&](int s, int t) { return base + s * stage_bytes + t * a_bytes; };
-    auto sB = [&](int s) { return base + s * stage_bytes + NM * a_bytes; };
+    volatile int* issued_s = tail + 2;    // [2] stage fills the producers have requested
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int bn = prm.bn;
     const int n_tiles = (prm.V + bn - 1) / bn;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 1), mbar_init(EMPTY(s), 1);
+        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 2), mbar_init(EMPTY(s), 1);
         for (int b = 0; b < 2; ++b) mbar_init(ACC_FULL(b), 1), mbar_init(ACC_EMPTY(b), 4);
         mbar_init(DRAIN, 1);
         mbar_fence_init();
-        *dead = 0, *issued_s = 0;
+        *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
         tma_prefetch_desc(&map_h), tma_prefetch_desc(&map_w);
     }
     if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), Cfg::kTmemCols);
@@ -96,49 +95,68 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = (uint32_t)*tmem_slot;
+    griddep_launch_dependents();
+    griddep_wait();  // the set-up above ran beside the kernel in front
     auto TM = [&](int buf, int t) { return tmem + (uint32_t)((buf * NM + t) * Cfg::kMaxBN); };
 
-    if (warp == 0) {
-        // ================= producer: hidden-state and weight tiles into the ring =================
-        if (lane == 0) {
+    // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: such a
+    // thread's instructions per slice are time the stream waits, so the two operands have a producer each.
+    if (warp == 0 || warp == 6) {
+        // ================= producers: weight tiles (warp 0) and hidden-state tiles (warp 6) into the ring =================
+        if (elect_one()) {
+            const bool states = warp == 6;
+            const int tx = states ? NM * a_bytes : stage_bytes - NM * a_bytes;
             int fill = 0, s = 0;
-            uint32_t ph = 0;  // the ring pass's parity (stage and parity are stepped, not divided out: S is not a constant)
+            uint32_t ph = 1, at = base + (states ? 0 : NM * a_bytes);  // the ring pass's parity; the stage's address
             bool ok = true;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
-                for (int ks = 0; ks < prm.k_steps; ++ks, ++fill, s = s + 1 == S ? 0 : s + 1, ph ^= (s == 0)) {
-                    ok = mbar_wait(EMPTY(s), ph ^ 1, dead);
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                const int row = tile * bn;
+                for (int ks = 0; ks < prm.k_steps; ++ks, ++fill) {
+                    ok = mbar_wait(EMPTY(s), ph, dead);
                     if (!ok) break;
-                    mbar_expect_tx(FULL(s), stage_bytes);
+                    mbar_expect_tx(FULL(s), tx);
+                    if (states) {
 #pragma unroll
-                    for (int t = 0; t < NM; ++t) tma_load_2d(sA(s, t), &map_h, FULL(s), ks * kLmBK, prm.row0 + t * kLmBM);
-                    tma_load_2d(sB(s), &map_w, FULL(s), ks * kLmBK, tile * bn);
+                        for (int t = 0; t < NM; ++t) tma_load_2d(at + t * a_bytes, &map_h, FULL(s), ks * kLmBK, prm.row0 + t * kLmBM);
+                    } else {
+                        tma_load_2d(at, &map_w, FULL(s), ks * kLmBK, row);
+                    }
+                    at += stage_bytes;
+                    if (++s == S) s = 0, ph ^= 1, at -= S * stage_bytes;
                 }
-            *issued_s = fill;
+            }
+            issued_s[states ? 1 : 0] = fill;
         }
         __syncwarp();
     } else if (warp == 1) {
         // ================= issuer: acc[t] = hidden tile t x weight tile^T over all K slices =================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc_bf16(kLmBM, bn, false);
+            const uint64_t h0 = smem_desc_sw128(base, 16, 1024), step = (uint64_t)(stage_bytes >> 4), t_step = (uint64_t)(a_bytes >> 4);
+            uint64_t h_desc = h0;
             int it = 0, s = 0;
             uint32_t ph = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++it) {
                 const int buf = it & 1;
                 ok = mbar_wait(ACC_EMPTY(buf), ((it >> 1) & 1) ^ 1, dead);  // the epilogue has read this buffer
-                for (int ks = 0; ks < prm.k_steps && ok; ++ks, s = s + 1 == S ? 0 : s + 1, ph ^= (s == 0)) {
+                const uint32_t acc = TM(buf, 0);
+                uint32_t accumulate = 0;
+                for (int ks = 0; ks < prm.k_steps && ok; ++ks) {
                     ok = mbar_wait(FULL(s), ph, dead);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t b_desc = smem_desc_sw128(sB(s), 16, 1024);
+                    const uint64_t w_desc = h_desc + NM * t_step;
 #pragma unroll
-                    for (int t = 0; t < NM; ++t) {
-                        const uint64_t a_desc = smem_desc_sw128(sA(s, t), 16, 1024);
+                    for (int kk = 0; kk < kLmBK / 16; ++kk) {  // 32 bytes per K step inside the swizzled row (field unit: 16 B)
 #pragma unroll
-                        for (int kk = 0; kk < kLmBK / 16; ++kk)  // 32 bytes per K step inside the swizzled row (field unit: 16 B)
-                            tc_mma_bf16(TM(buf, t), a_desc + 2u * kk, b_desc + 2u * kk, idesc, (ks > 0 || kk > 0) ? 1u : 0u);
+                        for (int t = 0; t < NM; ++t)
+                            tc_mma_bf16(acc + t * Cfg::kMaxBN, h_desc + t * t_step + 2u * kk, w_desc + 2u * kk, idesc, accumulate);
+                        accumulate = 1;
                     }
                     tc_commit(EMPTY(s));  // the stage is free once these products have read it
+                    h_desc += step;
+                    if (++s == S) s = 0, ph ^= 1, h_desc = h0;
                 }
                 if (ok) tc_commit(ACC_FULL(buf));
             }
@@ -228,29 +246,29 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
             const int r = t * kLmBM + q * 32 + lane;
 #pragma unroll
             for (int j = 0; j < KT; ++j) {
-                prm.part_v[((size_t)blockIdx.x * kLmRowsPerLaunch + r) * KT + j] = best_v[t][j];
-                prm.part_t[((size_t)blockIdx.x * kLmRowsPerLaunch + r) * KT + j] = best_t[t][j];
+                prm.part_v[((size_t)r * kLmMaxParts + blockIdx.x) * KT + j] = best_v[t][j];
+                prm.part_t[((size_t)r * kLmMaxParts + blockIdx.x) * KT + j] = best_t[t][j];
             }
         }
     }
-    griddep_launch_dependents();
     __syncthreads();
+    if (threadIdx.x == 0) prm.gave_up[blockIdx.x] = *dead ? 1 : 0;
     if (*dead) {
         // a wait was given up: nothing more is issued; what is still in flight lands before shared and tensor memory go
         if (threadIdx.x == 0) {
-            const int issued = *issued_s;
+            const int lo = min(issued_s[0], issued_s[1]), hi = max(issued_s[0], issued_s[1]);
+            for (int f = lo; f < hi; ++f) mbar_arrive(FULL(f % S));  // for the producer that stopped first
             for (int s = 0; s < S; ++s) {
                 int last = -1;  // the last fill requested into stage s
-                for (int f = s; f < issued; f += S) last = f;
+                for (int f = s; f < hi; f += S) last = f;
                 if (last >= 0) mbar_drain(FULL(s), (last / S) & 1);
             }
         }
-        if (warp == 1 && lane == 0) {
+        if (warp == 1 && elect_one()) {
             tc_commit(DRAIN);
             mbar_drain(DRAIN, 0);
         }
         __syncthreads();
-        if (threadIdx.x == 0 && prm.status) atomicOr(prm.status, S4C_SEQ_TIMEOUT);
     }
     if (warp == 1) {
         tc_fence_after();
@@ -258,50 +276,70 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
     }
 }
 
-// Per row: the k best of the CTAs' candidates, best first (greater logit, then lower token).  One warp per row: the
-// candidates (at most 1024 CTAs x 8) come into shared memory once -- independent loads, in flight together --, then round j
-// takes the best candidate that ranks after round j-1's (the candidates' tokens are distinct).
-constexpr int kLmMergeRows = 4;      // rows (warps) per CTA
-constexpr int kLmMergeStage = 1184;  // candidates staged per row: 148 CTAs x 8; beyond that the rounds read global memory
-__global__ void __launch_bounds__(kLmMergeRows * 32)
-lm_head_merge_kernel(const float* __restrict__ part_v, const int32_t* __restrict__ part_t, int n_parts, int kt, int rows, int k,
-                     int32_t* __restrict__ token, float* __restrict__ logit) {
-    __shared__ float sv[kLmMergeRows][kLmMergeStage];
-    __shared__ int st[kLmMergeRows][kLmMergeStage];
+// Per row: the k best of the CTAs' candidates, best first (greater logit, then lower token; the tokens are distinct).  One warp
+// per row: a lane takes the lists of CTAs lane, lane + 32, ... into registers -- they are sorted, so only their heads
+// compete -- and each of the k rounds takes the warp's best head and moves that list up.  (With the candidates in shared
+// memory and every round scanning all of them, four rounds over 148 lists of 4 took 16 us.)
+constexpr int kLmLists = kLmMaxParts / 32;
+template <int KT>
+__global__ void __launch_bounds__(32)
+lm_head_merge_kernel(const float* __restrict__ part_v, const int32_t* __restrict__ part_t, const int32_t* __restrict__ gave_up, int n_parts,
+                     int k, int first, int32_t* __restrict__ token, float* __restrict__ logit, int32_t* __restrict__ status) {
+    griddep_launch_dependents();
     griddep_wait();
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * kLmMergeRows + w;
-    if (r >= rows) return;
-    const int total = n_parts * kt;  // candidate c: CTA c / kt, rank c % kt
-    const bool staged = total <= kLmMergeStage;
-    auto at = [&](int c) { return ((size_t)(c / kt) * kLmRowsPerLaunch + r) * kt + (c % kt); };
-    if (staged) {
-        for (int c = lane; c < total; c += 32) sv[w][c] = part_v[at(c)], st[w][c] = part_t[at(c)];
-        __syncwarp();
+    const int lane = threadIdx.x, r = blockIdx.x;
+    float v[kLmLists][KT];
+    int t[kLmLists][KT];
+#pragma unroll
+    for (int i = 0; i < kLmLists; ++i) {
+        const int part = i * 32 + lane;
+        const bool in = part < n_parts;
+        const size_t at = ((size_t)r * kLmMaxParts + (in ? part : 0)) * KT;
+        if (KT == 1) {
+            v[i][0] = part_v[at], t[i][0] = part_t[at];
+        } else {
+#pragma unroll
+            for (int j = 0; j < KT; j += 4) {
+                const float4 a = *reinterpret_cast<const float4*>(part_v + at + j);
+                const int4 c = *reinterpret_cast<const int4*>(part_t + at + j);
+                v[i][j] = a.x, v[i][j + 1] = a.y, v[i][j + 2] = a.z, v[i][j + 3] = a.w;
+                t[i][j] = c.x, t[i][j + 1] = c.y, t[i][j + 2] = c.z, t[i][j + 3] = c.w;
+            }
+        }
+        if (!in) t[i][0] = INT_MAX;  // "none": ranks after everything
     }
-    float pv = INFINITY;
-    int pt = -1;
+    if (status && r == 0) {
+        int any = 0;
+        for (int i = lane; i < n_parts; i += 32) any |= gave_up[i];
+        any = __any_sync(0xffffffffu, any);
+        if (lane == 0) *status = (first ? 0 : *status) | (any ? S4C_SEQ_TIMEOUT : 0);
+    }
     for (int j = 0; j < k; ++j) {
         float bv = -INFINITY;
         int bt = INT_MAX;
-        for (int c = lane; c < total; c += 32) {
-            const float v = staged ? sv[w][c] : part_v[at(c)];
-            const int t = staged ? st[w][c] : part_t[at(c)];
-            const bool after = v < pv || (v == pv && t > pt);
-            if (t != INT_MAX && after && (v > bv || (v == bv && t < bt))) bv = v, bt = t;
-        }
+#pragma unroll
+        for (int i = 0; i < kLmLists; ++i)
+            if (t[i][0] != INT_MAX && (bt == INT_MAX || v[i][0] > bv || (v[i][0] == bv && t[i][0] < bt))) bv = v[i][0], bt = t[i][0];
+        const int mine = bt;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
             const int ot = __shfl_xor_sync(0xffffffffu, bt, o);
-            if (ov > bv || (ov == bv && ot < bt)) bv = ov, bt = ot;
+            if (ot != INT_MAX && (bt == INT_MAX || ov > bv || (ov == bv && ot < bt))) bv = ov, bt = ot;
         }
-        pv = bv, pt = bt;
         if (lane == 0) {
             token[(size_t)r * k + j] = bt == INT_MAX ? -1 : bt;  // fewer than k comparable logits in the row (k > V, NaN)
             if (logit) logit[(size_t)r * k + j] = bt == INT_MAX ? -INFINITY : bv;
         }
-        if (bt == INT_MAX) pv = -INFINITY, pt = INT_MAX;  // nothing ranks after "none"
+        if (mine == bt && bt != INT_MAX) {
+#pragma unroll
+            for (int i = 0; i < kLmLists; ++i)
+                if (t[i][0] == bt) {
+#pragma unroll
+                    for (int m = 0; m + 1 < KT; ++m) v[i][m] = v[i][m + 1], t[i][m] = t[i][m + 1];
+                    t[i][KT - 1] = INT_MAX;
+                }
+        }
     }
 }
 
@@ -312,7 +350,8 @@ struct TokWalkShared {
     int32_t tgt[S4C_MAX_T];
     int depth[S4C_MAX_T];
     uint32_t anc[S4C_MAX_T][S4C_MASK_WORDS];
-    int flag;
+    uint32_t hit[S4C_MASK_WORDS];
+    int flag, best;
 };
 
 __global__ void __launch_bounds__(128)
@@ -321,6 +360,8 @@ accept_tokens_kernel(const int32_t* __restrict__ target_token, const int32_t* __
                      int32_t* __restrict__ accept_len, int32_t* __restrict__ path, int32_t* __restrict__ next_token,
                      int32_t* __restrict__ status) {
     __shared__ TokWalkShared sh;
+    griddep_launch_dependents();
+    griddep_wait();
     const int b = blockIdx.x, tid = threadIdx.x;
     const int n = n_nodes ? n_nodes[b] : T;
     int32_t* pth = path + (size_t)b * (max_depth + 1);
@@ -345,22 +386,25 @@ accept_tokens_kernel(const int32_t* __restrict__ target_token, const int32_t* __
         if (tid == 0) accept_len[b] = -1, next_token[b] = -1;
         return;
     }
-    if (tid != 0) return;
-    // a node is accepted when every node on its path carries the target's choice at its parent; parents come first, so
-    // one pass in index order settles all nodes (at most 128): reuse the depth array's sign for "accepted"
-    int end = 0;
-    for (int i = 1; i < n; ++i) {
-        const int p = sh.par[i];
-        const bool ok = sh.depth[p] >= 0 && sh.tok[i] == sh.tgt[p];
-        if (!ok)
-            sh.depth[i] = -1 - sh.depth[i];  // not accepted (depth kept, negated)
-        else if (sh.depth[i] > sh.depth[end])
-            end = i;  // the deepest accepted node, the lowest index among equals
+    // A node is accepted when every node on its path carries the target's choice at its parent: one bit per node (a thread
+    // each, 128 threads), and a node's path is its ancestor mask.  The deepest accepted node ends the path, the lowest
+    // index among equals.  (One thread going through the nodes in order took 2 us for 64 of them.)
+    const bool hit = tid == 0 || (tid < n && sh.tok[tid] == sh.tgt[sh.par[tid]]);
+    const uint32_t bits = __ballot_sync(0xffffffffu, hit);
+    if ((tid & 31) == 0) sh.hit[tid >> 5] = bits;
+    if (tid == 0) sh.best = 0;
+    for (int j = tid; j <= max_depth; j += blockDim.x) pth[j] = -1;
+    __syncthreads();
+    if (tid < n) {
+        bool ok = true;
+#pragma unroll
+        for (int w = 0; w < S4C_MASK_WORDS; ++w) ok = ok && (sh.anc[tid][w] & ~sh.hit[w]) == 0;
+        if (ok) atomicMax(&sh.best, sh.depth[tid] * S4C_MAX_T + (S4C_MAX_T - 1 - tid));
     }
-    for (int j = 0; j <= max_depth; ++j) pth[j] = -1;
-    for (int t = end; t >= 0; t = sh.par[t]) pth[sh.depth[t]] = t;
-    accept_len[b] = sh.depth[end];
-    next_token[b] = sh.tgt[end];
+    __syncthreads();
+    const int end = S4C_MAX_T - 1 - sh.best % S4C_MAX_T;
+    if (tid < n && (sh.anc[end][tid >> 5] >> (tid & 31) & 1u)) pth[sh.depth[tid]] = tid;  // (written over the -1 of before the barriers)
+    if (tid == 0) accept_len[b] = sh.depth[end], next_token[b] = sh.tgt[end];
 }
 
 // ----------------------------------------------------------------------------- host side
@@ -406,14 +450,30 @@ static int lm_sm_count() {
 }
 
 static inline int lm_kt(int k) { return k <= 1 ? 1 : (k <= 4 ? 4 : 8); }  // candidates a thread keeps per row
-static inline size_t lm_ws_layout(int V, int k, char* base, float** part_v, int32_t** part_t) {
-    const size_t parts = (size_t)std::min(ceil_div(V, 64), 1024);  // at most one CTA per tile (64 entries or more), never more than this
+static inline size_t lm_ws_layout(int k, char* base, float** part_v, int32_t** part_t, int32_t** gave_up) {
     size_t off = 0;
     if (part_v) *part_v = reinterpret_cast<float*>(base + off);
-    off += round_up(parts * kLmRowsPerLaunch * lm_kt(k) * sizeof(float), 256);
+    off += round_up((size_t)kLmMaxParts * kLmRowsPerLaunch * lm_kt(k) * sizeof(float), 256);
     if (part_t) *part_t = reinterpret_cast<int32_t*>(base + off);
-    off += round_up(parts * kLmRowsPerLaunch * lm_kt(k) * sizeof(int32_t), 256);
-    return off;
+    off += round_up((size_t)kLmMaxParts * kLmRowsPerLaunch * lm_kt(k) * sizeof(int32_t), 256);
+    if (gave_up) *gave_up = reinterpret_cast<int32_t*>(base + off);
+    return off + round_up(kLmMaxParts * sizeof(int32_t), 256);
+}
+
+// Launched programmatically dependent: set-up overlaps the tail of the kernel in front.
+template <typename... KArgs, typename... Args>
+static s4c_status lm_dependent_launch(void (*kernel)(KArgs...), int grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1), cfg.blockDim = dim3(threads, 1, 1), cfg.dynamicSmemBytes = smem, cfg.stream = stream;
+    cfg.attrs = &pdl, cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...) != cudaSuccess) {
+        cudaGetLastError();
+        return S4C_ERR_CUDA;
+    }
+    return S4C_OK;
 }
 
 template <int NM, int KT>
@@ -424,16 +484,22 @@ static s4c_status lm_launch(const CUtensorMap& map_h, const CUtensorMap& map_w, 
         cudaGetLastError();
         return S4C_ERR_CUDA;
     }
-    lm_head_greedy_kernel<NM, KT><<<grid, kLmThreads, Cfg::kSmemBytes, stream>>>(map_h, map_w, prm);
-    S4C_RETURN_IF_CUDA_ERROR();
-    return S4C_OK;
+    return lm_dependent_launch(lm_head_greedy_kernel<NM, KT>, grid, kLmThreads, Cfg::kSmemBytes, stream, map_h, map_w, prm);
+}
+template <int KT>
+static s4c_status lm_run(const CUtensorMap& map_h, const CUtensorMap& map_w, const LmParams& prm, int grid, int k, int32_t* token, float* logit,
+                         int32_t* status, cudaStream_t stream) {
+    const s4c_status st = prm.rows > kLmBM ? lm_launch<2, KT>(map_h, map_w, prm, grid, stream) : lm_launch<1, KT>(map_h, map_w, prm, grid, stream);
+    if (st != S4C_OK) return st;
+    return lm_dependent_launch(lm_head_merge_kernel<KT>, prm.rows, 32, 0, stream, (const float*)prm.part_v, (const int32_t*)prm.part_t,
+                               (const int32_t*)prm.gave_up, grid, k, prm.row0 == 0 ? 1 : 0, token, logit, status);
 }
 
 }  // namespace s4c
 
 extern "C" size_t s4c_lm_head_topk_workspace_bytes(int R, int V, int H, int k) {
     if (R < 1 || V < 1 || H < 1 || k < 1 || k > 8) return 0;
-    return s4c::lm_ws_layout(V, k, nullptr, nullptr, nullptr);
+    return s4c::lm_ws_layout(k, nullptr, nullptr, nullptr, nullptr);
 }
 
 extern "C" s4c_status s4c_lm_head_topk(const void* hidden, const void* weight, int R, int V, int H, int k, int32_t* token,
@@ -445,22 +511,15 @@ extern "C" s4c_status s4c_lm_head_topk(const void* hidden, const void* weight, i
     if (k > 8) return S4C_ERR_UNSUPPORTED;
     if (!aligned16(hidden) || !aligned16(weight)) return S4C_ERR_ALIGN;
     if (R == 0) return S4C_OK;
-    float* part_v;
-    int32_t* part_t;
-    const size_t need = lm_ws_layout(V, k, nullptr, nullptr, nullptr);
+    LmParams prm;
+    const size_t need = lm_ws_layout(k, nullptr, nullptr, nullptr, nullptr);
     if (!workspace || workspace_bytes < need || !aligned256(workspace)) return S4C_ERR_WORKSPACE;
-    lm_ws_layout(V, k, static_cast<char*>(workspace), &part_v, &part_t);
+    lm_ws_layout(k, static_cast<char*>(workspace), &prm.part_v, &prm.part_t, &prm.gave_up);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    if (status && cudaMemsetAsync(status, 0, sizeof(int32_t), stream) != cudaSuccess) {
-        cudaGetLastError();
-        return S4C_ERR_CUDA;
-    }
-    const int sms = std::min(lm_sm_count(), 1024), kt = lm_kt(k);
+    const int sms = std::min(lm_sm_count(), kLmMaxParts), kt = lm_kt(k);
     // groups of up to 256 rows; each group streams the weights once
     for (int row0 = 0; row0 < R; row0 += kLmRowsPerLaunch) {
-        LmParams prm;
         prm.rows = std::min(kLmRowsPerLaunch, R - row0), prm.row0 = row0, prm.V = V, prm.k_steps = H / kLmBK;
-        prm.part_v = part_v, prm.part_t = part_t, prm.status = status;
         // tile width: the one that costs the fewest (rounds of tiles over the CTAs) x (entries per tile)
         prm.bn = 128;
         if (prm.rows <= kLmBM) {
@@ -481,21 +540,12 @@ extern "C" s4c_status s4c_lm_head_topk(const void* hidden, const void* weight, i
         CUtensorMap map_h, map_w;
         if (!lm_make_map(&map_h, hidden, (uint64_t)R, H, prm.a_rows) || !lm_make_map(&map_w, weight, (uint64_t)V, H, prm.bn))
             return S4C_ERR_CUDA;
-        const s4c_status st = kt == 1   ? (two ? lm_launch<2, 1>(map_h, map_w, prm, grid, stream) : lm_launch<1, 1>(map_h, map_w, prm, grid, stream))
-                              : kt == 4 ? (two ? lm_launch<2, 4>(map_h, map_w, prm, grid, stream) : lm_launch<1, 4>(map_h, map_w, prm, grid, stream))
-                                        : (two ? lm_launch<2, 8>(map_h, map_w, prm, grid, stream) : lm_launch<1, 8>(map_h, map_w, prm, grid, stream));
+        int32_t* tok = token + (size_t)row0 * k;
+        float* lgt = logit ? logit + (size_t)row0 * k : nullptr;
+        const s4c_status st = kt == 1   ? lm_run<1>(map_h, map_w, prm, grid, k, tok, lgt, status, stream)
+                              : kt == 4 ? lm_run<4>(map_h, map_w, prm, grid, k, tok, lgt, status, stream)
+                                        : lm_run<8>(map_h, map_w, prm, grid, k, tok, lgt, status, stream);
         if (st != S4C_OK) return st;
-        cudaLaunchAttribute pdl;
-        pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        pdl.val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.stream = stream, cfg.attrs = &pdl, cfg.numAttrs = 1;
-        cfg.gridDim = dim3(ceil_div(prm.rows, kLmMergeRows), 1, 1), cfg.blockDim = dim3(kLmMergeRows * 32, 1, 1);  // a warp per row
-        if (cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const float*)part_v, (const int32_t*)part_t, grid, kt, prm.rows, k,
-                               token + (size_t)row0 * k, logit ? logit + (size_t)row0 * k : (float*)nullptr) != cudaSuccess) {
-            cudaGetLastError();
-            return S4C_ERR_CUDA;
-        }
     }
     return S4C_OK;
 }
@@ -515,8 +565,6 @@ extern "C" s4c_status s4c_tree_accept_tokens(const int32_t* target_token, const 
     if (!target_token || !tokens || !parent || !accept_len || !path || !next_token) return S4C_ERR_NULL;
     if (B < 0 || T < 1 || T > S4C_MAX_T || V < 1 || max_depth < 0 || max_depth >= S4C_MAX_T) return S4C_ERR_SHAPE;
     if (B == 0) return S4C_OK;
-    accept_tokens_kernel<<<B, 128, 0, static_cast<cudaStream_t>(stream_)>>>(target_token, tokens, parent, n_nodes, T, V, max_depth,
-                                                                           accept_len, path, next_token, status);
-    S4C_RETURN_IF_CUDA_ERROR();
-    return S4C_OK;
+    return lm_dependent_launch(accept_tokens_kernel, B, 128, 0, static_cast<cudaStream_t>(stream_), target_token, tokens, parent, n_nodes, T, V,
+                               max_depth, accept_len, path, next_token, status);
 }

@@ -445,7 +445,7 @@ def lm_head_greedy(hidden, weight, token=None, max_logit=None, status=None, work
     dev = hidden.device
     token = torch.empty(R, dtype=torch.int32, device=dev) if token is None else token
     max_logit = torch.empty(R, dtype=torch.float32, device=dev) if max_logit is None else max_logit
-    status = torch.zeros(1, dtype=torch.int32, device=dev) if status is None else status
+    status = torch.empty(1, dtype=torch.int32, device=dev) if status is None else status  # (written by the call)
     if workspace is None:
         workspace = _workspace(int(_lib.s4c_lm_head_greedy_workspace_bytes(R, V, H)), dev, "lm_head")
     rc = _lib.s4c_lm_head_greedy(_dev(hidden, torch.bfloat16, "hidden"), _dev(weight, torch.bfloat16, "weight"), R, V, H,
@@ -557,7 +557,7 @@ def lm_head_topk(hidden, weight, k: int, token=None, logit=None, status=None, wo
     dev = hidden.device
     token = torch.empty(R, k, dtype=torch.int32, device=dev) if token is None else token
     logit = torch.empty(R, k, dtype=torch.float32, device=dev) if logit is None else logit
-    status = torch.zeros(1, dtype=torch.int32, device=dev) if status is None else status
+    status = torch.empty(1, dtype=torch.int32, device=dev) if status is None else status  # (written by the call)
     if workspace is None:
         workspace = _workspace(int(_lib.s4c_lm_head_topk_workspace_bytes(R, V, H, int(k))), dev, "lm_head")
     rc = _lib.s4c_lm_head_topk(_dev(hidden, torch.bfloat16, "hidden"), _dev(weight, torch.bfloat16, "weight"), R, V, H, int(k),
