@@ -2,10 +2,12 @@
 // generic fallback.
 //
 // Used for S4C_F32 inputs (fp32 FMA keeps the 1e-4 accuracy that tf32 tensor-core products would lose)
-// and for bf16 shapes the tensor-core kernel does not take.  Split-KV: grid (splits, Hq, B); each warp
-// owns one query row at a time and sweeps its split's cache slots with an online softmax, lanes spread
-// over the head dimension; the tree's own slots are filtered by the ancestor bitmask built in shared
-// memory from parent[].  Partial (max, sum, unnormalised output) per split go to the workspace and a
+// and for bf16 shapes the tensor-core kernel does not take.  Split-KV: grid (splits, Hq, B); a CTA stages
+// 32 cache slots at a time in shared memory and its 16 warps take the query rows in turn.  Scores: a lane per slot, the
+// whole dot product in one thread; one warp maximum and one sum per 32 slots; then the lanes spread over the head
+// dimension for P V.  (With the lanes over the head dimension throughout, every slot cost a chain of five shuffles and
+// two exponentials: 35 us for 4 heads x 15 rows x 143 slots of 64.)  The tree's own slots are filtered by the ancestor
+// bitmask built in shared memory from parent[].  Partial (max, sum, unnormalised output) per split go to the workspace and a
 // second kernel merges them in split order (deterministic, no float atomics).
 #include <math.h>
 
@@ -14,7 +16,8 @@
 
 namespace s4c {
 
-constexpr int kSimtThreads = 128;
+constexpr int kSimtThreads = 512;
+constexpr int kSimtTile = 32;  // cache slots staged at a time: one per lane
 constexpr int kSimtWarps = kSimtThreads / 32;
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -86,6 +89,7 @@ tree_attention_simt_kernel(const T_* __restrict__ q, const T_* __restrict__ kc, 
     __shared__ uint32_t anc_s[S4C_MAX_T][S4C_MASK_WORDS];
     __shared__ int flag_s;
     int n, L;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the merge waits for this grid on its own)
     const int flags = load_and_check_tree(parent, n_nodes, cache_len, b, T, C, par_s, anc_s, &flag_s, n, L);
     if (split == 0 && h == 0 && threadIdx.x == 0 && status) status[b] = flags;
     if (flags) return;
@@ -95,10 +99,15 @@ tree_attention_simt_kernel(const T_* __restrict__ q, const T_* __restrict__ kc, 
     const int k0 = split * chunk, k1 = min(total, k0 + chunk);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int hk = h / (Hq / Hkv);
-    const T_* kb = kc + ((size_t)b * Hkv + hk) * C * D + lane * DPL;
-    const T_* vb = vc + ((size_t)b * Hkv + hk) * C * D + lane * DPL;
+    const T_* kb = kc + ((size_t)b * Hkv + hk) * C * D;
+    const T_* vb = vc + ((size_t)b * Hkv + hk) * C * D;
+    __shared__ __align__(16) float ks[kSimtTile][D + 4];  // (rows a multiple of 16 bytes apart, a bank group per row: a float4 per lane)
+    __shared__ __align__(16) float vs[kSimtTile][D];
+    __shared__ __align__(16) float qs[kSimtWarps][D];
 
-    for (int i = warp; i < T; i += kSimtWarps) {
+    // rows warp, warp + 16, ... of a pass; trees of more than 16 nodes take several passes over the split's slots
+    for (int i0 = 0; i0 < T; i0 += kSimtWarps) {
+        const int i = i0 + warp;
         float acc[DPL];
 #pragma unroll
         for (int c = 0; c < DPL; ++c) acc[c] = 0.f;
@@ -107,30 +116,59 @@ tree_attention_simt_kernel(const T_* __restrict__ q, const T_* __restrict__ kc, 
             float qv[DPL];
             Elem<T_>::template load<DPL>(q + (((size_t)b * Hq + h) * T + i) * D + lane * DPL, qv);
 #pragma unroll
-            for (int c = 0; c < DPL; ++c) qv[c] *= scale_log2;
-            for (int j = k0; j < k1; ++j) {
-                if (j >= L) {
-                    const int t = j - L;
-                    if (!((anc_s[i][t >> 5] >> (t & 31)) & 1u)) continue;
+            for (int c = 0; c < DPL; ++c) qs[warp][lane * DPL + c] = qv[c] * scale_log2;
+        }
+        for (int j0 = k0; j0 < k1; j0 += kSimtTile) {
+            __syncthreads();
+            for (int e = threadIdx.x; e < kSimtTile * 32; e += kSimtThreads) {
+                const int row = e >> 5, at = (e & 31) * DPL;
+                float kv[DPL], vv[DPL];
+#pragma unroll
+                for (int c = 0; c < DPL; ++c) kv[c] = vv[c] = 0.f;
+                if (j0 + row < k1) {
+                    Elem<T_>::template load<DPL>(kb + (size_t)(j0 + row) * D + at, kv);
+                    Elem<T_>::template load<DPL>(vb + (size_t)(j0 + row) * D + at, vv);
                 }
-                float kv[DPL];
-                Elem<T_>::template load<DPL>(kb + (size_t)j * D, kv);
-                float s = 0.f;
 #pragma unroll
-                for (int c = 0; c < DPL; ++c) s = fmaf(qv[c], kv[c], s);
+                for (int c = 0; c < DPL; ++c) ks[row][at + c] = kv[c], vs[row][at + c] = vv[c];
+            }
+            __syncthreads();
+            if (i < n) {
+                const int j = j0 + lane, t = j - L;
+                const bool seen = j < k1 && (t < 0 || ((anc_s[i][t >> 5] >> (t & 31)) & 1u));
+                float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                const float mn = fmaxf(m, s);
-                const float corr = exp2f(m - mn);  // m = -inf on the first visible slot: corr = 0
-                const float p = exp2f(s - mn);
-                float vv[DPL];
-                Elem<T_>::template load<DPL>(vb + (size_t)j * D, vv);
-                l = l * corr + p;
+                for (int c = 0; c < D; c += 4) {
+                    const float4 kk = *reinterpret_cast<const float4*>(&ks[lane][c]);
+                    const float4 qq = *reinterpret_cast<const float4*>(&qs[warp][c]);
+                    s4[0] = fmaf(qq.x, kk.x, s4[0]), s4[1] = fmaf(qq.y, kk.y, s4[1]);
+                    s4[2] = fmaf(qq.z, kk.z, s4[2]), s4[3] = fmaf(qq.w, kk.w, s4[3]);
+                }
+                const float s = seen ? (s4[0] + s4[1]) + (s4[2] + s4[3]) : -INFINITY;
+                float mn = s;
 #pragma unroll
-                for (int c = 0; c < DPL; ++c) acc[c] = fmaf(acc[c], corr, p * vv[c]);
-                m = mn;
+                for (int o = 16; o > 0; o >>= 1) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+                mn = fmaxf(mn, m);
+                if (mn > -INFINITY) {  // (a tile of other branches' slots only leaves the row as it is)
+                    const float corr = exp2f(m - mn);  // m = -inf on the first visible slot: corr = 0
+                    const float p = exp2f(s - mn);
+                    float sum = p;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    l = l * corr + sum;
+                    m = mn;
+#pragma unroll
+                    for (int c = 0; c < DPL; ++c) acc[c] *= corr;
+#pragma unroll 8
+                    for (int jj = 0; jj < kSimtTile; ++jj) {
+                        const float pj = __shfl_sync(0xffffffffu, p, jj);
+#pragma unroll
+                        for (int c = 0; c < DPL; ++c) acc[c] = fmaf(pj, vs[jj][lane * DPL + c], acc[c]);
+                    }
+                }
             }
         }
+        if (i >= T) continue;
         if (splits == 1) {
             const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
@@ -156,7 +194,10 @@ tree_attention_combine_kernel(const float* __restrict__ ws, const int32_t* __res
     __shared__ uint32_t anc_s[S4C_MAX_T][S4C_MASK_WORDS];
     __shared__ int flag_s;
     int n, L;
-    if (load_and_check_tree(parent, n_nodes, cache_len, b, T, C, par_s, anc_s, &flag_s, n, L)) return;
+    // (launched dependent on the kernel that writes the partials: the tree's check runs beside its tail)
+    const int flags = load_and_check_tree(parent, n_nodes, cache_len, b, T, C, par_s, anc_s, &flag_s, n, L);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (flags) return;
     const float* w = ws + (((size_t)b * Hq + h) * T + i) * splits * (D + 2);
     float M = -INFINITY;
     for (int s = 0; s < splits; ++s) M = fmaxf(M, w[s * (D + 2) + D]);
@@ -175,7 +216,7 @@ tree_attention_combine_kernel(const float* __restrict__ ws, const int32_t* __res
 int simt_splits(int B, int Hq, int C) {
     int s = ceil_div(4 * 148, B * Hq);  // ~4 CTAs of 4 warps per SM
     s = s < 1 ? 1 : s;
-    const int cap = C / 32 > 0 ? C / 32 : 1;  // at least 32 slots per split
+    const int cap = ceil_div(C, kSimtTile);  // a staged tile of slots per split at least
     return s > cap ? cap : (s > 64 ? 64 : s);
 }
 
@@ -188,9 +229,16 @@ template <typename T_, int D>
 static s4c_status launch_combine(const void* ws, const int32_t* cache_len, const int32_t* parent, const int32_t* n_nodes,
                                  void* out, int B, int T, int Hq, int C, int splits, cudaStream_t stream, int out_rows = 0) {
     dim3 g2(T, Hq, B);
-    tree_attention_combine_kernel<T_, D><<<g2, D, 0, stream>>>(static_cast<const float*>(ws), cache_len, parent, n_nodes,
-                                                              static_cast<T_*>(out), T, Hq, C, splits, out_rows);
-    S4C_RETURN_IF_CUDA_ERROR();
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g2, cfg.blockDim = dim3(D, 1, 1), cfg.stream = stream, cfg.attrs = &pdl, cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, tree_attention_combine_kernel<T_, D>, static_cast<const float*>(ws), cache_len, parent, n_nodes,
+                           static_cast<T_*>(out), T, Hq, C, splits, out_rows) != cudaSuccess) {
+        cudaGetLastError();
+        return S4C_ERR_CUDA;
+    }
     return S4C_OK;
 }
 
