@@ -1,14 +1,18 @@
-"""In-tree build of libs4c.so (hand-written CUDA for sm_100a) with nvcc.  No JIT cache, no torch types."""
+"""In-tree build of libs4c.so (hand-written CUDA for sm_100a) with nvcc -- no torch types -- and of _bind.so, the native
+marshalling of the eager calls (bind.cpp: torch tensors to the C ABI), with g++.  No JIT cache."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(os.path.dirname(_HERE), "include")
 _LIB = os.path.join(_HERE, "libs4c.so")
+_BIND_SRC = os.path.join(_CSRC, "bind.cpp")
+_BIND = os.path.join(_HERE, "_bind.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]
@@ -34,6 +38,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("no CUDA sources found under " + _CSRC)
     newest = max(os.path.getmtime(p) for p in deps)
     if not force and os.path.exists(_LIB) and os.path.getmtime(_LIB) >= newest:
+        _build_bind(force)
         return _LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     objs = []
@@ -51,4 +56,24 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = _LIB + f".tmp{os.getpid()}"
     subprocess.run([nvcc, "-shared", "-o", tmp, *objs, "-lcudart"], check=True)
     os.replace(tmp, _LIB)
+    _build_bind(force)
     return _LIB
+
+
+def _build_bind(force: bool = False) -> str:
+    """Compile bind.cpp against torch's headers and libs4c.so (found next to it at run time)."""
+    newest = max(os.path.getmtime(p) for p in [_BIND_SRC] + glob.glob(os.path.join(_INC, "*.h")))
+    if not force and os.path.exists(_BIND) and os.path.getmtime(_BIND) >= newest:
+        return _BIND
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    lib = os.path.join(root, "lib")
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), _INC,
+           sysconfig.get_paths()["include"], os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
+    tmp = _BIND + f".tmp{os.getpid()}"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                    *[f"-I{p}" for p in inc], _BIND_SRC, "-o", tmp, f"-L{_HERE}", "-l:libs4c.so", f"-L{lib}", "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+                    "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{lib}"], check=True)
+    os.replace(tmp, _BIND)
+    return _BIND

@@ -1,4 +1,5 @@
-"""ctypes binding of ``libs4c.so`` -- argument marshalling only; every step runs in the library's CUDA kernels.
+"""Binding of ``libs4c.so`` -- argument marshalling only; every step runs in the library's CUDA kernels.  The calls a program
+makes eagerly per layer or step go through ``_bind.so`` (native marshalling), the others through ctypes.
 
 The functions mirror the C ABI declared in ``include/s4c.h`` (same names, same argument meaning).  Tensors are
 torch CUDA tensors used purely as device buffers: the binding checks dtype / contiguity / device, passes raw
@@ -50,18 +51,10 @@ def _load() -> ctypes.CDLL:
     lib.s4c_status_string.argtypes = [i]
     lib.s4c_tree_attention_workspace_bytes.restype = sz
     lib.s4c_tree_attention_workspace_bytes.argtypes = [i, i, i, i, i, i, i]
-    lib.s4c_tree_attention.restype = i
-    lib.s4c_tree_attention.argtypes = [vp, vp, vp, i32p, i32p, i32p, vp, i, i, i, i, i, i, i, i, f, i32p, vp, sz, vp]
-    lib.s4c_tree_attention_rows.restype = i
-    lib.s4c_tree_attention_rows.argtypes = [vp, vp, vp, i32p, i32p, i32p, vp, i, i, i, i, i, i, i, i, f, i32p, vp, sz, vp]
     lib.s4c_tree_accept_workspace_bytes.restype = sz
     lib.s4c_tree_accept_workspace_bytes.argtypes = [i, i, i]
-    lib.s4c_tree_accept.restype = i
-    lib.s4c_tree_accept.argtypes = [vp, vp, i32p, i32p, i32p, f, vp, i, i, i, i, i32p, i32p, i32p, vp, i32p, vp, sz, vp]
     lib.s4c_tree_accept_noalloc.restype = i
     lib.s4c_tree_accept_noalloc.argtypes = [vp, vp, i32p, i32p, i32p, f, vp, i, i, i, i, i32p, i32p, i32p, vp, i32p, vp]
-    lib.s4c_kv_compact.restype = i
-    lib.s4c_kv_compact.argtypes = [vp, vp, i, i32p, i32p, i32p, i, vp, vp, i, i, i, i, i, i, i, i32p, vp]
     lib.s4c_selftest_attention_timeout.restype = i
     lib.s4c_selftest_attention_timeout.argtypes = [vp, vp, vp, i32p, i32p, vp, i, i, i, i, i, i, i, i, i, i32p, vp]
     lib.s4c_tree_build_workspace_bytes.restype = sz
@@ -78,10 +71,6 @@ def _load() -> ctypes.CDLL:
     lib.s4c_tree_accept_filtered.argtypes = [vp, vp, i32p, i32p, i32p, f, i, f, vp, i, i, i, i, i32p, i32p, i32p, vp, i32p, vp, sz, vp]
     lib.s4c_lm_head_greedy_workspace_bytes.restype = sz
     lib.s4c_lm_head_greedy_workspace_bytes.argtypes = [i, i, i]
-    lib.s4c_lm_head_greedy.restype = i
-    lib.s4c_lm_head_greedy.argtypes = [vp, vp, i, i, i, i32p, vp, i32p, vp, sz, vp]
-    lib.s4c_tree_accept_tokens.restype = i
-    lib.s4c_tree_accept_tokens.argtypes = [i32p, i32p, i32p, i32p, i, i, i, i, i32p, i32p, i32p, i32p, vp]
     lib.s4c_qkv_rope_workspace_bytes.restype = sz
     lib.s4c_qkv_rope_workspace_bytes.argtypes = [i, i, i]
     lib.s4c_qkv_rope.restype = i
@@ -92,8 +81,6 @@ def _load() -> ctypes.CDLL:
     lib.s4c_qkv_rope_same_tree.argtypes = [vp, vp, vp, vp, vp, i, i, i, i, i, i, i, i32p, vp, sz, vp]
     lib.s4c_lm_head_topk_workspace_bytes.restype = sz
     lib.s4c_lm_head_topk_workspace_bytes.argtypes = [i, i, i, i]
-    lib.s4c_lm_head_topk.restype = i
-    lib.s4c_lm_head_topk.argtypes = [vp, vp, i, i, i, i, i32p, vp, i32p, vp, sz, vp]
     lib.s4c_tree_build_topk.restype = i
     lib.s4c_tree_build_topk.argtypes = [i32p, i, vp, i, i32p, i32p, i, i, i32p, i32p, i32p, i32p, vp]
     lib.s4c_lm_head_logits_workspace_bytes.restype = sz
@@ -117,6 +104,10 @@ def _load() -> ctypes.CDLL:
 
 _lib = None
 _lib = _load()
+try:
+    from . import _bind
+except ImportError as e:
+    raise ImportError(f"_bind.so is missing or does not load ({e}): build it with `python -c 'import __graft_entry__ as g; g.build()'`") from e
 
 
 def version() -> int:
@@ -149,13 +140,15 @@ def _stream(stream) -> int:
 
 
 _ws_cache = {}
+_attn_scratch = lambda nbytes, t: _workspace(nbytes, t.device, "attn")
+_head_scratch = lambda nbytes, t: _workspace(nbytes, t.device, "lm_head")
 
 
 def _workspace(nbytes: int, device, tag: str) -> Optional[torch.Tensor]:
     """A cached scratch buffer per (device, call family); reused by calls ordered on one stream."""
     if nbytes == 0:
         return None
-    key = (str(device), tag)
+    key = (device, tag)
     buf = _ws_cache.get(key)
     if buf is None or buf.numel() < nbytes:
         buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
@@ -174,25 +167,8 @@ def tree_attention(q, k_cache, v_cache, cache_len, parent, n_nodes=None, out=Non
 
     ``max_cache_len``: the host's upper bound on ``cache_len`` (0 = unknown); it shapes the launch, never the result.
     ``rows``: s4c_tree_attention_rows -- out is [B,T,Hq,d], the rows the output projection reads (bf16 only)."""
-    B, Hq, T, d = q.shape
-    _, Hkv, C, _ = k_cache.shape
-    if k_cache.shape != (B, Hkv, C, d) or v_cache.shape != (B, Hkv, C, d):
-        raise ValueError("k_cache / v_cache must be [B,Hkv,C,d]")
-    if k_cache.dtype != q.dtype or v_cache.dtype != q.dtype:
-        raise TypeError("q, k_cache and v_cache must share one dtype")
-    if out is None:
-        out = torch.empty(B, T, Hq, d, dtype=q.dtype, device=q.device) if rows else torch.empty_like(q)
-    dt = _dt(q)
-    need = int(_lib.s4c_tree_attention_workspace_bytes(B, T, Hq, Hkv, d, C, dt))
-    if workspace is None:
-        workspace = _workspace(need, q.device, "attn")
-    rc = (_lib.s4c_tree_attention_rows if rows else _lib.s4c_tree_attention)(
-        _dev(q, name="q"), _dev(k_cache, name="k_cache"), _dev(v_cache, name="v_cache"),
-        _dev(cache_len, torch.int32, "cache_len"), _dev(parent, torch.int32, "parent"),
-        _dev(n_nodes, torch.int32, "n_nodes"), _dev(out, q.dtype, "out"), B, T, Hq, Hkv, d, C, int(max_cache_len), dt,
-        float(scale),
-        _dev(status, torch.int32, "status"), _dev(workspace, name="workspace"),
-        0 if workspace is None else workspace.numel() * workspace.element_size(), _stream(stream))
+    rc, out = _bind.attention(q, k_cache, v_cache, cache_len, parent, n_nodes, out, scale, status, workspace, stream, max_cache_len, rows,
+                              _attn_scratch)
     if rc:
         raise S4CError("s4c_tree_attention_rows" if rows else "s4c_tree_attention", rc)
     return out
@@ -216,17 +192,10 @@ def tree_accept(target_logits, draft_probs, tokens, parent, temperature: float, 
     next_token = torch.empty(B, **i32) if next_token is None else next_token
     near_tie = torch.empty(B, T, dtype=torch.uint8, device=dev) if near_tie is None else near_tie
     status = torch.empty(B, **i32) if status is None else status
-    need = int(_lib.s4c_tree_accept_workspace_bytes(B, T, V))
     if workspace is None:
-        workspace = _workspace(need, dev, "accept")
-    rc = _lib.s4c_tree_accept(
-        _dev(target_logits, torch.float32, "target_logits"), _dev(draft_probs, torch.float32, "draft_probs"),
-        _dev(tokens, torch.int32, "tokens"), _dev(parent, torch.int32, "parent"), _dev(n_nodes, torch.int32, "n_nodes"),
-        float(temperature), _dev(uniforms, torch.float32, "uniforms"), B, T, V, int(max_depth),
-        _dev(accept_len, torch.int32, "accept_len"), _dev(path, torch.int32, "path"),
-        _dev(next_token, torch.int32, "next_token"), _dev(near_tie, torch.uint8, "near_tie"),
-        _dev(status, torch.int32, "status"), _dev(workspace, name="workspace"),
-        0 if workspace is None else workspace.numel() * workspace.element_size(), _stream(stream))
+        workspace = _workspace(int(_lib.s4c_tree_accept_workspace_bytes(B, T, V)), dev, "accept")
+    rc = _bind.accept(target_logits, draft_probs, tokens, parent, temperature, uniforms, n_nodes, max_depth, accept_len, path, next_token,
+                      near_tie, status, workspace, stream)
     if rc:
         raise S4CError("s4c_tree_accept", rc)
     return dict(accept_len=accept_len, path=path, next_token=next_token, near_tie=near_tie, status=status)
@@ -279,7 +248,6 @@ def kv_compact(k_ptrs, v_ptrs, n_layers: int, cache_shape, dtype, cache_len, pat
     """s4c_kv_compact.  k_ptrs / v_ptrs: device int64 arrays from :func:`cache_pointer_array`;
     cache_shape = (B,Hkv,C,d); cache_len is updated in place.  Returns status [B]."""
     B, Hkv, C, d = cache_shape
-    max_depth = path.shape[1] - 1
     dt = F32 if dtype == torch.float32 else BF16
     if status is None:
         status = torch.empty(B, dtype=torch.int32, device=cache_len.device)
@@ -287,14 +255,10 @@ def kv_compact(k_ptrs, v_ptrs, n_layers: int, cache_shape, dtype, cache_len, pat
     if feat_in is not None:
         if feat_in.dtype != dtype or feat_out is None or feat_out.dtype != dtype:
             raise TypeError("features must have the cache dtype")
-        if feat_in.shape[:2] != (B, T) or feat_out.shape != (B, max_depth + 1, feat_in.shape[2]):
+        if feat_in.shape[:2] != (B, T) or feat_out.shape != (B, path.shape[1], feat_in.shape[2]):
             raise ValueError("feat_in must be [B,T,hid] and feat_out [B,max_depth+1,hid]")
         hid = feat_in.shape[2]
-    rc = _lib.s4c_kv_compact(
-        _dev(k_ptrs, torch.int64, "k_ptrs") if n_layers else None, _dev(v_ptrs, torch.int64, "v_ptrs") if n_layers else None,
-        int(n_layers), _dev(cache_len, torch.int32, "cache_len"), _dev(path, torch.int32, "path"),
-        _dev(accept_len, torch.int32, "accept_len"), max_depth, _dev(feat_in, name="feat_in"),
-        _dev(feat_out, name="feat_out"), B, T, Hkv, d, C, hid, dt, _dev(status, torch.int32, "status"), _stream(stream))
+    rc = _bind.compact(k_ptrs, v_ptrs, n_layers, B, Hkv, C, d, dt == F32, cache_len, path, accept_len, T, feat_in, feat_out, hid, status, stream)
     if rc:
         raise S4CError("s4c_kv_compact", rc)
     return status
@@ -440,18 +404,7 @@ def lm_head_greedy_workspace_bytes(R, V, H) -> int:
 
 def lm_head_greedy(hidden, weight, token=None, max_logit=None, status=None, workspace=None, stream=None):
     """s4c_lm_head_greedy: token[r] = argmax_v sum_h hidden[r,h] * weight[v,h] (bf16 in, f32 accumulation), no logits in memory."""
-    R, H = hidden.shape
-    V = weight.shape[0]
-    dev = hidden.device
-    token = torch.empty(R, dtype=torch.int32, device=dev) if token is None else token
-    max_logit = torch.empty(R, dtype=torch.float32, device=dev) if max_logit is None else max_logit
-    status = torch.empty(1, dtype=torch.int32, device=dev) if status is None else status  # (written by the call)
-    if workspace is None:
-        workspace = _workspace(int(_lib.s4c_lm_head_greedy_workspace_bytes(R, V, H)), dev, "lm_head")
-    rc = _lib.s4c_lm_head_greedy(_dev(hidden, torch.bfloat16, "hidden"), _dev(weight, torch.bfloat16, "weight"), R, V, H,
-                                 _dev(token, torch.int32, "token"), _dev(max_logit, torch.float32, "max_logit"),
-                                 _dev(status, torch.int32, "status"), _dev(workspace, name="workspace"),
-                                 workspace.numel() * workspace.element_size(), _stream(stream))
+    rc, (token, max_logit, status) = _bind.lm_head(hidden, weight, 0, token, max_logit, status, workspace, stream, _head_scratch)
     if rc:
         raise S4CError("s4c_lm_head_greedy", rc)
     return dict(token=token, max_logit=max_logit, status=status)
@@ -480,20 +433,8 @@ def lm_head_logits(hidden, weight, logits=None, status=None, workspace=None, str
 def tree_accept_tokens(target_token, tokens, parent, V: int, n_nodes=None, max_depth: Optional[int] = None, accept_len=None,
                        path=None, next_token=None, status=None, stream=None):
     """s4c_tree_accept_tokens: greedy verification from the target's choice per node (target_token [B,T] int32)."""
-    B, T = target_token.shape
-    dev = target_token.device
-    if max_depth is None:
-        max_depth = T - 1
-    i32 = dict(dtype=torch.int32, device=dev)
-    accept_len = torch.empty(B, **i32) if accept_len is None else accept_len
-    path = torch.empty(B, max_depth + 1, **i32) if path is None else path
-    next_token = torch.empty(B, **i32) if next_token is None else next_token
-    status = torch.empty(B, **i32) if status is None else status
-    rc = _lib.s4c_tree_accept_tokens(_dev(target_token, torch.int32, "target_token"), _dev(tokens, torch.int32, "tokens"),
-                                     _dev(parent, torch.int32, "parent"), _dev(n_nodes, torch.int32, "n_nodes"), B, T, int(V),
-                                     int(max_depth), _dev(accept_len, torch.int32, "accept_len"), _dev(path, torch.int32, "path"),
-                                     _dev(next_token, torch.int32, "next_token"), _dev(status, torch.int32, "status"),
-                                     _stream(stream))
+    rc, (accept_len, path, next_token, status) = _bind.accept_tokens(target_token, tokens, parent, V, n_nodes, max_depth, accept_len, path,
+                                                                     next_token, status, stream)
     if rc:
         raise S4CError("s4c_tree_accept_tokens", rc)
     return dict(accept_len=accept_len, path=path, next_token=next_token, status=status)
@@ -552,18 +493,9 @@ def lm_head_topk_workspace_bytes(R, V, H, k) -> int:
 
 def lm_head_topk(hidden, weight, k: int, token=None, logit=None, status=None, workspace=None, stream=None):
     """s4c_lm_head_topk: the k best tokens per row of hidden @ weight^T, best first (ties to the lower token)."""
-    R, H = hidden.shape
-    V = weight.shape[0]
-    dev = hidden.device
-    token = torch.empty(R, k, dtype=torch.int32, device=dev) if token is None else token
-    logit = torch.empty(R, k, dtype=torch.float32, device=dev) if logit is None else logit
-    status = torch.empty(1, dtype=torch.int32, device=dev) if status is None else status  # (written by the call)
-    if workspace is None:
-        workspace = _workspace(int(_lib.s4c_lm_head_topk_workspace_bytes(R, V, H, int(k))), dev, "lm_head")
-    rc = _lib.s4c_lm_head_topk(_dev(hidden, torch.bfloat16, "hidden"), _dev(weight, torch.bfloat16, "weight"), R, V, H, int(k),
-                               _dev(token, torch.int32, "token"), _dev(logit, torch.float32, "logit"),
-                               _dev(status, torch.int32, "status"), _dev(workspace, name="workspace"),
-                               0 if workspace is None else workspace.numel() * workspace.element_size(), _stream(stream))
+    if k < 1:
+        raise S4CError("s4c_lm_head_topk", 2)
+    rc, (token, logit, status) = _bind.lm_head(hidden, weight, int(k), token, logit, status, workspace, stream, _head_scratch)
     if rc:
         raise S4CError("s4c_lm_head_topk", rc)
     return dict(token=token, logit=logit, status=status)
