@@ -29,9 +29,9 @@ constexpr int kLnBN = 256;       // most accumulator columns per CTA (the launch
 constexpr int kLnBK = 64;        // K elements per stage (one 128-byte swizzled row)
 constexpr int kLnMaxStages = 12;
 constexpr int kLnRingBytes = 192 * 1024;
-constexpr int kLnThreads = 192;  // producer warp, issuer warp, four epilogue warps
+constexpr int kLnThreads = 224;  // weight producer, issuer, four epilogue warps, input producer
 constexpr int kLnBars = 2 * kLnMaxStages + 2;  // full[], empty[], acc_full, drain
-constexpr int kLnSmemBytes = 1024 + kLnRingBytes + kLnBars * 8 + 16;
+constexpr int kLnSmemBytes = 1024 + kLnRingBytes + kLnBars * 8 + 32;
 
 struct LnParams {
     int R, N, k1_steps, k2_steps;  // K slices of the first and of the second input
@@ -69,9 +69,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
     volatile int* tail = reinterpret_cast<volatile int*>(gen + kLnRingBytes + kLnBars * 8);
     volatile int* tmem_slot = tail;  // written by tcgen05.alloc
     volatile int* dead = tail + 1;   // a wait was given up
-    volatile int* issued_s = tail + 2;
-    auto sX = [&](int s) { return base + s * stage_bytes; };
-    auto sW = [&](int s) { return base + s * stage_bytes + x_bytes; };
+    volatile int* issued_s = tail + 2;  // [2]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ntile = blockIdx.x, mtile = blockIdx.y;
@@ -81,10 +79,10 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
     const int cols = prm.cols;
     const int n0 = ntile * cols;  // first output column of this tile
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 1), mbar_init(EMPTY(s), 1);
+        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 2), mbar_init(EMPTY(s), 1);
         mbar_init(ACC_FULL, 1), mbar_init(DRAIN, 1);
         mbar_fence_init();
-        *dead = 0, *issued_s = 0;
+        *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
         tma_prefetch_desc(&map_x1), tma_prefetch_desc(&map_w);
         if (prm.k2_steps) tma_prefetch_desc(&map_x2);
     }
@@ -96,63 +94,78 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
     const uint32_t tmem = tmem_cta;
     griddep_launch_dependents();  // the kernel behind may set itself up; it waits for this one's results on its own
 
+    // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: what such
+    // a thread computes per slice is time the stream waits, so the two operands have a producer each.
+    // Every CTA walks the K slices from a start of its own (the CTAs of a row tile read the same input tiles).
+    const int k_first = k_begin + (int)((blockIdx.x * 7u + blockIdx.y * 3u) % (uint32_t)k_steps);
     if (warp == 0) {
-        // ================= producer =================
-        if (lane == 0) {
-            // every CTA walks the K slices from a start of its own (the CTAs of a row tile read the same input tiles)
-            const int k0 = (int)((blockIdx.x * 7u + blockIdx.y * 3u) % (uint32_t)k_steps);
-            auto slice_of = [&](int fill) { return k_begin + (fill + k0 < k_steps ? fill + k0 : fill + k0 - k_steps); };
-            auto load_w = [&](int s, int ks) {
-                mbar_expect_tx(FULL(s), stage_bytes);
-                tma_load_2d(sW(s), &map_w, FULL(s), ks * kLnBK, n0);
-                if (prm.gate) tma_load_2d(sW(s) + cols * kLnBK * 2, &map_w, FULL(s), ks * kLnBK, prm.N + n0);  // cols gate rows, then their up rows
-            };
-            auto load_x = [&](int s, int ks) {
-                if (ks < prm.k1_steps)
-                    tma_load_2d(sX(s), &map_x1, FULL(s), ks * kLnBK, mtile * kLnBM * prm.nm);
-                else
-                    tma_load_2d(sX(s), &map_x2, FULL(s), (ks - prm.k1_steps) * kLnBK, mtile * kLnBM * prm.nm);
-            };
-            // the weights do not come from the kernel in front: the first ring of weight tiles is under way before that
-            // kernel has ended; the inputs follow once it has
-            const int pre = k_steps < S ? k_steps : S;
-            for (int f = 0; f < pre; ++f) load_w(f, slice_of(f));
-            griddep_wait();
-            for (int f = 0; f < pre; ++f) load_x(f, slice_of(f));
-            int fill = pre, s = pre == S ? 0 : pre;
-            uint32_t ph = pre == S ? 1 : 0;
-            for (; fill < k_steps; ++fill, s = s + 1 == S ? 0 : s + 1, ph ^= (s == 0)) {
-                if (!mbar_wait(EMPTY(s), ph ^ 1, dead)) break;
-                const int ks = slice_of(fill);
-                load_w(s, ks);
-                load_x(s, ks);
+        // ================= weight producer =================
+        // The weights do not come from the kernel in front: the first ring of weight tiles is under way before it has ended.
+        if (elect_one()) {
+            int s = 0, ks = k_first, fill = 0;
+            uint32_t ph = 0, at = base + x_bytes;
+            const int tx = bn * kLnBK * 2;
+            for (; fill < k_steps; ++fill) {
+                if (fill == S) griddep_wait();  // (a stage is freed only after its input tile has come: the bounded waits start here)
+                if (fill >= S && !mbar_wait(EMPTY(s), ph ^ 1, dead)) break;
+                mbar_expect_tx(FULL(s), tx);
+                tma_load_2d(at, &map_w, FULL(s), ks * kLnBK, n0);
+                if (prm.gate) tma_load_2d(at + cols * kLnBK * 2, &map_w, FULL(s), ks * kLnBK, prm.N + n0);  // cols gate rows, then their up rows
+                at += stage_bytes;
+                if (++s == S) s = 0, ph ^= 1, at = base + x_bytes;
+                if (++ks == k_end) ks = k_begin;
             }
-            *issued_s = fill;
+            issued_s[0] = fill;
+        }
+        __syncwarp();
+    } else if (warp == 6) {
+        // ================= input producer =================
+        if (elect_one()) {
+            griddep_wait();
+            int s = 0, ks = k_first, fill = 0;
+            uint32_t ph = 0, at = base;
+            const int row = mtile * kLnBM * prm.nm, k1 = prm.k1_steps;
+            for (; fill < k_steps; ++fill) {
+                if (fill >= S && !mbar_wait(EMPTY(s), ph ^ 1, dead)) break;
+                mbar_expect_tx(FULL(s), x_bytes);
+                if (ks < k1)
+                    tma_load_2d(at, &map_x1, FULL(s), ks * kLnBK, row);
+                else
+                    tma_load_2d(at, &map_x2, FULL(s), (ks - k1) * kLnBK, row);
+                at += stage_bytes;
+                if (++s == S) s = 0, ph ^= 1, at = base;
+                if (++ks == k_end) ks = k_begin;
+            }
+            issued_s[1] = fill;
         }
         __syncwarp();
     } else if (warp == 1) {
         // ================= issuer: acc = input tile x (this tile's weight rows)^T =================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc_bf16(kLnBM, bn, false);
+            const uint64_t x0 = smem_desc_sw128(base, 16, 1024), w_off = (uint64_t)(x_bytes >> 4), step = (uint64_t)(stage_bytes >> 4);
+            constexpr uint64_t kTile = kLnBM * kLnBK * 2 >> 4;  // from the stage's first 128 rows to its second
+            const bool two = prm.nm == 2;
+            uint64_t x_desc = x0;
             bool ok = true;
             int s = 0;
-            uint32_t ph = 0;
+            uint32_t ph = 0, accumulate = 0;
             griddep_wait();  // the input rows are requested only after the kernel in front has ended: the bounded waits below start then
-            for (int ks = 0; ks < k_steps; ++ks, s = s + 1 == S ? 0 : s + 1, ph ^= (s == 0)) {
+            for (int ks = 0; ks < k_steps; ++ks) {
                 ok = mbar_wait(FULL(s), ph, dead);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t a_desc = smem_desc_sw128(sX(s), 16, 1024), b_desc = smem_desc_sw128(sW(s), 16, 1024);
+                const uint64_t w_desc = x_desc + w_off;
 #pragma unroll
-                for (int kk = 0; kk < kLnBK / 16; ++kk)  // 32 bytes per K step inside the swizzled row (field unit: 16 B)
-                    tc_mma_bf16(tmem, a_desc + 2u * kk, b_desc + 2u * kk, idesc, (ks > 0 || kk > 0) ? 1u : 0u);
-                if (prm.nm == 2) {  // the second 128 rows of the stage (16 KB further on) meet the same weight tile
-                    const uint64_t a2_desc = smem_desc_sw128(sX(s) + kLnBM * kLnBK * 2, 16, 1024);
-#pragma unroll
-                    for (int kk = 0; kk < kLnBK / 16; ++kk)
-                        tc_mma_bf16(tmem + kLnBN, a2_desc + 2u * kk, b_desc + 2u * kk, idesc, (ks > 0 || kk > 0) ? 1u : 0u);
+                for (int kk = 0; kk < kLnBK / 16; ++kk) {  // 32 bytes per K step inside the swizzled row (field unit: 16 B)
+                    tc_mma_bf16(tmem, x_desc + 2u * kk, w_desc + 2u * kk, idesc, accumulate);
+                    // the second 128 rows of the stage meet the same weight tile
+                    if (two) tc_mma_bf16(tmem + kLnBN, x_desc + kTile + 2u * kk, w_desc + 2u * kk, idesc, accumulate);
+                    accumulate = 1;
                 }
                 tc_commit(EMPTY(s));
+                x_desc += step;
+                if (++s == S) s = 0, ph ^= 1, x_desc = x0;
             }
             if (ok) tc_commit(ACC_FULL);
         }
@@ -254,14 +267,15 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
     if (*dead) {
         // a wait was given up: nothing more is issued; what is still in flight lands before shared and tensor memory go
         if (threadIdx.x == 0) {
-            const int issued = *issued_s;
+            const int lo = min(issued_s[0], issued_s[1]), hi = max(issued_s[0], issued_s[1]);
+            for (int f = lo; f < hi; ++f) mbar_arrive(FULL(f % S));  // for the producer that stopped first
             for (int s = 0; s < S; ++s) {
                 int last = -1;
-                for (int f = s; f < issued; f += S) last = f;
+                for (int f = s; f < hi; f += S) last = f;
                 if (last >= 0) mbar_drain(FULL(s), (last / S) & 1);
             }
         }
-        if (warp == 1 && lane == 0) {
+        if (warp == 1 && elect_one()) {
             tc_commit(DRAIN);
             mbar_drain(DRAIN, 0);
         }
@@ -318,8 +332,8 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
                      const __nv_bfloat16* __restrict__ norm_weight, float norm_eps, __nv_bfloat16* __restrict__ norm_out,
                      float* __restrict__ out_f32) {
     __shared__ float red[8];
+    griddep_launch_dependents();  // (the next product sets itself up and requests weights meanwhile)
     griddep_wait();
-    griddep_launch_dependents();
     const int r = blockIdx.x;
     const int w_rows = gate ? 2 * N : N;
     float ss = 0.f;
@@ -377,8 +391,8 @@ rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restr
     __shared__ float red[8];
     const size_t row = blockIdx.x;
     const __nv_bfloat16* xr = x + row * H;
-    griddep_wait();
     griddep_launch_dependents();
+    griddep_wait();
     float ss = 0.f;
     for (int i = threadIdx.x * 8; i < H; i += blockDim.x * 8)  // H is a multiple of 8
         ss = sumsq8(ss, __ldg(reinterpret_cast<const uint4*>(xr + i)));
@@ -395,8 +409,8 @@ __global__ void __launch_bounds__(256)
 embed_gather_kernel(const __nv_bfloat16* __restrict__ table, const int32_t* __restrict__ tokens, int V, int H,
                     __nv_bfloat16* __restrict__ out) {
     const size_t row = blockIdx.x;
-    griddep_wait();
     griddep_launch_dependents();
+    griddep_wait();
     const int t = tokens[row];
     const bool ok = t >= 0 && t < V;
     for (int i = threadIdx.x * 8; i < H; i += blockDim.x * 8) {

@@ -27,9 +27,9 @@ constexpr int kQkBM = 128;       // rows per CTA (tensor-memory lanes)
 constexpr int kQkBK = 64;        // hidden elements per stage (one 128-byte swizzled row)
 constexpr int kQkMaxStages = 12;
 constexpr int kQkRingBytes = 192 * 1024;  // cut into stages at launch: a stage holds the rows that exist and the head's d weight rows
-constexpr int kQkThreads = 192;  // producer warp, issuer warp, four epilogue warps
+constexpr int kQkThreads = 224;  // weight producer, issuer, four epilogue warps, state producer
 constexpr int kQkBars = 2 * kQkMaxStages + 2;  // full[], empty[], acc_full, drain
-constexpr int kQkSmemBytes = 1024 + kQkRingBytes + kQkBars * 8 + 16;
+constexpr int kQkSmemBytes = 1024 + kQkRingBytes + kQkBars * 8 + 32;
 
 struct QkParams {
     int R, T, Hq, Hkv, d, C, k_steps;
@@ -95,18 +95,16 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     volatile int* tail = reinterpret_cast<volatile int*>(gen + kQkRingBytes + kQkBars * 8);
     volatile int* tmem_slot = tail;  // written by tcgen05.alloc
     volatile int* dead = tail + 1;   // a wait was given up
-    volatile int* issued_s = tail + 2;
-    auto sX = [&](int s) { return base + s * stage_bytes; };
-    auto sW = [&](int s) { return base + s * stage_bytes + x_bytes; };
+    volatile int* issued_s = tail + 2;  // [2]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int head = blockIdx.x, mtile = blockIdx.y, d = prm.d;
     const uint32_t tmem_cols = d <= 64 ? 64u : 128u;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 1), mbar_init(EMPTY(s), 1);
+        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 2), mbar_init(EMPTY(s), 1);
         mbar_init(ACC_FULL, 1), mbar_init(DRAIN, 1);
         mbar_fence_init();
-        *dead = 0, *issued_s = 0;
+        *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
         tma_prefetch_desc(&map_x), tma_prefetch_desc(&map_w);
     }
     if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), tmem_cols);
@@ -115,54 +113,60 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     tc_fence_after();
     const uint32_t tmem = (uint32_t)*tmem_slot;
 
-    if (warp == 0) {
-        // ================= producer =================
-        if (lane == 0) {
-            // every CTA walks the K slices from a start of its own: the CTAs of a row tile all read the same state tiles,
-            // and in step they would all ask the same L2 lines at the same moment (the order of a sum's terms is free)
-            const int k0 = (int)((blockIdx.x * 7u + blockIdx.y * 3u) % (uint32_t)prm.k_steps);
-            auto slice_of = [&](int fill) { return fill + k0 < prm.k_steps ? fill + k0 : fill + k0 - prm.k_steps; };
-            int fill = 0, s = 0;
-            uint32_t ph = 0;  // the ring pass's parity (stage and parity are stepped, not divided out: S is not a constant)
-            if (prm.wait_x) {
-                // no table kernel in front: the weights (which no kernel of the step writes) fill the first ring while the
-                // kernel that produces the input rows is still running; the rows follow once it has ended
-                const int pre = prm.k_steps < S ? prm.k_steps : S;
-                for (int f = 0; f < pre; ++f) {
-                    mbar_expect_tx(FULL(f), stage_bytes);
-                    tma_load_2d(sW(f), &map_w, FULL(f), slice_of(f) * kQkBK, head * d);
-                }
-                griddep_wait();
-                for (int f = 0; f < pre; ++f) tma_load_2d(sX(f), &map_x, FULL(f), slice_of(f) * kQkBK, mtile * kQkBM);
-                fill = pre, s = pre == S ? 0 : pre, ph = pre == S ? 1 : 0;
+    griddep_launch_dependents();
+    // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: what such
+    // a thread computes per slice is time the stream waits, so the two operands have a producer each.
+    // Every CTA walks the K slices from a start of its own: the CTAs of a row tile all read the same state tiles, and in step
+    // they would all ask the same L2 lines at the same moment (the order of a sum's terms is free).
+    const int k_steps = prm.k_steps, k_first = (int)((blockIdx.x * 7u + blockIdx.y * 3u) % (uint32_t)k_steps);
+    if (warp == 0 || warp == 6) {
+        // ================= producers: weights (warp 0), states (warp 6) =================
+        // The weights, which no kernel of the step writes, fill the first ring while the kernel in front is still running;
+        // the states follow once it has ended.
+        if (elect_one()) {
+            const bool states = warp == 6;
+            int s = 0, ks = k_first, fill = 0;
+            uint32_t ph = 0;
+            const uint32_t first = base + (states ? 0 : x_bytes);
+            uint32_t at = first;
+            const int tx = states ? x_bytes : stage_bytes - x_bytes, row = states ? mtile * kQkBM : head * d;
+            const CUtensorMap* map = states ? &map_x : &map_w;
+            const bool wait_x = prm.wait_x != 0;  // (else the table kernel is in front, and the states were there before it)
+            if (states && wait_x) griddep_wait();
+            for (; fill < k_steps; ++fill) {
+                if (fill == S && wait_x) griddep_wait();  // (a stage is freed only after its states have come: the bounded waits start here)
+                if (fill >= S && !mbar_wait(EMPTY(s), ph ^ 1, dead)) break;
+                mbar_expect_tx(FULL(s), tx);
+                tma_load_2d(at, map, FULL(s), ks * kQkBK, row);
+                at += stage_bytes;
+                if (++s == S) s = 0, ph ^= 1, at = first;
+                if (++ks == k_steps) ks = 0;
             }
-            for (; fill < prm.k_steps; ++fill, s = s + 1 == S ? 0 : s + 1, ph ^= (s == 0)) {
-                if (!mbar_wait(EMPTY(s), ph ^ 1, dead)) break;
-                const int ks = slice_of(fill);
-                mbar_expect_tx(FULL(s), stage_bytes);
-                tma_load_2d(sX(s), &map_x, FULL(s), ks * kQkBK, mtile * kQkBM);
-                tma_load_2d(sW(s), &map_w, FULL(s), ks * kQkBK, head * d);
-            }
-            *issued_s = fill;
+            issued_s[states ? 1 : 0] = fill;
         }
         __syncwarp();
     } else if (warp == 1) {
         // ================= issuer: acc = state tile x (this head's weight rows)^T =================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc_bf16(kQkBM, d, false);
+            const uint64_t x0 = smem_desc_sw128(base, 16, 1024), w_off = (uint64_t)(x_bytes >> 4), step = (uint64_t)(stage_bytes >> 4);
+            uint64_t x_desc = x0;
             bool ok = true;
             int s = 0;
-            uint32_t ph = 0;
+            uint32_t ph = 0, accumulate = 0;
             if (prm.wait_x) griddep_wait();  // the rows are requested only after the kernel in front has ended: the bounded waits start then
-            for (int ks = 0; ks < prm.k_steps; ++ks, s = s + 1 == S ? 0 : s + 1, ph ^= (s == 0)) {
+            for (int ks = 0; ks < k_steps; ++ks) {
                 ok = mbar_wait(FULL(s), ph, dead);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t a_desc = smem_desc_sw128(sX(s), 16, 1024), b_desc = smem_desc_sw128(sW(s), 16, 1024);
 #pragma unroll
-                for (int kk = 0; kk < kQkBK / 16; ++kk)  // 32 bytes per K step inside the swizzled row (field unit: 16 B)
-                    tc_mma_bf16(tmem, a_desc + 2u * kk, b_desc + 2u * kk, idesc, (ks > 0 || kk > 0) ? 1u : 0u);
+                for (int kk = 0; kk < kQkBK / 16; ++kk) {  // 32 bytes per K step inside the swizzled row (field unit: 16 B)
+                    tc_mma_bf16(tmem, x_desc + 2u * kk, x_desc + w_off + 2u * kk, idesc, accumulate);
+                    accumulate = 1;
+                }
                 tc_commit(EMPTY(s));
+                x_desc += step;
+                if (++s == S) s = 0, ph ^= 1, x_desc = x0;
             }
             if (ok) tc_commit(ACC_FULL);
         }
@@ -171,11 +175,11 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         // ================= epilogue: rotate, round, store =================
         const int q = warp & 3;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
         const int r = mtile * kQkBM + q * 32 + lane;
+        griddep_wait();  // the rows' bases and the rotary table are complete; the bounded wait starts here
         bool ok = mbar_wait(ACC_FULL, 0, dead);
         ok = __all_sync(0xffffffffu, ok);
         if (ok) {
             tc_fence_after();
-            griddep_wait();  // the rows' bases and the rotary table are complete
             const int Lb = r < prm.R ? prm.row_base[r] : -1;
             const int b = r / prm.T, t = r - b * prm.T, half = d >> 1;
             __nv_bfloat16* dst = nullptr;
@@ -225,14 +229,15 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     if (*dead) {
         // a wait was given up: nothing more is issued; what is still in flight lands before shared and tensor memory go
         if (threadIdx.x == 0) {
-            const int issued = *issued_s;
+            const int lo = min(issued_s[0], issued_s[1]), hi = max(issued_s[0], issued_s[1]);
+            for (int f = lo; f < hi; ++f) mbar_arrive(FULL(f % S));  // for the producer that stopped first
             for (int s = 0; s < S; ++s) {
                 int last = -1;
-                for (int f = s; f < issued; f += S) last = f;
+                for (int f = s; f < hi; f += S) last = f;
                 if (last >= 0) mbar_drain(FULL(s), (last / S) & 1);
             }
         }
-        if (warp == 1 && lane == 0) {
+        if (warp == 1 && elect_one()) {
             tc_commit(DRAIN);
             mbar_drain(DRAIN, 0);
         }
