@@ -300,14 +300,15 @@ __device__ __forceinline__ float sumsq8(float ss, const uint4& v) {
     }
     return ss;
 }
-__device__ __forceinline__ float cta_sum_256(float ss, float* red) {  // 256 threads; red: 8 floats of shared memory
+constexpr int kRowThreads = 512;  // a CTA per row: one pass over 4096 columns, eight per thread
+__device__ __forceinline__ float cta_row_sum(float ss, float* red) {  // kRowThreads threads; red: a float per warp of shared memory
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
     __syncthreads();
     float tot = 0.f;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) tot += red[w];
+    for (int w = 0; w < kRowThreads / 32; ++w) tot += red[w];
     return tot;
 }
 __device__ __forceinline__ uint4 scale8(const uint4& v, const uint4& g, float scale) {
@@ -326,30 +327,52 @@ __device__ __forceinline__ uint4 scale8(const uint4& v, const uint4& g, float sc
 // After a product whose K slices were shared out: per output element the shares in split order, then bias, gate,
 // residual, one rounding to bf16.  grid (rows), eight columns per thread at a time.  With norm_weight the CTA, which
 // holds the whole row, also writes its root-mean-square normalisation (of the rounded row, as a separate call would).
-__global__ void __launch_bounds__(256)
+// Nothing here is work, everything is latency between two products: the shares' loads go out together, four at a time (one
+// after the other, with 256 threads and two passes, a 4096-wide row of four shares took 6 us).
+__global__ void __launch_bounds__(kRowThreads)
 linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N, int gate, const __nv_bfloat16* __restrict__ bias,
                      const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ out,
                      const __nv_bfloat16* __restrict__ norm_weight, float norm_eps, __nv_bfloat16* __restrict__ norm_out,
                      float* __restrict__ out_f32) {
-    __shared__ float red[8];
+    __shared__ float red[kRowThreads / 32];
     griddep_launch_dependents();  // (the next product sets itself up and requests weights meanwhile)
+    const int r = blockIdx.x, first = threadIdx.x * 8;
+    uint4 g = make_uint4(0, 0, 0, 0);  // the norm weight, which no kernel in front writes, under way before the wait
+    if (norm_weight && first < N) g = __ldg(reinterpret_cast<const uint4*>(norm_weight + first));
     griddep_wait();
-    const int r = blockIdx.x;
     const int w_rows = gate ? 2 * N : N;
+    const size_t share = (size_t)R * w_rows;
     float ss = 0.f;
-    for (int col = threadIdx.x * 8; col < N; col += blockDim.x * 8) {
+    uint4 packed = make_uint4(0, 0, 0, 0);
+    for (int col = first; col < N; col += kRowThreads * 8) {
         float y[8], up[8];
+        uint4 rv = make_uint4(0, 0, 0, 0);
+        if (residual) rv = *reinterpret_cast<const uint4*>(residual + (size_t)r * N + col);
 #pragma unroll
         for (int j = 0; j < 8; ++j) y[j] = 0.f, up[j] = 0.f;
-        for (int z = 0; z < splits; ++z) {
-            const float* p = partial + ((size_t)z * R + r) * w_rows;
-            const float4 a0 = *reinterpret_cast<const float4*>(p + col), a1 = *reinterpret_cast<const float4*>(p + col + 4);
-            y[0] += a0.x, y[1] += a0.y, y[2] += a0.z, y[3] += a0.w, y[4] += a1.x, y[5] += a1.y, y[6] += a1.z, y[7] += a1.w;
-            if (gate) {
-                const float4 u0 = *reinterpret_cast<const float4*>(p + N + col), u1 = *reinterpret_cast<const float4*>(p + N + col + 4);
-                up[0] += u0.x, up[1] += u0.y, up[2] += u0.z, up[3] += u0.w, up[4] += u1.x, up[5] += u1.y, up[6] += u1.z, up[7] += u1.w;
+        const float* p = partial + (size_t)r * w_rows + col;
+        for (int z0 = 0; z0 < splits; z0 += 4) {
+            float4 a[4][2], u[4][2];
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+                a[z][0] = a[z][1] = u[z][0] = u[z][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (z0 + z < splits) {
+                    const float4* q = reinterpret_cast<const float4*>(p + (z0 + z) * share);
+                    a[z][0] = q[0], a[z][1] = q[1];
+                    if (gate) q = reinterpret_cast<const float4*>(p + (z0 + z) * share + N), u[z][0] = q[0], u[z][1] = q[1];
+                }
+            }
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {  // (a share that does not exist adds zero)
+                y[0] += a[z][0].x, y[1] += a[z][0].y, y[2] += a[z][0].z, y[3] += a[z][0].w;
+                y[4] += a[z][1].x, y[5] += a[z][1].y, y[6] += a[z][1].z, y[7] += a[z][1].w;
+                if (gate) {
+                    up[0] += u[z][0].x, up[1] += u[z][0].y, up[2] += u[z][0].z, up[3] += u[z][0].w;
+                    up[4] += u[z][1].x, up[5] += u[z][1].y, up[6] += u[z][1].z, up[7] += u[z][1].w;
+                }
             }
         }
+        const __nv_bfloat16* rp = reinterpret_cast<const __nv_bfloat16*>(&rv);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             if (bias) y[j] += __bfloat162float(bias[col + j]);
@@ -357,7 +380,7 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
                 if (bias) up[j] += __bfloat162float(bias[N + col + j]);
                 y[j] = silu(y[j]) * up[j];
             }
-            if (residual) y[j] += __bfloat162float(residual[(size_t)r * N + col + j]);
+            if (residual) y[j] += __bfloat162float(rp[j]);
         }
         if (out_f32) {  // the sums as they are (logits); no normalisation in this form
             float4* dst = reinterpret_cast<float4*>(out_f32 + (size_t)r * N + col);
@@ -370,25 +393,28 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
             const __nv_bfloat162 p2 = __floats2bfloat162_rn(y[2 * j], y[2 * j + 1]);
             pk[j] = *reinterpret_cast<const uint32_t*>(&p2);
         }
-        const uint4 packed = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        packed = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(out + (size_t)r * N + col) = packed;
         ss = sumsq8(ss, packed);
     }
     if (norm_weight) {  // (uniform over the CTA)
-        const float scale = rsqrtf(cta_sum_256(ss, red) / (float)N + norm_eps);
-        for (int col = threadIdx.x * 8; col < N; col += blockDim.x * 8) {
-            const uint4 v = *reinterpret_cast<const uint4*>(out + (size_t)r * N + col);  // this thread's own stores
-            const uint4 g = __ldg(reinterpret_cast<const uint4*>(norm_weight + col));
-            *reinterpret_cast<uint4*>(norm_out + (size_t)r * N + col) = scale8(v, g, scale);
+        const float scale = rsqrtf(cta_row_sum(ss, red) / (float)N + norm_eps);
+        const bool whole = N <= kRowThreads * 8;  // the row is in the threads' registers
+        for (int col = first; col < N; col += kRowThreads * 8) {
+            if (!whole) {
+                packed = *reinterpret_cast<const uint4*>(out + (size_t)r * N + col);  // this thread's own stores
+                g = __ldg(reinterpret_cast<const uint4*>(norm_weight + col));
+            }
+            *reinterpret_cast<uint4*>(norm_out + (size_t)r * N + col) = scale8(packed, g, scale);
         }
     }
 }
 
 // root-mean-square normalisation: one CTA per row, float32 arithmetic, one rounding to bf16
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kRowThreads)
 rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ weight, float eps, int H,
                __nv_bfloat16* __restrict__ out) {
-    __shared__ float red[8];
+    __shared__ float red[kRowThreads / 32];
     const size_t row = blockIdx.x;
     const __nv_bfloat16* xr = x + row * H;
     griddep_launch_dependents();
@@ -396,7 +422,7 @@ rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restr
     float ss = 0.f;
     for (int i = threadIdx.x * 8; i < H; i += blockDim.x * 8)  // H is a multiple of 8
         ss = sumsq8(ss, __ldg(reinterpret_cast<const uint4*>(xr + i)));
-    const float scale = rsqrtf(cta_sum_256(ss, red) / (float)H + eps);
+    const float scale = rsqrtf(cta_row_sum(ss, red) / (float)H + eps);
     for (int i = threadIdx.x * 8; i < H; i += blockDim.x * 8) {
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(xr + i));
         const uint4 g = __ldg(reinterpret_cast<const uint4*>(weight + i));
@@ -482,9 +508,11 @@ struct LnPlan {
     int bn, splits, x_rows, stages, cols_per_tile, m_tiles, n_tiles, nm;
 };
 static LnPlan ln_plan(int R, int K1, int K2, int N, int gate) {
-    constexpr double kIssueUs = 0.30, kMmaUsPerCol = 0.27 / 256.0, kSmBytesPerUs = 55e3, kHbmBytesPerUs = 6.4e6, kL2BytesPerUs = 100e3,
+    constexpr double kIssueUs = 0.30, kMmaUsPerCol = 0.27 / 256.0, kHbmBytesPerUs = 6.4e6, kL2BytesPerUs = 100e3,
                      kTurnUs = 1.3, kWaveUs = 2.5, kFinishUs = 3.0, kPartialBytesPerUs = 4.0e6, kIssueTwo = 1.5;
     constexpr int kSms = 148;
+    // (what one SM pulls of the weight stream: with two row tiles per CTA the ring is deeper in time, and waves of few CTAs pay)
+    const double kSmBytesPerUs = R > kLnBM ? 80e3 : 55e3;
     const int k_steps = (K1 + K2) / kLnBK;
     const int w_rows = gate ? 2 * N : N;
     LnPlan best = {};
@@ -584,10 +612,10 @@ static s4c_status ln_run(const void* x1, const void* x2, const void* w, const vo
     bool ok = ln_launch(linear_kernel, dim3(pl.n_tiles, pl.m_tiles, pl.splits), kLnThreads, kLnSmemBytes, stream, map_x1, map_x2, map_w,
                         prm) == cudaSuccess;
     if (ok && pl.splits > 1)  // the finishing kernel holds whole rows: it normalises them as well
-        ok = ln_launch(linear_finish_kernel, dim3(R, 1, 1), 256, 0, stream, (const float*)prm.partial, pl.splits, R, N, gate ? 1 : 0,
+        ok = ln_launch(linear_finish_kernel, dim3(R, 1, 1), kRowThreads, 0, stream, (const float*)prm.partial, pl.splits, R, N, gate ? 1 : 0,
                        prm.bias, prm.residual, prm.out, nw, norm_eps, no, prm.out_f32) == cudaSuccess;
     else if (ok && nw)
-        ok = ln_launch(rmsnorm_kernel, dim3(R, 1, 1), 256, 0, stream, (const __nv_bfloat16*)prm.out, nw, norm_eps, N, no) == cudaSuccess;
+        ok = ln_launch(rmsnorm_kernel, dim3(R, 1, 1), kRowThreads, 0, stream, (const __nv_bfloat16*)prm.out, nw, norm_eps, N, no) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         return S4C_ERR_CUDA;
@@ -625,7 +653,7 @@ extern "C" s4c_status s4c_rmsnorm(const void* x, const void* weight, float eps, 
     if (R < 0 || H < 8 || H % 8 != 0 || !(eps >= 0.f)) return S4C_ERR_SHAPE;
     if (!aligned16(x) || !aligned16(weight) || !aligned16(out)) return S4C_ERR_ALIGN;
     if (R == 0) return S4C_OK;
-    if (ln_launch(rmsnorm_kernel, dim3(R, 1, 1), 256, 0, static_cast<cudaStream_t>(stream_), static_cast<const __nv_bfloat16*>(x),
+    if (ln_launch(rmsnorm_kernel, dim3(R, 1, 1), kRowThreads, 0, static_cast<cudaStream_t>(stream_), static_cast<const __nv_bfloat16*>(x),
                   static_cast<const __nv_bfloat16*>(weight), eps, H, static_cast<__nv_bfloat16*>(out)) != cudaSuccess) {
         cudaGetLastError();
         return S4C_ERR_CUDA;
