@@ -18,12 +18,18 @@ struct PathInfo {
     int L;
 };
 
-// Same checks in both kernels, evaluated redundantly by every thread that needs them (<= 128 ints).
-__device__ __forceinline__ PathInfo check_path(const int32_t* cache_len, const int32_t* path,
-                                               const int32_t* accept_len, int b, int max_depth, int T, int C) {
+// Same checks in both kernels, by one whole warp: a lane per path entry, so that the entries are one round of loads (one thread
+// going through them took a load latency each).  The path's entries are left in `spath` (shared memory) if it is given.
+__device__ __forceinline__ PathInfo check_path(const int32_t* cache_len, const int32_t* path, const int32_t* accept_len, int b,
+                                               int max_depth, int T, int C, int32_t* spath) {
+    const int lane = threadIdx.x & 31;
     PathInfo r;
     r.a = accept_len[b];
     r.L = cache_len[b];
+    const int32_t* p = path + (size_t)b * (max_depth + 1);
+    int v[(S4C_MAX_T + 31) / 32];
+#pragma unroll
+    for (int i = 0; i < (S4C_MAX_T + 31) / 32; ++i) v[i] = i * 32 + lane <= max_depth ? p[i * 32 + lane] : 0;
     r.flags = 0;
     if (r.a < 0) {
         r.flags = -1;
@@ -32,16 +38,23 @@ __device__ __forceinline__ PathInfo check_path(const int32_t* cache_len, const i
     if (r.a > max_depth) r.flags |= S4C_SEQ_DEPTH;
     if (r.L < 0 || (long long)r.L + T > (long long)C) r.flags |= S4C_SEQ_CAPACITY;
     if (r.flags) return r;
-    const int32_t* p = path + (size_t)b * (max_depth + 1);
-    if (p[0] != 0) r.flags |= S4C_SEQ_BAD_PATH;
-    int prev = -1;
-    for (int j = 0; j <= r.a; ++j) {
-        const int v = p[j];
-        if (v < j || v >= T || v <= prev) r.flags |= S4C_SEQ_BAD_PATH;
-        prev = v;
+    bool bad = false;
+    int before = -1;  // the last entry of the 32 in front
+#pragma unroll
+    for (int i = 0; i < (S4C_MAX_T + 31) / 32; ++i) {
+        const int j = i * 32 + lane, up = __shfl_up_sync(0xffffffffu, v[i], 1), prev = lane ? up : before;
+        if (j <= r.a) {
+            bad |= v[i] < j || v[i] >= T || v[i] <= prev || (j == 0 && v[i] != 0);
+            if (spath) spath[j] = v[i];
+        }
+        before = __shfl_sync(0xffffffffu, v[i], 31);
     }
+    if (__any_sync(0xffffffffu, bad)) r.flags |= S4C_SEQ_BAD_PATH;
     return r;
 }
+
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 constexpr int kCompactThreads = 256;
 constexpr int kBatch = 4;
@@ -66,25 +79,39 @@ __device__ __forceinline__ int load_tree_pages(const Paging& pg, int b, int L, i
     return flags;
 }
 
-// grid: (item blocks, n_layers, B).  Items of one (layer, b): Hkv heads x {K,V} x words per row.
+// grid: (item blocks, n_layers + 1, B).  Items of one (layer, b): Hkv heads x {K,V} x words per row; the last layer index is
+// the feature gather, which runs beside the cache rows.
 __global__ void __launch_bounds__(kCompactThreads)
 kv_compact_rows_kernel(void* const* __restrict__ k_caches, void* const* __restrict__ v_caches,
                        const int32_t* __restrict__ cache_len, const int32_t* __restrict__ path,
                        const int32_t* __restrict__ accept_len, int max_depth, int T, int Hkv, int C,
-                       int words_per_row, const Paging pg) {
+                       int words_per_row, const Paging pg, int n_layers, const uint4* __restrict__ feat_in,
+                       uint4* __restrict__ feat_out, int feat_words) {
     const int b = blockIdx.z, layer = blockIdx.y;
     __shared__ PathInfo info;
     __shared__ int32_t spath[S4C_MAX_T];
     __shared__ int pages[kMaxTreeBlocks];
-    if (threadIdx.x == 0) {
-        info = check_path(cache_len, path, accept_len, b, max_depth, T, C);
-        if (pg.table && info.flags == 0) info.flags |= load_tree_pages(pg, b, info.L, T, pages);
+    griddep_launch_dependents();
+    griddep_wait();
+    if (threadIdx.x < 32) {
+        PathInfo r = check_path(cache_len, path, accept_len, b, max_depth, T, C, spath);
+        if (threadIdx.x == 0) {
+            if (pg.table && r.flags == 0) r.flags |= load_tree_pages(pg, b, r.L, T, pages);
+            info = r;
+        }
     }
     __syncthreads();
-    if (info.flags != 0 || info.a == 0) return;  // nothing to move (path[0] == 0 stays in place)
+    if (info.flags != 0) return;
     const int a = info.a;
-    for (int j = threadIdx.x; j <= a; j += blockDim.x) spath[j] = path[(size_t)b * (max_depth + 1) + j];
-    __syncthreads();
+    if (layer == n_layers) {
+        const int total = (a + 1) * feat_words;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+            const int j = i / feat_words, w = i - j * feat_words;
+            feat_out[((size_t)b * (max_depth + 1) + j) * feat_words + w] = feat_in[((size_t)b * T + spath[j]) * feat_words + w];
+        }
+        return;
+    }
+    if (a == 0) return;  // nothing to move (path[0] == 0 stays in place)
 
     const int items = Hkv * 2 * words_per_row;
     const int item = blockIdx.x * blockDim.x + threadIdx.x;
@@ -112,34 +139,19 @@ kv_compact_rows_kernel(void* const* __restrict__ k_caches, void* const* __restri
     }
 }
 
-// grid: (B).  Gathers the features, writes the per-sequence status and the new cache length.
-__global__ void __launch_bounds__(kCompactThreads)
+// grid: (B), one warp.  Writes the per-sequence status and the new cache length, once nobody reads the old one any more.
+__global__ void __launch_bounds__(32)
 kv_compact_finish_kernel(int32_t* __restrict__ cache_len, const int32_t* __restrict__ path,
-                         const int32_t* __restrict__ accept_len, int max_depth, int T, int C,
-                         const uint4* __restrict__ feat_in, uint4* __restrict__ feat_out, int feat_words,
-                         int32_t* __restrict__ status, const Paging pg) {
+                         const int32_t* __restrict__ accept_len, int max_depth, int T, int C, int32_t* __restrict__ status,
+                         const Paging pg) {
     const int b = blockIdx.x;
-    __shared__ PathInfo info;
-    if (threadIdx.x == 0) {
-        info = check_path(cache_len, path, accept_len, b, max_depth, T, C);
-        int pages[kMaxTreeBlocks];
-        if (pg.table && info.flags == 0) info.flags |= load_tree_pages(pg, b, info.L, T, pages);
-    }
-    __syncthreads();
-    const PathInfo r = info;
-    if (threadIdx.x == 0 && status) status[b] = r.flags < 0 ? 0 : r.flags;
-    if (r.flags != 0) return;
-    if (feat_in && feat_out) {
-        const int32_t* p = path + (size_t)b * (max_depth + 1);
-        const int total = (r.a + 1) * feat_words;
-        for (int i = threadIdx.x; i < total; i += blockDim.x) {
-            const int j = i / feat_words, w = i - j * feat_words;
-            feat_out[((size_t)b * (max_depth + 1) + j) * feat_words + w] =
-                feat_in[((size_t)b * T + p[j]) * feat_words + w];
-        }
-    }
-    __syncthreads();  // every thread has read cache_len (through `info`) before it changes
-    if (threadIdx.x == 0) cache_len[b] = r.L + r.a + 1;
+    griddep_wait();
+    PathInfo r = check_path(cache_len, path, accept_len, b, max_depth, T, C, nullptr);
+    if (threadIdx.x != 0) return;
+    int pages[kMaxTreeBlocks];
+    if (pg.table && r.flags == 0) r.flags |= load_tree_pages(pg, b, r.L, T, pages);
+    if (status) status[b] = r.flags < 0 ? 0 : r.flags;
+    if (r.flags == 0) cache_len[b] = r.L + r.a + 1;
 }
 
 }  // namespace s4c
@@ -163,17 +175,28 @@ static s4c_status kv_compact_launch(void* const* k_caches, void* const* v_caches
     if (!aligned16(feat_in) || !aligned16(feat_out)) return S4C_ERR_ALIGN;
     if (B == 0) return S4C_OK;
     const int words_per_row = (int)(d * es / 16);
-    if (n_layers > 0) {
+    // Both kernels are launched dependent on the one in front: what they cost is latency, not bytes.
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = stream, cfg.attrs = &pdl, cfg.numAttrs = 1;
+    cudaError_t err = cudaSuccess;
+    if (n_layers > 0 || feat_in) {
         const int items = Hkv * 2 * words_per_row;
-        dim3 grid(ceil_div(items, kCompactThreads), n_layers, B);
-        kv_compact_rows_kernel<<<grid, kCompactThreads, 0, stream>>>(k_caches, v_caches, cache_len, path, accept_len,
-                                                                      max_depth, T, Hkv, C, words_per_row, pg);
-        S4C_RETURN_IF_CUDA_ERROR();
+        cfg.gridDim = dim3(ceil_div(items, kCompactThreads), n_layers + (feat_in ? 1 : 0), B), cfg.blockDim = dim3(kCompactThreads, 1, 1);
+        err = cudaLaunchKernelEx(&cfg, kv_compact_rows_kernel, k_caches, v_caches, (const int32_t*)cache_len, path, accept_len, max_depth, T,
+                                 Hkv, C, words_per_row, pg, n_layers, static_cast<const uint4*>(feat_in), static_cast<uint4*>(feat_out),
+                                 feat_in ? (int)(hid * es / 16) : 0);
     }
-    kv_compact_finish_kernel<<<B, kCompactThreads, 0, stream>>>(
-        cache_len, path, accept_len, max_depth, T, C, static_cast<const uint4*>(feat_in),
-        static_cast<uint4*>(feat_out), feat_in ? (int)(hid * es / 16) : 0, status, pg);
-    S4C_RETURN_IF_CUDA_ERROR();
+    if (err == cudaSuccess) {
+        cfg.gridDim = dim3(B, 1, 1), cfg.blockDim = dim3(32, 1, 1);
+        err = cudaLaunchKernelEx(&cfg, kv_compact_finish_kernel, cache_len, path, accept_len, max_depth, T, C, status, pg);
+    }
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        return S4C_ERR_CUDA;
+    }
     return S4C_OK;
 }
 

@@ -194,6 +194,7 @@ template <bool STOCH, bool VEC>
 __global__ void __launch_bounds__(kRowThreads)
 accept_rowstats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ n_nodes, int T, int V,
                        double inv_tau, float floor_span, RowPartial* __restrict__ out) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk's set-up runs beside this)
     const int split = blockIdx.x, node = blockIdx.y, b = blockIdx.z;
     if (n_nodes && node >= n_nodes[b]) return;
     const float* row = logits + ((size_t)b * T + node) * V;
@@ -363,6 +364,7 @@ accept_stats_cluster_kernel(const float* __restrict__ logits, const float* __res
                             const int32_t* __restrict__ tokens, const int32_t* __restrict__ parent,
                             const int32_t* __restrict__ n_nodes, int T, int V, int chunk, double inv_tau,
                             float floor_span, NodeSummary* __restrict__ out) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk's set-up runs beside this)
     const int node = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
     const int n = n_nodes ? n_nodes[b] : T;
     if (node >= n || n > T) return;  // the whole cluster leaves together: nobody is left waiting at a barrier
@@ -527,6 +529,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WalkClShared& cs = *reinterpret_cast<WalkClShared*>(smem_raw);
     WalkShared& sh = cs.w;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.y, tid = threadIdx.x;
     const uint32_t rank = STOCH ? cl_rank() : 0u;
     const bool writer = rank == 0;  // CTA 0 writes everything except the final token, which its finder writes
@@ -550,6 +553,15 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         __syncthreads();
         flags = sh.flag;
     }
+    if (STOCH && !flags)  // what the walk will need of the big rows, fetched by all threads at once instead of one test at a time
+        for (int i = 1 + tid; i < n; i += blockDim.x) {
+            const size_t at = ((size_t)b * T + sh.par[i]) * V + sh.tok[i];
+            cs.tq0[i] = (double)__ldg(dprobs + at);
+            cs.tp0[i] = (double)__ldg(logits + at);  // turned into a probability below, once the parent's statistics are in
+        }
+    // Everything above reads the caller's inputs only, which were complete before the statistics kernel began; from here on
+    // its results are needed.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!(flags & S4C_SEQ_BAD_PARENT)) {
         // ---- per-node statistics into shared memory (n is in 1..T here), and the check that every row is usable
         if (seg_row && STOCH) {
@@ -600,13 +612,6 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         }
         return;
     }
-    if (STOCH)  // what the walk will need of the big rows, fetched by all threads at once instead of one test at a time
-        for (int i = 1 + tid; i < n; i += blockDim.x) {
-            const int pr = sh.par[i], x = sh.tok[i];
-            const size_t at = ((size_t)b * T + pr) * V + x;
-            cs.tq0[i] = (double)__ldg(dprobs + at);
-            cs.tp0[i] = (double)__ldg(logits + at);  // turned into a probability below, once the parent's statistics are in
-        }
     __syncthreads();
     if (STOCH)
         for (int i = 1 + tid; i < n; i += blockDim.x) {
@@ -890,7 +895,7 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
     const bool seg_stats = !(vec && V <= kClMaxV) || (size_t)B * T * V > kSegStatsMinElems;
     const int chunk = (int)round_up((size_t)ceil_div(V, kCl), 4);
     const float floor_span = kExpFloorSpan * (stoch ? temperature : 1.f);
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kCl, attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
@@ -932,7 +937,11 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
             return S4C_ERR_CUDA;
         }
     }
-    // ---- the walk: one cluster per sequence (greedy: one CTA, no vocabulary pass)
+    // ---- the walk: one cluster per sequence (greedy: one CTA, no vocabulary pass), launched dependent on the statistics
+    cudaLaunchAttribute& pdl = attr[stoch ? 1 : 0];
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = stoch ? 2 : 1;
     const NodeSummary* summary = seg_stats ? nullptr : ws.summary;
     const RowPartial* seg_row = seg_stats ? ws.row : nullptr;
     if (stoch) {
@@ -963,10 +972,13 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
             return S4C_ERR_CUDA;
         }
     } else {
-        accept_walk_cluster_kernel<false><<<dim3(1, B), 128, sizeof(WalkClShared), stream>>>(
-            target_logits, draft_probs, tokens, parent, n_nodes, uniforms, T, V, chunk, 0, max_depth, inv_tau, summary,
-            splits, seg_row, accept_len, path, next_token, near_tie, status);
-        S4C_RETURN_IF_CUDA_ERROR();
+        cfg.gridDim = dim3(1, B, 1), cfg.blockDim = dim3(128, 1, 1), cfg.dynamicSmemBytes = sizeof(WalkClShared);
+        if (cudaLaunchKernelEx(&cfg, accept_walk_cluster_kernel<false>, target_logits, draft_probs, tokens, parent, n_nodes, uniforms, T, V,
+                               chunk, 0, max_depth, inv_tau, summary, splits, seg_row, accept_len, path, next_token, near_tie,
+                               status) != cudaSuccess) {
+            cudaGetLastError();
+            return S4C_ERR_CUDA;
+        }
     }
     return S4C_OK;
 }
