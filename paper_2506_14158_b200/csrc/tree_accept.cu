@@ -318,6 +318,7 @@ __device__ __forceinline__ void chain_eval(double p0, double q0, int v, int r, c
 constexpr int kCl = 8;             // CTAs per cluster
 constexpr int kClEpt = 16;         // row elements per thread
 constexpr int kClMaxThreads = 1024;
+constexpr int kWalkGroup = 128;    // vocabulary entries that a warp of the walk takes at once: four per lane
 constexpr int kClMaxV = kCl * kClMaxThreads * kClEpt;
 constexpr size_t kSegStatsMinElems = (size_t)8 << 20;  // B*T*V above which the segment kernels win (measured)
 
@@ -506,13 +507,17 @@ accept_stats_cluster_kernel(const float* __restrict__ logits, const float* __res
     cl_sync();  // nobody leaves while a peer may still read its slots
 }
 
+__device__ __forceinline__ double accept_ratio(double p, double q) { return q > 0.0 ? p / q : (p > 0.0 ? (double)INFINITY : 0.0); }
+
 // ---- the walk, one cluster per sequence (greedy: one CTA, no cluster, no vocabulary pass)
 struct WalkClShared {
     WalkShared w;
     double tab[32];
     double slots[2][2];  // two alternating sets of (sum a, sum b): set k is rewritten two cluster barriers later
-    double ga[kCl], gb[kCl];
+    double gab[2][kCl];
     double tp0[S4C_MAX_T], tq0[S4C_MAX_T];  // node i's token under its parent's row: target and draft probability
+    double ratio0[S4C_MAX_T];               // ... and what its test compares with while no sibling has been rejected
+    uint32_t kids[S4C_MAX_T][S4C_MASK_WORDS];  // node i's children
     double pa[33], pb[33];                  // scratch of the paired block reduction
 };
 
@@ -521,7 +526,7 @@ __global__ void __launch_bounds__(STOCH ? 1024 : 128, 1)
 accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __restrict__ dprobs,
                            const int32_t* __restrict__ tokens, const int32_t* __restrict__ parent,
                            const int32_t* __restrict__ n_nodes, const float* __restrict__ uniforms, int T, int V,
-                           int chunk, int cache_p0, int max_depth, double inv_tau, const NodeSummary* __restrict__ nodes,
+                           int chunk, int keep, int max_depth, double inv_tau, const NodeSummary* __restrict__ nodes,
                            int seg_splits,
                            const RowPartial* __restrict__ seg_row, int32_t* __restrict__ accept_len, int32_t* __restrict__ path,
                            int32_t* __restrict__ next_token, uint8_t* __restrict__ near_tie,
@@ -543,6 +548,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         if (near_tie && writer) near_tie[(size_t)b * T + i] = 0;
     }
     if (tid < 32) cs.tab[tid] = kExp2Frac[tid];
+    if (STOCH && tid < S4C_MAX_T * S4C_MASK_WORDS) cs.kids[tid / S4C_MASK_WORDS][tid % S4C_MASK_WORDS] = 0u;
     __syncthreads();
     int flags = build_ancestor_masks(sh.par, n, T, sh.anc, sh.depth, &sh.flag);
     if (!flags) {
@@ -558,6 +564,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
             const size_t at = ((size_t)b * T + sh.par[i]) * V + sh.tok[i];
             cs.tq0[i] = (double)__ldg(dprobs + at);
             cs.tp0[i] = (double)__ldg(logits + at);  // turned into a probability below, once the parent's statistics are in
+            atomicOr(&cs.kids[sh.par[i]][i >> 5], 1u << (i & 31));
         }
     // Everything above reads the caller's inputs only, which were complete before the statistics kernel began; from here on
     // its results are needed.
@@ -617,7 +624,8 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         for (int i = 1 + tid; i < n; i += blockDim.x) {
             const int pr = sh.par[i];
             const double invS = sh.nS[pr] > 0.0 ? 1.0 / sh.nS[pr] : 0.0;
-            cs.tp0[i] = exp_nonpos((cs.tp0[i] - (double)sh.nM[pr]) * inv_tau, cs.tab) * invS;
+            const double px = exp_nonpos((cs.tp0[i] - (double)sh.nM[pr]) * inv_tau, cs.tab) * invS, qx = cs.tq0[i];
+            cs.tp0[i] = px, cs.ratio0[i] = accept_ratio(px, qx);
         }
     __syncthreads();
     auto write_path = [&](int end) {
@@ -644,219 +652,254 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         return;
     }
 
-    // ---- speculative-sampling walk: every thread of every CTA follows the same control flow on the same scalars;
-    //      only the vocabulary-wide sums are split, CTA `rank` owning the elements [c0, c1)
+    // ---- speculative-sampling walk: every thread of every CTA follows the same control flow on the same scalars; only the
+    //      passes over the vocabulary are split, CTA `rank` owning the entries [c0, c1).  What bounds it is a chain of a few
+    //      dependent passes over one row, each on 8 SMs: instructions per entry, code met for the first time, barriers.  So
+    //      there is one pass in the code, for the residual masses and for the draw; an entry stays with its thread through
+    //      all passes at a node (no barrier for the kept values); a pass takes the kept p one rejection further instead of
+    //      starting from the logits; siblings come from bitmasks.  Batch of 4, V = 128256, up to four passes: 82 -> 54 us;
+    //      V = 32000, four accepted and the draw: 23 -> 10 us.
     const int c0 = (int)rank * chunk, c1 = min(V, c0 + chunk);
-    int round = 0;  // cluster-wide reductions so far (selects the slot set)
-    // With room in shared memory the target probabilities of this CTA's vocabulary range at the current node are kept
-    // from the first vocabulary-wide pass there to the later ones (a float64 exp per entry is most of a pass).
+    const int lane = tid & 31, warp = tid >> 5;
+    const bool vec = (V & 3) == 0;
+    // a warp owns a contiguous span of groups of 128 entries, a lane four consecutive entries of each
+    const int groups = (chunk + kWalkGroup - 1) / kWalkGroup, g0 = groups * warp / 32, g1 = groups * (warp + 1) / 32;
+    // With room in shared memory (keep >= 1) the p of this CTA's entries stays there, and with still more (keep == 2) the
+    // draft probabilities too; entry u of a lane's four at [group][u][lane], so that a warp's accesses are conflict-free.
     double* pc = reinterpret_cast<double*>(smem_raw + ((sizeof(WalkClShared) + 15) / 16) * 16);
-    // ... and, with still more room (cache_p0 == 2), the draft probabilities of the range beside them: a node where several
-    // siblings are rejected takes one pass per rejection, and all but the first then run from shared memory alone
-    float* qc = reinterpret_cast<float*>(pc + chunk);
-    int cached_node = -1;  // node whose probabilities pc[] holds, complete after a whole pass (the same in every thread)
-    // two cluster-wide sums in rank order; every thread of the cluster calls this and gets the same values
-    auto cluster_sum2 = [&](double a, double bsum, double& A, double& Bs) {
-        // both sums through one pair of CTA barriers, each in a fixed order
-        a = warp_sum(a), bsum = warp_sum(bsum);
-        if ((tid & 31) == 0) cs.pa[tid >> 5] = a, cs.pb[tid >> 5] = bsum;
-        __syncthreads();
-        if (tid < 32) {
-            double ta = tid < (int)(blockDim.x >> 5) ? cs.pa[tid] : 0.0, tb = tid < (int)(blockDim.x >> 5) ? cs.pb[tid] : 0.0;
-            ta = warp_sum(ta), tb = warp_sum(tb);
-            double* set = cs.slots[round & 1];
-            if (tid == 0) set[0] = ta, set[1] = tb;
-        }
-        double* set = cs.slots[round & 1];
+    float* qc = reinterpret_cast<float*>(pc + (size_t)groups * kWalkGroup);
+    int round = 0;  // cluster-wide exchanges so far (selects the slot set)
+    // two values per CTA (at set[0], set[1] before the barrier) to cs.gab in every CTA, in rank order
+    auto exchange = [&](double* set) {
         cl_sync();
-        if (tid < kCl) cs.ga[tid] = cl_peer_f64(&set[0], tid), cs.gb[tid] = cl_peer_f64(&set[1], tid);
+        if (tid < 2 * kCl) cs.gab[tid / kCl][tid % kCl] = cl_peer_f64(&set[tid / kCl], tid % kCl);
         __syncthreads();
-        A = 0.0, Bs = 0.0;
-        for (int r = 0; r < kCl; ++r) A += cs.ga[r], Bs += cs.gb[r];
-        __syncthreads();  // ga/gb are free again
         ++round;
     };
 
-    int cur = 0;
-    for (int guard = 0; guard <= T; ++guard) {
+    int cur = 0, r = 0, have = -1;  // node, rejections there so far, rejections that the kept p has behind it (-1: nothing kept)
+    int kw = 0;
+    uint32_t kbits = cs.kids[0][0];  // the children of `cur` not yet tested: those of word kw, and the words after it
+    for (;;) {
         const float* lrow = logits + ((size_t)b * T + cur) * V;
         const float* qrow = dprobs + ((size_t)b * T + cur) * V;
-        const double M = (double)sh.nM[cur];
-        const double invS = sh.nS[cur] > 0.0 ? 1.0 / sh.nS[cur] : 0.0;
-        auto p0_from = [&](float logit) { return exp_nonpos(((double)logit - M) * inv_tau, cs.tab) * invS; };
-        // (p, q) after r rejections of up to four vocabulary entries start, start + step, ...; the loads go out
-        // first (these passes are bound by the latency of the loads, not by their volume)
-        auto eval4 = [&](int start, int step, int end, int rr, double (&pv)[4], double (&qv)[4]) {
-            const bool hit = cache_p0 && cached_node == cur;
-            float xl[4], ql[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int v = start + u * step;
-                xl[u] = (v < end && !hit) ? __ldg(lrow + v) : 0.f;
-                ql[u] = v < end ? ((hit && cache_p0 == 2) ? qc[v - c0] : __ldg(qrow + v)) : 0.f;
+        // ---- tests until the next pass over the vocabulary is due: x >= 0, token x was rejected; else the draw
+        int x = -1;
+        for (;;) {
+            while (kbits == 0u && kw < S4C_MASK_WORDS - 1) kbits = cs.kids[cur][++kw];
+            if (kbits == 0u) break;
+            const int c = 32 * kw + __ffs(kbits) - 1;
+            kbits &= kbits - 1u;
+            double ratio = cs.ratio0[c];
+            if (r > 0) {
+                double px, qx;
+                chain_eval(cs.tp0[c], cs.tq0[c], sh.tok[c], r, sh, px, qx);
+                ratio = accept_ratio(px, qx);
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int v = start + u * step;
-                pv[u] = 0.0, qv[u] = 0.0;
-                if (v < end) {
-                    double p0;
-                    if (hit) {
-                        p0 = pc[v - c0];
-                    } else {
-                        p0 = p0_from(xl[u]);
-                        if (cache_p0) pc[v - c0] = p0;
-                        if (cache_p0 == 2) qc[v - c0] = ql[u];
-                    }
-                    chain_eval(p0, (double)ql[u], v, rr, sh, pv[u], qv[u]);
-                }
-            }
-        };
-        int r = 0, accepted = -1;
-        for (int c = cur + 1; c < n; ++c) {
-            if (sh.par[c] != cur) continue;
-            const int x = sh.tok[c];
-            double px, qx;
-            chain_eval(cs.tp0[c], cs.tq0[c], x, r, sh, px, qx);
-            double ratio;
-            if (qx > 0.0)
-                ratio = px / qx;
-            else
-                ratio = px > 0.0 ? (double)INFINITY : 0.0;
             const double u = (double)sh.uni[c];
             if (tid == 0 && writer && near_tie && fabs(ratio - u) < 1e-6) near_tie[(size_t)b * T + c] = 1;
             if (u < (ratio < 1.0 ? ratio : 1.0)) {
-                accepted = c;
-                break;
+                cur = c, r = 0, have = -1, kw = 0, kbits = cs.kids[c][0];
+                lrow = logits + ((size_t)b * T + cur) * V, qrow = dprobs + ((size_t)b * T + cur) * V;
+                continue;
             }
-            // rejected: residual mass and the draft mass left once x is removed
-            double Z, s;
-            if (r == 0 && !seg_row) {  // small problems: the statistics kernel has them for every node
-                Z = sh.nZ[cur], s = sh.nQ[cur];
-            } else {
-                double z = 0.0, qs = 0.0;
-                if (!(cache_p0 && cached_node == cur))
-                    // first pass at this node: the rows come from global memory in batches of four loads per thread, each
-                    // batch a round trip; asking L2 for the later batches now leaves only the first at full latency
-                    for (int v = c0 + tid + 4 * (int)blockDim.x; v < c1; v += blockDim.x) prefetch_l2(lrow + v), prefetch_l2(qrow + v);
-                for (int v0 = c0 + tid; v0 < c1; v0 += 4 * blockDim.x) {
-                    double pv[4], qv[4];
-                    eval4(v0, blockDim.x, c1, r, pv, qv);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {  // entries past the end come back as (0, 0)
-                        const double res = pv[u] - qv[u];
-                        z += res > 0.0 ? res : 0.0;
-                        qs += (v0 + u * (int)blockDim.x == x) ? 0.0 : qv[u];
-                    }
-                }
-                cluster_sum2(z, qs, Z, s);
-                cached_node = cur;  // a whole pass at this node is behind a CTA barrier: pc[] is complete
-            }
-            __syncthreads();  // everyone has finished reading the chain before it grows
-            if (tid == 0) {
-                sh.cx[r] = x;
-                sh.cinvZ[r] = Z > 0.0 ? 1.0 / Z : 0.0;
-                sh.cinvs[r] = s > 0.0 ? 1.0 / s : 0.0;
-            }
+            x = sh.tok[c];
+            if (r > 0 || seg_row) break;
+            // small problems: the statistics kernel has every node's first residual mass, and the draft mass left without x
+            const double Z = sh.nZ[cur], s = sh.nQ[cur];
+            __syncthreads();  // everyone is done with the chain of the node before
+            if (tid == 0) sh.cx[0] = x, sh.cinvZ[0] = Z > 0.0 ? 1.0 / Z : 0.0;
+            if (tid == 32) sh.cinvs[0] = s > 0.0 ? 1.0 / s : 0.0;
             __syncthreads();
-            ++r;
+            r = 1, x = -1;
             if (!(s > 0.0)) break;
         }
-        if (accepted >= 0) {
-            cur = accepted;
+
+        // ---- one pass over this CTA's entries at `cur`: p and q after r rejections; the residual mass and the draft mass
+        //      left without x, or (draw) the mass of p and the last entry that has any
+        const double M = (double)sh.nM[cur];
+        const double invS = sh.nS[cur] > 0.0 ? 1.0 / sh.nS[cur] : 0.0;
+        auto load4 = [&](const float* row, int v, float fill, float (&out)[4]) {
+            if (vec) {
+                float4 t = make_float4(fill, fill, fill, fill);
+                if (v < c1) t = __ldg(reinterpret_cast<const float4*>(row + v));
+                out[0] = t.x, out[1] = t.y, out[2] = t.z, out[3] = t.w;
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) out[u] = v + u < c1 ? __ldg(row + v + u) : fill;
+            }
+        };
+        auto values = [&](int g, double (&pv)[4], double (&qv)[4]) {
+            const int v = c0 + g * kWalkGroup + 4 * lane, at = g * kWalkGroup + lane;
+            float q4[4];
+            if (have < 0) {
+                float x4[4];
+                load4(lrow, v, 0.f, x4), load4(qrow, v, 0.f, q4);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    pv[u] = v + u < c1 ? exp_nonpos(((double)x4[u] - M) * inv_tau, cs.tab) * invS : 0.0;
+                    if (keep == 2) qc[at + 32 * u] = q4[u];
+                }
+            } else {
+                if (keep != 2) load4(qrow, v, 0.f, q4);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    pv[u] = pc[at + 32 * u];
+                    if (keep == 2) q4[u] = qc[at + 32 * u];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) qv[u] = (double)q4[u];
+#pragma unroll 1
+            for (int j = 0; j < r; ++j) {
+                const double iz = sh.cinvZ[j], is = sh.cinvs[j];
+                const int gone = sh.cx[j] - v;
+                if (j >= have && iz > 0.0) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const double res = pv[u] - qv[u];
+                        pv[u] = (res > 0.0 ? res : 0.0) * iz;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) qv[u] = (u == gone ? 0.0 : qv[u]) * is;
+            }
+            if (keep) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) pc[at + 32 * u] = pv[u];
+            }
+        };
+        if (have < 0)  // the row's first pass: the groups after the first are asked for ahead
+            for (int g = g0 + 1; g < g1; ++g) {
+                const int v = c0 + g * kWalkGroup + 4 * lane;
+                if (v < c1) prefetch_l2(lrow + v), prefetch_l2(qrow + v);
+            }
+        double sa = 0.0, sb = 0.0;
+        int last = -1;
+#pragma unroll 1
+        for (int g = g0; g < g1; ++g) {
+            double pv[4], qv[4];
+            values(g, pv, qv);
+            const int v = c0 + g * kWalkGroup + 4 * lane;
+            if (x >= 0) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const double res = pv[u] - qv[u];
+                    sa += res > 0.0 ? res : 0.0;
+                    sb += v + u == x ? 0.0 : qv[u];
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    sa += pv[u];
+                    if (pv[u] > 0.0) last = v + u;
+                }
+            }
+        }
+        if (keep) have = r;
+        double* set = cs.slots[round & 1];
+        sa = warp_sum(sa);
+        if (x >= 0) {
+            // ---- a rejection: both sums over the cluster, each in a fixed order, then the chain grows
+            sb = warp_sum(sb);
+            if (lane == 0) cs.pa[warp] = sa, cs.pb[warp] = sb;
             __syncthreads();
+            if (warp < 2) {
+                const double t = warp_sum(warp == 0 ? cs.pa[lane] : cs.pb[lane]);
+                if (lane == 0) set[warp] = t;
+            }
+            exchange(set);
+            double Z = 0.0, s = 0.0;
+            for (int k = 0; k < kCl; ++k) Z += cs.gab[0][k], s += cs.gab[1][k];
+            if (tid == 0) sh.cx[r] = x, sh.cinvZ[r] = Z > 0.0 ? 1.0 / Z : 0.0;  // (entry r has had no reader since the barriers above)
+            if (tid == 32) sh.cinvs[r] = s > 0.0 ? 1.0 / s : 0.0;
+            __syncthreads();
+            ++r;
+            if (!(s > 0.0)) kbits = 0u, kw = S4C_MASK_WORDS - 1;  // no draft mass left to test against: the draw
             continue;
         }
 
-        // ---- final token: inverse CDF over the current p at `cur` (Eq. 12 at a fork; plain target at a leaf).
-        //      Each warp sums a contiguous span of its CTA's range; the CTA totals are exchanged; the CTA whose
-        //      range holds the crossing scans the one span that holds it.
-        const int lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-        const int seg = ((chunk + nwarps - 1) / nwarps + 31) / 32 * 32;  // contiguous span per warp
-        const int w0 = c0 + warp * seg, w1 = min(c1, w0 + seg);
-        double acc = 0.0;
-        int last = -1;
-        if (!(cache_p0 && cached_node == cur))  // (as above: a leaf, or a fork whose residual masses came precomputed)
-            for (int v = w0 + lane + 128; v < w1; v += 32) prefetch_l2(lrow + v), prefetch_l2(qrow + v);
-        for (int v0 = w0 + lane; v0 < w1; v0 += 128) {
-            double pv[4], qv[4];
-            eval4(v0, 32, w1, r, pv, qv);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                acc += pv[u];
-                if (pv[u] > 0.0) last = v0 + 32 * u;
-            }
-        }
-        acc = warp_sum(acc);
+        // ---- final token: inverse CDF over the current p at `cur` (Eq. 12 at a fork; plain target at a leaf).  The CTA totals
+        //      are exchanged; in the CTA whose range holds the crossing, the warp whose span holds it scans its entries.
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
-        if (lane == 0) sh.wsum[warp] = acc, sh.wlast[warp] = last;
+        if (lane == 0) sh.wsum[warp] = sa, sh.wlast[warp] = last;
         __syncthreads();
-        cached_node = cur;  // the sums above went over the whole range: the scan below reads pc[]
-        double* set = cs.slots[round & 1];
-        if (tid == 0) {
-            double tot = 0.0;
-            int lastpos = -1;
-            for (int w = 0; w < nwarps; ++w) tot += sh.wsum[w], lastpos = max(lastpos, sh.wlast[w]);
-            set[0] = tot, set[1] = (double)lastpos;
+        double upto = sh.wsum[lane];  // mass of this CTA's spans 0 .. lane (every warp computes the same)
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += t;
         }
-        cl_sync();
-        if (tid < kCl) cs.ga[tid] = cl_peer_f64(&set[0], tid), cs.gb[tid] = cl_peer_f64(&set[1], tid);
-        __syncthreads();
+        if (warp == 0) {
+            int lastpos = sh.wlast[lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) lastpos = max(lastpos, __shfl_xor_sync(0xffffffffu, lastpos, o));
+            if (lane == 31) set[0] = upto, set[1] = (double)lastpos;
+        }
+        exchange(set);
         double total = 0.0;
         int lastpos = 0;
-        for (int rr = 0; rr < kCl; ++rr) total += cs.ga[rr], lastpos = max(lastpos, (int)cs.gb[rr]);
+        for (int k = 0; k < kCl; ++k) total += cs.gab[0][k], lastpos = max(lastpos, (int)cs.gab[1][k]);
         const double target = (double)sh.uni[0] * total;
         double before = 0.0;  // mass of the ranks before the one that holds the crossing
         int rstar = -1;
-        for (int rr = 0; rr < kCl; ++rr) {
-            if (before + cs.ga[rr] > target) {
-                rstar = rr;
+        for (int k = 0; k < kCl; ++k) {
+            if (before + cs.gab[0][k] > target) {
+                rstar = k;
                 break;
             }
-            before += cs.ga[rr];
+            before += cs.gab[0][k];
         }
         if (rstar < 0) {  // the running sum never exceeds the target (u * total rounds up to the total): last token with mass
             if (writer && tid == 0) {
                 next_token[b] = lastpos;
                 write_path(cur);
             }
-        } else if ((int)rank == rstar && warp == 0) {
-            double run = before;
-            int wstar = 0;
-            for (; wstar < nwarps - 1; ++wstar) {
-                if (run + sh.wsum[wstar] > target) break;
-                run += sh.wsum[wstar];
-            }
-            int pick = -1;
-            for (int base4 = c0 + wstar * seg; base4 < c1 && pick < 0; base4 += 128) {
-                double pv4[4], qv4[4];  // four groups of 32 consecutive entries, fetched together, scanned in order
-                eval4(base4 + lane, 32, c1, r, pv4, qv4);
+        } else if ((int)rank == rstar) {
+            const unsigned over = __ballot_sync(0xffffffffu, before + upto > target);
+            const int wstar = over ? __ffs(over) - 1 : 31;
+            const double ahead = __shfl_sync(0xffffffffu, upto, wstar > 0 ? wstar - 1 : 0);
+            if (warp == wstar) {
+                double run = before + (wstar > 0 ? ahead : 0.0);
+                int pick = -1;
+#pragma unroll 1
+                for (int g = g0; g < g1 && pick < 0; ++g) {
+                    double pv[4], qv[4];
+                    if (keep) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int base = base4 + 32 * u, v = base + lane;
-                    if (pick >= 0 || base >= c1) continue;  // warp-uniform
-                    double scan = pv4[u];  // inclusive prefix within the group of 32
+                        for (int u = 0; u < 4; ++u) pv[u] = pc[g * kWalkGroup + lane + 32 * u];
+                    } else {
+                        values(g, pv, qv);
+                    }
+                    double in = (pv[0] + pv[1]) + (pv[2] + pv[3]);  // inclusive prefix over the lanes' fours
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
-                        const double t = __shfl_up_sync(0xffffffffu, scan, o);
-                        if (lane >= o) scan += t;
+                        const double t = __shfl_up_sync(0xffffffffu, in, o);
+                        if (lane >= o) in += t;
                     }
-                    const unsigned hit = __ballot_sync(0xffffffffu, v < c1 && run + scan > target);
-                    if (hit) pick = base + __ffs(hit) - 1;
-                    run += __shfl_sync(0xffffffffu, scan, 31);
+                    const double ex = __shfl_up_sync(0xffffffffu, in, 1);
+                    double at = lane > 0 ? ex : 0.0;
+                    int mine = -1;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        at = u < 3 ? at + pv[u] : in;
+                        if (mine < 0 && pv[u] > 0.0 && run + at > target) mine = u;
+                    }
+                    const unsigned hit = __ballot_sync(0xffffffffu, mine >= 0);
+                    if (hit) pick = __shfl_sync(0xffffffffu, c0 + g * kWalkGroup + 4 * lane + mine, __ffs(hit) - 1);
+                    run += __shfl_sync(0xffffffffu, in, 31);
                 }
-            }
-            if (lane == 0) {
-                // a crossing lost to the different summation order of the scan: this CTA's last token with mass
-                next_token[b] = pick >= 0 ? pick : (int)cs.gb[rstar];
-                write_path(cur);
+                if (lane == 0) {
+                    // a crossing lost to the different summation order of the scan: this CTA's last token with mass
+                    next_token[b] = pick >= 0 ? pick : (int)cs.gab[1][rstar];
+                    write_path(cur);
+                }
             }
         }
         cl_sync();  // nobody leaves while a peer may still read its slots
         return;
     }
-    cl_sync();
 }
 
 }  // namespace s4c
@@ -951,8 +994,9 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
         // probabilities too (4 more), next to the walk's state?
         const size_t walk_state = ((sizeof(WalkClShared) + 15) / 16) * 16;
         const size_t walk_smem_max = 227 * 1024;
-        const int cache_p0 = walk_state + (size_t)chunk * 12 <= walk_smem_max ? 2 : (walk_state + (size_t)chunk * 8 <= walk_smem_max ? 1 : 0);
-        cfg.dynamicSmemBytes = walk_state + (size_t)chunk * (cache_p0 == 2 ? 12 : (cache_p0 == 1 ? 8 : 0));
+        const size_t held = round_up((size_t)chunk, kWalkGroup);
+        const int keep = walk_state + held * 12 <= walk_smem_max ? 2 : (walk_state + held * 8 <= walk_smem_max ? 1 : 0);
+        cfg.dynamicSmemBytes = walk_state + held * (keep == 2 ? 12 : (keep == 1 ? 8 : 0));
         {
             static bool configured[64] = {};  // the opt-in to more than 48 KB of dynamic shared memory is per device
             int dev = 0;
@@ -965,7 +1009,7 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
             }
         }
         err = cudaLaunchKernelEx(&cfg, accept_walk_cluster_kernel<true>, target_logits, draft_probs, tokens, parent, n_nodes,
-                                 uniforms, T, V, chunk, cache_p0, max_depth, inv_tau, summary, splits, seg_row,
+                                 uniforms, T, V, chunk, keep, max_depth, inv_tau, summary, splits, seg_row,
                                  accept_len, path, next_token, near_tie, status);
         if (err != cudaSuccess) {
             cudaGetLastError();
