@@ -231,6 +231,55 @@ tree_emit_topk_kernel(const int32_t* __restrict__ topk, int k, const __grid_cons
     if (threadIdx.x == 0) n_nodes[b] = shape.n;
 }
 
+// Between two heads of a drafting round: a block per row of the next head (its token, position, embedding row and parent's
+// feature row), and one block per sequence that stores the choices and writes the tree.  Every block takes the tokens of the new
+// level from `choice` itself, so none waits for another.  Bound by the launch: as six calls (the choices' copy, the tree, two
+// copies of slices, two gathers) this was 13 us of launches between two heads of a 7B round, 2.6 us as one.
+__global__ void __launch_bounds__(256)
+draft_level_kernel(const int32_t* __restrict__ choice, int k, const __grid_constant__ TreeShape shape, int from_first, int from_count,
+                   int to_first, int to_count, const int32_t* __restrict__ root_token, const int32_t* __restrict__ root_position, int T,
+                   int32_t* __restrict__ topk_all, int32_t* __restrict__ tokens, int32_t* __restrict__ parent,
+                   int32_t* __restrict__ position, int32_t* __restrict__ n_nodes, const uint4* __restrict__ embedding, int V,
+                   const uint4* __restrict__ features, int words, uint4* __restrict__ e_out, uint4* __restrict__ f_out,
+                   int32_t* __restrict__ tok_out, int32_t* __restrict__ pos_out) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int b = blockIdx.y, tid = threadIdx.x;
+    const int base = root_position ? root_position[b] : 0;
+    const int32_t* mine = choice + (size_t)b * from_count * k;
+    if ((int)blockIdx.x < to_count) {
+        const int node = to_first + blockIdx.x, p = shape.parent[node];
+        const int tok = mine[(p - from_first) * k + node - (int)shape.first_child[p]];
+        const size_t row = (size_t)b * to_count + blockIdx.x, from = (size_t)b * from_count + (p - from_first);
+        const bool ok = tok >= 0 && tok < V;
+        if (tid == 0) tok_out[row] = tok, pos_out[row] = base + (int)shape.depth[node];
+        for (int i = tid; i < words; i += blockDim.x) {
+            uint4 e = make_uint4(0, 0, 0, 0);
+            if (ok) e = embedding[(size_t)tok * words + i];
+            const uint4 f = features[from * words + i];
+            e_out[row * words + i] = e, f_out[row * words + i] = f;
+        }
+        return;
+    }
+    int32_t* all = topk_all + (size_t)b * T * k;
+    for (int i = tid; i < from_count * k; i += blockDim.x) all[from_first * k + i] = mine[i];
+    for (int i = tid; i < T; i += blockDim.x) {
+        const bool used = i < shape.n;
+        const int p = used ? (int)shape.parent[i] : -1;
+        int tok = 0;
+        if (i == 0) {
+            tok = root_token[b];
+        } else if (used) {
+            const int rank = i - (int)shape.first_child[p], at = p - from_first;
+            tok = at >= 0 && at < from_count ? mine[at * k + rank] : all[p * k + rank];
+        }
+        parent[(size_t)b * T + i] = p;
+        position[(size_t)b * T + i] = used ? base + (int)shape.depth[i] : 0;
+        tokens[(size_t)b * T + i] = tok;
+    }
+    if (tid == 0) n_nodes[b] = shape.n;
+}
+
 static inline int tb_segments(int V) { return ceil_div(V, kTbSeg); }
 
 }  // namespace s4c
@@ -290,5 +339,42 @@ extern "C" s4c_status s4c_tree_build_topk(const int32_t* topk, int k, const int3
     tree_emit_topk_kernel<<<B, 128, 0, static_cast<cudaStream_t>(stream_)>>>(topk, k, shape, root_token, cache_len, T, tokens, parent,
                                                                             position, n_nodes);
     S4C_RETURN_IF_CUDA_ERROR();
+    return S4C_OK;
+}
+
+extern "C" s4c_status s4c_draft_level(const int32_t* choice, int k, const int32_t* branching, int depth, int from_first, int from_count,
+                                      int to_first, int to_count, const int32_t* root_token, const int32_t* root_position, int B,
+                                      int T, int32_t* topk_all, int32_t* tokens, int32_t* parent, int32_t* position,
+                                      int32_t* n_nodes, const void* embedding, int V, const void* features, int H, void* e_out,
+                                      void* f_out, int32_t* tok_out, int32_t* pos_out, s4c_stream_t stream_) {
+    using namespace s4c;
+    if (!choice || !topk_all || !root_token || !tokens || !parent || !position || !n_nodes || (depth > 0 && !branching)) return S4C_ERR_NULL;
+    if (to_count > 0 && (!embedding || !features || !e_out || !f_out || !tok_out || !pos_out)) return S4C_ERR_NULL;
+    if (B < 0 || B > 65535 || T < 1 || T > S4C_MAX_T || k < 1 || depth < 0 || depth >= S4C_MAX_T) return S4C_ERR_SHAPE;
+    for (int l = 0; l < depth; ++l)
+        if (branching[l] < 1 || branching[l] > k) return S4C_ERR_SHAPE;
+    TreeShape shape;
+    lay_out_tree(branching, depth, T, &shape);
+    if (from_first < 0 || from_count < 1 || from_first + from_count > shape.n || to_count < 0) return S4C_ERR_SHAPE;
+    if (to_count > 0) {
+        if (V < 1 || H < 8 || H % 8 != 0 || to_first < 1 || to_first + to_count > shape.n) return S4C_ERR_SHAPE;
+        for (int i = to_first; i < to_first + to_count; ++i)  // every one a child of a node whose choices these are
+            if (shape.parent[i] < from_first || shape.parent[i] >= from_first + from_count) return S4C_ERR_SHAPE;
+        if (!aligned16(embedding) || !aligned16(features) || !aligned16(e_out) || !aligned16(f_out)) return S4C_ERR_ALIGN;
+    }
+    if (B == 0) return S4C_OK;
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(to_count + 1, B, 1), cfg.blockDim = dim3(256, 1, 1), cfg.stream = static_cast<cudaStream_t>(stream_);
+    cfg.attrs = &pdl, cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, draft_level_kernel, choice, k, shape, from_first, from_count, to_first, to_count, root_token, root_position,
+                           T, topk_all, tokens, parent, position, n_nodes, static_cast<const uint4*>(embedding), V,
+                           static_cast<const uint4*>(features), H / 8, static_cast<uint4*>(e_out), static_cast<uint4*>(f_out), tok_out,
+                           pos_out) != cudaSuccess) {
+        cudaGetLastError();
+        return S4C_ERR_CUDA;
+    }
     return S4C_OK;
 }

@@ -89,8 +89,12 @@ class DrafterHead:
         ``position_base`` [B] int32: the roots' positions in the text when the head's own cache is shorter than the text
         (s4c_qkv_rope_at); None: the cache lengths.
         Returns dict(token [B*T,k], logit [B*T,k], features [B*T,H])."""
+        s4c.embed_gather(self.w.embedding, tokens.reshape(-1), out=self.e)
+        return self._layer(features, cache_len, parent, k_cache, v_cache, n_nodes, max_cache_len, position_base)
+
+    def _layer(self, features, cache_len, parent, k_cache, v_cache, n_nodes=None, max_cache_len=0, position_base=None):
+        """`forward` behind the embedding (the tokens' rows stand in `self.e`)."""
         w = self.w
-        s4c.embed_gather(w.embedding, tokens.reshape(-1), out=self.e)
         s4c.linear_rmsnorm(self.e, w.fc, w.norm1, self.eps, x2=features, bias=w.fc_bias, out=self.h, norm_out=self.a,
                            workspace=self.ws_lin)
         s4c.qkv_rope(self.a.view(self.B, self.T, -1), w.qkv, cache_len, parent, self.q, k_cache, v_cache, n_nodes, self.rope_theta,
@@ -114,12 +118,12 @@ class MultiHeadDrafter:
     the attention call (T = 1), so a head's cache holds one copy of the prefix per row of its level.  A row's input is
     (Embedding(the node's token), the output feature of the node's parent); for depth 1 that parent is the root and its
     feature is the target's f_0, shared by all of the root's candidates.  The head's ranked choices give the node's children
-    their tokens (child r = the r-th choice): `s4c_tree_build_topk` is called after every head on the choices known so far.
+    their tokens (child r = the r-th choice): `s4c_draft_level` extends the tree after every head and lays out the next head's rows.
     A row's rotary position is root_position + depth (`position_base` of `s4c_qkv_rope_at`); its cache slot counts the
     head's own entries.
 
     Only buffers, the static row maps and the order of the calls live here; the per-row work is `DrafterHead`'s chain of
-    library calls, the feature hand-over between levels is `s4c_embed_gather` with the previous level's features as its table.
+    library calls.
     """
 
     def __init__(self, heads, B: int, T: int, branching, Hq: int, Hkv: int, d: int, C: int, k: int, eps: float = 1e-5,
@@ -144,17 +148,11 @@ class MultiHeadDrafter:
             assert nodes == list(range(nodes[0], nodes[-1] + 1))
             self.levels.append((nodes[0], nodes[-1] + 1))
         self.n_passes = min(len(heads), len(self.levels))  # leaves below the last head's level get tokens, no pass
-        self.heads, self.parent_rows, self.minus_one, self.feat_in = [], [], [], []
+        self.heads, self.minus_one, self.feat_in = [], [], []
         for j in range(self.n_passes):
             s, e = self.levels[j]
             nj = e - s
             self.heads.append(DrafterHead(heads[j], B * nj, 1, Hq, Hkv, d, C, k, eps, rope_theta))
-            if j == 0:
-                rows = [b for b in range(B) for _ in range(nj)]  # the root's feature f_0[b], reused by all its candidates
-            else:
-                ps, pe = self.levels[j - 1]
-                rows = [b * (pe - ps) + parent[i] - ps for b in range(B) for i in range(s, e)]
-            self.parent_rows.append(torch.tensor(rows, **i32))
             self.minus_one.append(torch.full((B * nj, 1), -1, **i32))
             self.feat_in.append(torch.empty(B * nj, self.H, dtype=torch.bfloat16, device=dev))
         self.tok_rows = [torch.empty(B * (e - s), 1, **i32) for s, e in self.levels[: self.n_passes]]
@@ -166,20 +164,19 @@ class MultiHeadDrafter:
         (k_cache, v_cache, cache_len) with one sequence per row of the head's level ([B * n_j, Hkv, C, d], [B * n_j] int32).
         Returns dict(tokens, parent, position, n_nodes) of the tree and the heads' features per level."""
         B, k = self.B, self.k
-        self.topk_all[:, 0, :].copy_(target_topk)
-        tree = s4c.tree_build_topk(self.topk_all, self.branching, root_token, root_position, **self.tree)
-        feats_prev = f0
+        choice = target_topk
+        if choice.dtype != torch.int32 or choice.shape != (B, k) or not choice.is_contiguous():
+            choice = torch.empty(B, k, dtype=torch.int32, device=self.topk_all.device).copy_(target_topk)
+        tree = self.tree
+        feats_prev, level = f0, (0, 1)  # the root's feature is shared by all its candidates
         features = []
         for j in range(self.n_passes):
-            s, e = self.levels[j]
-            nj = e - s
-            self.tok_rows[j].view(B, nj).copy_(tree["tokens"][:, s:e])
-            self.pos_rows[j].view(B, nj).copy_(tree["position"][:, s:e])  # root_position + depth
-            s4c.embed_gather(feats_prev, self.parent_rows[j], out=self.feat_in[j])
+            head = self.heads[j]
+            s4c.draft_level(choice, self.branching, (level, self.levels[j]), self.topk_all, tree, root_token, root_position,
+                            head.w.embedding, feats_prev, head.e, self.feat_in[j], self.tok_rows[j], self.pos_rows[j])
             kc, vc, cl = caches[j]
-            out = self.heads[j].forward(self.tok_rows[j], self.feat_in[j], cl, self.minus_one[j], kc, vc, position_base=self.pos_rows[j])
-            self.topk_all[:, s:e, :].copy_(out["token"].view(B, nj, k))
-            feats_prev = out["features"]
+            out = head._layer(self.feat_in[j], cl, self.minus_one[j], kc, vc, position_base=self.pos_rows[j])
+            choice, feats_prev, level = out["token"], out["features"], self.levels[j]
             features.append(feats_prev)
-            tree = s4c.tree_build_topk(self.topk_all, self.branching, root_token, root_position, **self.tree)
+        s4c.draft_level(choice, self.branching, (level, None), self.topk_all, tree, root_token, root_position)
         return dict(tokens=tree["tokens"], parent=tree["parent"], position=tree["position"], n_nodes=tree["n_nodes"], features=features)

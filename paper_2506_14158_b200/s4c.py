@@ -27,7 +27,7 @@ EXPORTS = ["s4c_version", "s4c_status_string", "s4c_tree_attention_workspace_byt
            "s4c_tree_attention_paged", "s4c_kv_compact_paged", "s4c_tree_accept_filtered_workspace_bytes",
            "s4c_tree_accept_filtered", "s4c_lm_head_greedy_workspace_bytes", "s4c_lm_head_greedy", "s4c_tree_accept_tokens",
            "s4c_qkv_rope_workspace_bytes", "s4c_qkv_rope", "s4c_qkv_rope_at", "s4c_qkv_rope_same_tree", "s4c_lm_head_topk_workspace_bytes", "s4c_lm_head_topk",
-           "s4c_tree_build_topk", "s4c_lm_head_logits_workspace_bytes", "s4c_lm_head_logits", "s4c_linear_workspace_bytes", "s4c_linear", "s4c_linear_rmsnorm", "s4c_rmsnorm", "s4c_embed_gather"]
+           "s4c_tree_build_topk", "s4c_draft_level", "s4c_lm_head_logits_workspace_bytes", "s4c_lm_head_logits", "s4c_linear_workspace_bytes", "s4c_linear", "s4c_linear_rmsnorm", "s4c_rmsnorm", "s4c_embed_gather"]
 NOALLOC_SCRATCH_BYTES = 1 << 20
 
 
@@ -95,6 +95,8 @@ def _load() -> ctypes.CDLL:
     lib.s4c_linear_rmsnorm.argtypes = [vp, vp, vp, vp, vp, vp, i, i, i, i, vp, f, vp, i32p, vp, sz, vp]
     lib.s4c_rmsnorm.restype = i
     lib.s4c_rmsnorm.argtypes = [vp, vp, f, i, i, vp, vp]
+    lib.s4c_draft_level.restype = i
+    lib.s4c_draft_level.argtypes = [i32p, i, vp, i, i, i, i, i, i32p, i32p, i, i, i32p, i32p, i32p, i32p, i32p, vp, i, vp, i, vp, vp, i32p, i32p, vp]
     lib.s4c_embed_gather.restype = i
     lib.s4c_embed_gather.argtypes = [vp, i32p, i, i, i, vp, vp]
     lib.s4c_launch_floor.restype = i
@@ -519,6 +521,34 @@ def tree_build_topk(topk, branching, root_token, cache_len=None, tokens=None, pa
     if rc:
         raise S4CError("s4c_tree_build_topk", rc)
     return dict(tokens=tokens, parent=parent, position=position, n_nodes=n_nodes)
+
+
+def draft_level(choice, branching, levels, topk_all, tree, root_token, root_position=None, embedding=None, features=None,
+                e_out=None, f_out=None, tok_out=None, pos_out=None, stream=None):
+    """s4c_draft_level: ranked choices [B * n, k] of the nodes levels[0] = (first, past the last) into topk_all [B,T,k] and the
+    tree's arrays, and the next head's inputs for the nodes levels[1], their children (None: no next head)."""
+    B, T, k = topk_all.shape
+    br = (ctypes.c_int32 * max(1, len(branching)))(*[int(x) for x in branching])
+    (s, e), (ns, ne) = levels[0], levels[1] or (0, 0)
+    if choice.numel() != B * (e - s) * k:
+        raise ValueError("choice must be [B * nodes of the level, k]")
+    rows = B * (ne - ns)
+    if rows:
+        H = embedding.shape[1]
+        if features.shape != (B * (e - s), H) or e_out.shape != (rows, H) or f_out.shape != (rows, H):
+            raise ValueError("features must be [B * nodes of the level, H], e_out and f_out [B * nodes of the next, H]")
+        if tok_out.numel() != rows or pos_out.numel() != rows:
+            raise ValueError("tok_out and pos_out need an entry per node of the next level")
+    bf, i32 = torch.bfloat16, torch.int32
+    rc = _lib.s4c_draft_level(
+        _dev(choice, i32, "choice"), k, ctypes.cast(br, ctypes.c_void_p), len(branching), s, e - s, ns, ne - ns,
+        _dev(root_token, i32, "root_token"), _dev(root_position, i32, "root_position"), B, T, _dev(topk_all, i32, "topk_all"),
+        _dev(tree["tokens"], i32, "tokens"), _dev(tree["parent"], i32, "parent"), _dev(tree["position"], i32, "position"),
+        _dev(tree["n_nodes"], i32, "n_nodes"), _dev(embedding, bf, "embedding"), embedding.shape[0] if rows else 0,
+        _dev(features, bf, "features"), embedding.shape[1] if rows else 0, _dev(e_out, bf, "e_out"), _dev(f_out, bf, "f_out"),
+        _dev(tok_out, i32, "tok_out"), _dev(pos_out, i32, "pos_out"), _stream(stream))
+    if rc:
+        raise S4CError("s4c_draft_level", rc)
 
 
 def linear_workspace_bytes(R, K1, K2, N, gate: bool = False) -> int:
