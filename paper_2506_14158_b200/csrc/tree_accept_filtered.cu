@@ -645,7 +645,9 @@ struct SparseShared {
     double kp[kMaxTopK];     // their current target probabilities
     double kq0[kMaxTopK];    // their draft probabilities as given
     int kgone[kMaxTopK];     // 1: the token was rejected here and has left the draft distribution
-    int order[kMaxTopK];     // the kept tokens' list positions in token order (the order the vocabulary is scanned in)
+    int vtok[kMaxTopK];      // the kept tokens in token order (the order the vocabulary is scanned in)
+    double vp[kMaxTopK];     // ... and their probabilities
+    uint32_t kids[S4C_MAX_T][S4C_MASK_WORDS];  // node i's children
     int flag;
 };
 
@@ -664,6 +666,7 @@ accept_walk_sparse_kernel(const float* __restrict__ dprobs, const int32_t* __res
         sh.uni[i] = uniforms[(size_t)b * T + i];
         if (near_tie) near_tie[(size_t)b * T + i] = 0;
     }
+    for (int i = tid; i < S4C_MAX_T * S4C_MASK_WORDS; i += blockDim.x) sh.kids[i / S4C_MASK_WORDS][i % S4C_MASK_WORDS] = 0u;
     __syncthreads();
     int flags = build_ancestor_masks(sh.par, n, T, sh.anc, sh.depth, &sh.flag);
     if (!flags) {
@@ -675,8 +678,10 @@ accept_walk_sparse_kernel(const float* __restrict__ dprobs, const int32_t* __res
         flags = sh.flag;
     }
     if (!flags)  // (tokens are in range) -- these reads of the caller's inputs need not wait for the lists either
-        for (int i = 1 + tid; i < n; i += blockDim.x)
+        for (int i = 1 + tid; i < n; i += blockDim.x) {
             sh.tq0[i] = (double)__ldg(dprobs + ((size_t)b * T + sh.par[i]) * V + sh.tok[i]);
+            atomicOr(&sh.kids[sh.par[i]][i >> 5], 1u << (i & 31));
+        }
     griddep_wait();  // the kept lists are complete
     if (!flags) {
         for (int i = tid; i < n; i += blockDim.x)
@@ -702,8 +707,15 @@ accept_walk_sparse_kernel(const float* __restrict__ dprobs, const int32_t* __res
             sh.ktok[j] = kept.tok[at * k + j], sh.kp[j] = kept.p[at * k + j], sh.kq0[j] = (double)kept.q0[at * k + j], sh.kgone[j] = 0;
         __syncwarp();
         int accepted = -1;
-        for (int c = cur + 1; c < n; ++c) {
-            if (sh.par[c] != cur) continue;
+        // the children from bitmasks, the draw by a prefix sum over the lanes: as loops over the nodes and over the kept tokens
+        // these cost a step with a 60-node tree and 50 kept tokens 6 us more (603 -> 597 us)
+        int kw = 0;
+        uint32_t kbits = sh.kids[cur][0];
+        for (;;) {
+            while (kbits == 0u && kw < S4C_MASK_WORDS - 1) kbits = sh.kids[cur][++kw];
+            if (kbits == 0u) break;
+            const int c = 32 * kw + __ffs(kbits) - 1;
+            kbits &= kbits - 1u;
             const int x = sh.tok[c];
             // position of token x among the kept ones, or -1
             const uint32_t h0 = __ballot_sync(0xffffffffu, lane < m && sh.ktok[lane] == x);
@@ -754,25 +766,24 @@ accept_walk_sparse_kernel(const float* __restrict__ dprobs, const int32_t* __res
         for (int j = lane; j < m; j += 32) {
             int pos = 0;
             for (int i = 0; i < m; ++i) pos += sh.ktok[i] < sh.ktok[j] ? 1 : 0;
-            sh.order[pos] = j;
+            sh.vtok[pos] = sh.ktok[j], sh.vp[pos] = sh.kp[j];
         }
         __syncwarp();
+        const double p0 = 2 * lane < m ? sh.vp[2 * lane] : 0.0, p1 = 2 * lane + 1 < m ? sh.vp[2 * lane + 1] : 0.0;
+        double in = p0 + p1;  // mass up to and with this lane's two
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(0xffffffffu, in, o);
+            if (lane >= o) in += t;
+        }
+        const double ex = __shfl_up_sync(0xffffffffu, in, 1), target = (double)sh.uni[0] * __shfl_sync(0xffffffffu, in, 31);
+        const bool hit0 = p0 > 0.0 && (lane ? ex + p0 : p0) > target, hit1 = p1 > 0.0 && in > target;
+        const uint32_t hits = __ballot_sync(0xffffffffu, hit0 || hit1), some = __ballot_sync(0xffffffffu, p0 > 0.0 || p1 > 0.0);
+        // the first entry that crosses, or the last one with mass (the target rounded up to the total), or the first of all
+        const int from = hits ? __ffs(hits) - 1 : (some ? 31 - __clz(some) : 0);
+        const int at2 = __shfl_sync(0xffffffffu, hits ? 2 * lane + (hit0 ? 0 : 1) : (some ? 2 * lane + (p1 > 0.0 ? 1 : 0) : 0), from);
         if (lane == 0) {
-            double tot = 0.0;
-            for (int i = 0; i < m; ++i) tot += sh.kp[sh.order[i]];
-            const double target = (double)sh.uni[0] * tot;
-            double run = 0.0;
-            int pick = -1, last = sh.ktok[sh.order[0]];
-            for (int i = 0; i < m; ++i) {
-                const int j = sh.order[i];
-                if (sh.kp[j] > 0.0) last = sh.ktok[j];
-                run += sh.kp[j];
-                if (run > target) {
-                    pick = sh.ktok[j];
-                    break;
-                }
-            }
-            next_token[b] = pick >= 0 ? pick : last;
+            next_token[b] = sh.vtok[at2];
             for (int j = 0; j <= max_depth; ++j) pth[j] = -1;
             for (int t = cur; t >= 0; t = sh.par[t]) pth[sh.depth[t]] = t;
             accept_len[b] = sh.depth[cur];
