@@ -657,6 +657,7 @@ accept_walk_sparse_kernel(const float* __restrict__ dprobs, const int32_t* __res
                           int max_depth, KeptLists kept, int32_t* __restrict__ accept_len, int32_t* __restrict__ path,
                           int32_t* __restrict__ next_token, uint8_t* __restrict__ near_tie, int32_t* __restrict__ status) {
     __shared__ SparseShared sh;
+    griddep_launch_dependents();  // (what follows sets itself up beside this and waits for its end)
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int n = n_nodes ? n_nodes[b] : T;
     int32_t* pth = path + (size_t)b * (max_depth + 1);
