@@ -288,11 +288,9 @@ struct WalkShared {
     int cx[S4C_MAX_T];
     double cinvZ[S4C_MAX_T];  // 1/Z_j, or 0 when Z_j == 0 (p kept)
     double cinvs[S4C_MAX_T];  // 1/s_j
-    double scratch[33];
     double wsum[32];  // per warp of a 1024-thread CTA
     int wlast[32];
     int flag;
-    int result_tok;
 };
 
 // p and q of vocabulary entry v after r rejections at the current node.
