@@ -1,12 +1,13 @@
 // Native marshalling for the calls a program makes eagerly, once per layer or step: the attention, acceptance, compaction and
-// LM-head entry points.  Checks and pointers are the same as in s4c.py's ctypes calls; what differs is the price of a call -- a
-// dozen attribute look-ups, conversions and allocations through the interpreter took 12 us of host time around a kernel of
+// LM-head entry points.  What is accepted, and what is raised for the rest, is the same as with s4c.py's ctypes calls; what differs
+// is the price of a call -- a dozen attribute look-ups, conversions and allocations through the interpreter took 12 us of host time around a kernel of
 // 8 us.  Everything else stays with ctypes.
 #include <Python.h>
 
 #include <ATen/ops/empty.h>
 #include <ATen/ops/empty_like.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "s4c.h"
@@ -46,15 +47,32 @@ T* i32(PyObject* o, const char* name) {
 }
 float* f32(PyObject* o, const char* name) { return static_cast<float*>(ptr(o, at::kFloat, name)); }
 
-long integer(PyObject* o) {
+int integer(PyObject* o) {  // an int or what stands for one (`__index__`); a float is refused
     const long v = PyLong_AsLong(o);
     if (v == -1 && PyErr_Occurred()) throw BadArgument();
-    return v;
+    return (int)v;
 }
-double real(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw BadArgument();
-    return v;
+int to_integer(PyObject* o) {  // int(o)
+    if (PyLong_Check(o)) return integer(o);
+    PyObject* i = PyNumber_Long(o);
+    if (!i) throw BadArgument();
+    const long v = PyLong_AsLong(i);
+    Py_DECREF(i);
+    if (v == -1 && PyErr_Occurred()) throw BadArgument();
+    return (int)v;
+}
+float to_real(PyObject* o) {  // float(o)
+    if (PyFloat_Check(o)) return (float)PyFloat_AS_DOUBLE(o);
+    PyObject* f = PyNumber_Float(o);
+    if (!f) throw BadArgument();
+    const double v = PyFloat_AsDouble(f);
+    Py_DECREF(f);
+    return (float)v;
+}
+bool truth(PyObject* o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw BadArgument();
+    return v == 1;
 }
 void* stream_of(PyObject* o) {  // None: the current stream; else an object with `cuda_stream`
     if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
@@ -89,17 +107,19 @@ PyObject* answer(int rc, PyObject* result) {
     PyTuple_SET_ITEM(t, 1, result);
     return t;
 }
+// Exceptions leave as the Python exceptions that torch's own functions raise for them (out of memory, index, type ...).
 template <typename F>
 PyObject* guarded(F f) {
+    HANDLE_TH_ERRORS
     try {
         return f();
     } catch (const BadArgument&) {
         return nullptr;
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
     }
+    END_HANDLE_TH_ERRORS
 }
+// The arguments are taken one by one in the order of the call (the order in which a compiler evaluates the arguments of a C++ call
+// is its own): of several wrong ones the first is named, and no CUDA call is made before all of them have passed.
 
 // attention(q, k_cache, v_cache, cache_len, parent, n_nodes, out, scale, status, workspace, stream, max_cache_len, rows, scratch_fn)
 // -> (rc, out); scratch_fn(nbytes, device) gives a workspace where one is needed and none was passed
@@ -116,7 +136,7 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
             throw BadArgument();
         }
         const int B = (int)q.size(0), Hq = (int)q.size(1), T = (int)q.size(2), d = (int)q.size(3), Hkv = (int)k.size(1), C = (int)k.size(2);
-        const bool rows = PyObject_IsTrue(a[12]) == 1;
+        const bool rows = truth(a[12]);
         const s4c_dtype dt = dtype_of(q);
         PyObject* out = a[6];
         if (out == Py_None)
@@ -130,11 +150,16 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
                 ws = PyObject_CallFunction(a[13], "nO", (Py_ssize_t)need, a[0]);
                 if (!ws) throw BadArgument();
             }
+            const void *qp = ptr(q, kAny, "q"), *kp = ptr(k, kAny, "k_cache"), *vp = ptr(v, kAny, "v_cache");
+            const int32_t *len = i32(a[3], "cache_len"), *parent = i32(a[4], "parent"), *n_nodes = i32(a[5], "n_nodes");
+            void* op = ptr(out, q.scalar_type(), "out");
+            const int max_len = to_integer(a[11]);
+            const float scale = to_real(a[7]);
+            int32_t* status = i32(a[8], "status");
             const Scratch scratch(ws ? ws : a[9]);
-            const int rc = (rows ? s4c_tree_attention_rows : s4c_tree_attention)(
-                ptr(q, kAny, "q"), ptr(k, kAny, "k_cache"), ptr(v, kAny, "v_cache"), i32(a[3], "cache_len"), i32(a[4], "parent"),
-                i32(a[5], "n_nodes"), ptr(out, q.scalar_type(), "out"), B, T, Hq, Hkv, d, C, (int)integer(a[11]), dt, (float)real(a[7]),
-                i32(a[8], "status"), scratch.p, scratch.bytes, stream_of(a[10]));
+            void* stream = stream_of(a[10]);
+            const int rc = (rows ? s4c_tree_attention_rows : s4c_tree_attention)(qp, kp, vp, len, parent, n_nodes, op, B, T, Hq, Hkv, d, C, max_len,
+                                                                                 dt, scale, status, scratch.p, scratch.bytes, stream);
             Py_XDECREF(ws);
             return answer(rc, out);
         } catch (...) {
@@ -150,13 +175,20 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* accept(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         count(n, 15);
-        const at::Tensor& logits = tensor(a[0], "target_logits");
+        const at::Tensor& t = tensor(a[0], "target_logits");
+        const float *logits = static_cast<const float*>(ptr(t, at::kFloat, "target_logits")), *probs = f32(a[1], "draft_probs");
+        const int32_t *tokens = i32(a[2], "tokens"), *parent = i32(a[3], "parent"), *n_nodes = i32(a[6], "n_nodes");
+        const float temperature = to_real(a[4]);
+        const float* uniforms = f32(a[5], "uniforms");
+        const int max_depth = to_integer(a[7]);
+        int32_t *accept_len = i32(a[8], "accept_len"), *path = i32(a[9], "path"), *next_token = i32(a[10], "next_token");
+        uint8_t* near_tie = static_cast<uint8_t*>(ptr(a[11], at::kByte, "near_tie"));
+        int32_t* status = i32(a[12], "status");
         const Scratch scratch(a[13]);
-        return PyLong_FromLong(s4c_tree_accept(
-            static_cast<const float*>(ptr(logits, at::kFloat, "target_logits")), f32(a[1], "draft_probs"), i32(a[2], "tokens"), i32(a[3], "parent"),
-            i32(a[6], "n_nodes"), (float)real(a[4]), f32(a[5], "uniforms"), (int)logits.size(0), (int)logits.size(1), (int)logits.size(2),
-            (int)integer(a[7]), i32(a[8], "accept_len"), i32(a[9], "path"), i32(a[10], "next_token"),
-            static_cast<uint8_t*>(ptr(a[11], at::kByte, "near_tie")), i32(a[12], "status"), scratch.p, scratch.bytes, stream_of(a[14])));
+        void* stream = stream_of(a[14]);
+        const int rc = s4c_tree_accept(logits, probs, tokens, parent, n_nodes, temperature, uniforms, (int)t.size(0), (int)t.size(1),
+                                       (int)t.size(2), max_depth, accept_len, path, next_token, near_tie, status, scratch.p, scratch.bytes, stream);
+        return PyLong_FromLong(rc);
     });
 }
 
@@ -164,14 +196,20 @@ PyObject* accept(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* compact(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         count(n, 17);
-        const int layers = (int)integer(a[2]);
-        const at::Tensor& path = tensor(a[9], "path");
-        return PyLong_FromLong(s4c_kv_compact(
-            layers ? static_cast<void* const*>(ptr(a[0], at::kLong, "k_ptrs")) : nullptr,
-            layers ? static_cast<void* const*>(ptr(a[1], at::kLong, "v_ptrs")) : nullptr, layers, i32(a[8], "cache_len"),
-            static_cast<const int32_t*>(ptr(path, at::kInt, "path")), i32(a[10], "accept_len"), (int)path.size(1) - 1, ptr(a[12], kAny, "feat_in"),
-            ptr(a[13], kAny, "feat_out"), (int)integer(a[3]), (int)integer(a[11]), (int)integer(a[4]), (int)integer(a[6]), (int)integer(a[5]),
-            (int)integer(a[14]), integer(a[7]) ? S4C_F32 : S4C_BF16, i32(a[15], "status"), stream_of(a[16])));
+        const at::Tensor& p = tensor(a[9], "path");
+        const int max_depth = (int)p.size(1) - 1, layers = to_integer(a[2]);
+        void* const* k_ptrs = layers ? static_cast<void* const*>(ptr(a[0], at::kLong, "k_ptrs")) : nullptr;
+        void* const* v_ptrs = layers ? static_cast<void* const*>(ptr(a[1], at::kLong, "v_ptrs")) : nullptr;
+        int32_t* len = i32(a[8], "cache_len");
+        const int32_t *path = static_cast<const int32_t*>(ptr(p, at::kInt, "path")), *accept_len = i32(a[10], "accept_len");
+        const void* feat_in = ptr(a[12], kAny, "feat_in");
+        void* feat_out = ptr(a[13], kAny, "feat_out");
+        const int B = integer(a[3]), T = integer(a[11]), Hkv = integer(a[4]), d = integer(a[6]), C = integer(a[5]), hid = integer(a[14]);
+        const s4c_dtype dt = truth(a[7]) ? S4C_F32 : S4C_BF16;
+        int32_t* status = i32(a[15], "status");
+        void* stream = stream_of(a[16]);
+        const int rc = s4c_kv_compact(k_ptrs, v_ptrs, layers, len, path, accept_len, max_depth, feat_in, feat_out, B, T, Hkv, d, C, hid, dt, status, stream);
+        return PyLong_FromLong(rc);
     });
 }
 
@@ -185,7 +223,7 @@ PyObject* lm_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
             PyErr_SetString(PyExc_ValueError, "hidden must be [R,H] and weight [V,H]");
             throw BadArgument();
         }
-        const int R = (int)h.size(0), H = (int)h.size(1), V = (int)w.size(0), k = (int)integer(a[2]);
+        const int R = (int)h.size(0), H = (int)h.size(1), V = (int)w.size(0), k = integer(a[2]);
         PyObject* made[3] = {};
         PyObject* ws = nullptr;
         try {
@@ -201,9 +239,13 @@ PyObject* lm_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
                 ws = PyObject_CallFunction(a[8], "nO", (Py_ssize_t)s4c_lm_head_topk_workspace_bytes(R, V, H, k ? k : 1), a[0]);
                 if (!ws) throw BadArgument();
             }
+            const void *hidden = ptr(h, at::kBFloat16, "hidden"), *weight = ptr(w, at::kBFloat16, "weight");
+            int32_t* token = i32(made[0], "token");
+            float* logit = f32(made[1], k ? "logit" : "max_logit");
+            int32_t* status = i32(made[2], "status");
             const Scratch scratch(ws ? ws : a[6]);
-            const int rc = s4c_lm_head_topk(ptr(h, at::kBFloat16, "hidden"), ptr(w, at::kBFloat16, "weight"), R, V, H, k ? k : 1, i32(made[0], "token"),
-                                            f32(made[1], k ? "logit" : "max_logit"), i32(made[2], "status"), scratch.p, scratch.bytes, stream_of(a[7]));
+            void* stream = stream_of(a[7]);
+            const int rc = s4c_lm_head_topk(hidden, weight, R, V, H, k ? k : 1, token, logit, status, scratch.p, scratch.bytes, stream);
             Py_XDECREF(ws);
             PyObject* t = PyTuple_New(3);
             for (int i = 0; i < 3; ++i) PyTuple_SET_ITEM(t, i, made[i]);
@@ -226,7 +268,7 @@ PyObject* accept_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
             PyErr_SetString(PyExc_ValueError, "target_token must be [B,T]");
             throw BadArgument();
         }
-        const int B = (int)t.size(0), T = (int)t.size(1), max_depth = a[5] == Py_None ? T - 1 : (int)integer(a[5]);
+        const int B = (int)t.size(0), T = (int)t.size(1), max_depth = a[5] == Py_None ? T - 1 : to_integer(a[5]);
         PyObject* made[4] = {};
         try {
             for (int i = 0; i < 4; ++i) {
@@ -235,9 +277,13 @@ PyObject* accept_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
                 else
                     made[i] = THPVariable_Wrap(i == 1 ? at::empty({B, max_depth + 1}, t.options().dtype(at::kInt)) : at::empty({B}, t.options().dtype(at::kInt)));
             }
-            const int rc = s4c_tree_accept_tokens(static_cast<const int32_t*>(ptr(t, at::kInt, "target_token")), i32(a[1], "tokens"), i32(a[2], "parent"),
-                                                  i32(a[4], "n_nodes"), B, T, (int)integer(a[3]), max_depth, i32(made[0], "accept_len"),
-                                                  i32(made[1], "path"), i32(made[2], "next_token"), i32(made[3], "status"), stream_of(a[10]));
+            const int32_t* target = static_cast<const int32_t*>(ptr(t, at::kInt, "target_token"));
+            const int32_t *tokens = i32(a[1], "tokens"), *parent = i32(a[2], "parent"), *n_nodes = i32(a[4], "n_nodes");
+            const int V = to_integer(a[3]);
+            int32_t *accept_len = i32(made[0], "accept_len"), *path = i32(made[1], "path"), *next_token = i32(made[2], "next_token");
+            int32_t* status = i32(made[3], "status");
+            void* stream = stream_of(a[10]);
+            const int rc = s4c_tree_accept_tokens(target, tokens, parent, n_nodes, B, T, V, max_depth, accept_len, path, next_token, status, stream);
             PyObject* r = PyTuple_New(4);
             for (int i = 0; i < 4; ++i) PyTuple_SET_ITEM(r, i, made[i]);
             return answer(rc, r);

@@ -21,3 +21,23 @@ def test_binding_refuses_cpu_tensors_wrong_shapes_and_types(s4c_lib):
         s4c.tree_attention(q, kv, kv, i, par, workspace=i, stream=type("S", (), {"cuda_stream": 0})())
     with pytest.raises(ValueError):
         s4c.tree_accept_tokens(i, par, par, 100)
+
+
+def test_of_several_wrong_arguments_the_first_is_named(s4c_lib):
+    # the order of the call decides, not the compiler's order of evaluation, and no CUDA call is made for arguments that are refused
+    from paper_2506_14158_b200 import s4c
+
+    q, kv = torch.zeros(1, 4, 8, 64), torch.zeros(1, 2, 128, 64)
+    i, par = torch.zeros(1, dtype=torch.int32), torch.zeros(1, 8, dtype=torch.int32)
+    with pytest.raises(ValueError, match="^q must be a CUDA tensor"):
+        s4c.tree_attention(q, kv, kv, i, par, max_cache_len=128.0)
+    with pytest.raises(ValueError, match="^hidden must be a CUDA tensor"):
+        s4c.lm_head_greedy(torch.zeros(3, 64), torch.zeros(5, 64))
+    with pytest.raises(ValueError, match="^target_token must be a CUDA tensor"):
+        s4c.tree_accept_tokens(par, par, par, 100)
+    with pytest.raises(ValueError, match="^target_logits must be a CUDA tensor"):
+        s4c.tree_accept(torch.zeros(1, 8, 10), None, par, par, 0.0)
+    with pytest.raises(RuntimeError, match="ambiguous"):  # what `rows` itself raises, not a SystemError
+        s4c.tree_attention(q, kv, kv, i, par, rows=torch.ones(2))
+    with pytest.raises(IndexError):
+        s4c.kv_compact(None, None, 0, (1, 2, 128, 64), torch.float32, i, i, i, 8, status=i)
