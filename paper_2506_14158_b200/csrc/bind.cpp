@@ -89,6 +89,17 @@ s4c_dtype dtype_of(const at::Tensor& t) {
     PyErr_Format(PyExc_TypeError, "unsupported dtype %s: the library takes float32 or bfloat16", c10::toString(t.scalar_type()));
     throw BadArgument();
 }
+// The interpreter lock is given up around allocations and the library's calls, as torch and ctypes do: a launch that finds the
+// stream's queue full waits there for as long as the GPU takes, and the program's other threads go on meanwhile.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <typename F>
+auto unlocked(F f) {
+    const Unlocked u;
+    return f();
+}
 struct Scratch {
     void* p;
     size_t bytes;
@@ -140,7 +151,7 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const s4c_dtype dt = dtype_of(q);
         PyObject* out = a[6];
         if (out == Py_None)
-            out = THPVariable_Wrap(rows ? at::empty({B, T, Hq, d}, q.options()) : at::empty_like(q));
+            out = THPVariable_Wrap(unlocked([&] { return rows ? at::empty({B, T, Hq, d}, q.options()) : at::empty_like(q); }));
         else
             Py_INCREF(out);
         PyObject* ws = nullptr;
@@ -158,8 +169,10 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
             int32_t* status = i32(a[8], "status");
             const Scratch scratch(ws ? ws : a[9]);
             void* stream = stream_of(a[10]);
-            const int rc = (rows ? s4c_tree_attention_rows : s4c_tree_attention)(qp, kp, vp, len, parent, n_nodes, op, B, T, Hq, Hkv, d, C, max_len,
-                                                                                 dt, scale, status, scratch.p, scratch.bytes, stream);
+            const int rc = unlocked([&] {
+                return (rows ? s4c_tree_attention_rows : s4c_tree_attention)(qp, kp, vp, len, parent, n_nodes, op, B, T, Hq, Hkv, d, C, max_len, dt,
+                                                                             scale, status, scratch.p, scratch.bytes, stream);
+            });
             Py_XDECREF(ws);
             return answer(rc, out);
         } catch (...) {
@@ -186,8 +199,11 @@ PyObject* accept(PyObject*, PyObject* const* a, Py_ssize_t n) {
         int32_t* status = i32(a[12], "status");
         const Scratch scratch(a[13]);
         void* stream = stream_of(a[14]);
-        const int rc = s4c_tree_accept(logits, probs, tokens, parent, n_nodes, temperature, uniforms, (int)t.size(0), (int)t.size(1),
-                                       (int)t.size(2), max_depth, accept_len, path, next_token, near_tie, status, scratch.p, scratch.bytes, stream);
+        const int B = (int)t.size(0), T = (int)t.size(1), V = (int)t.size(2);
+        const int rc = unlocked([&] {
+            return s4c_tree_accept(logits, probs, tokens, parent, n_nodes, temperature, uniforms, B, T, V, max_depth, accept_len, path, next_token,
+                                   near_tie, status, scratch.p, scratch.bytes, stream);
+        });
         return PyLong_FromLong(rc);
     });
 }
@@ -208,7 +224,9 @@ PyObject* compact(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const s4c_dtype dt = truth(a[7]) ? S4C_F32 : S4C_BF16;
         int32_t* status = i32(a[15], "status");
         void* stream = stream_of(a[16]);
-        const int rc = s4c_kv_compact(k_ptrs, v_ptrs, layers, len, path, accept_len, max_depth, feat_in, feat_out, B, T, Hkv, d, C, hid, dt, status, stream);
+        const int rc = unlocked([&] {
+            return s4c_kv_compact(k_ptrs, v_ptrs, layers, len, path, accept_len, max_depth, feat_in, feat_out, B, T, Hkv, d, C, hid, dt, status, stream);
+        });
         return PyLong_FromLong(rc);
     });
 }
@@ -233,7 +251,7 @@ PyObject* lm_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
                     continue;
                 }
                 const auto opt = h.options().dtype(i == 1 ? at::kFloat : at::kInt);
-                made[i] = THPVariable_Wrap(i == 2 ? at::empty({1}, opt) : k ? at::empty({R, k}, opt) : at::empty({R}, opt));
+                made[i] = THPVariable_Wrap(unlocked([&] { return i == 2 ? at::empty({1}, opt) : k ? at::empty({R, k}, opt) : at::empty({R}, opt); }));
             }
             if (a[6] == Py_None) {
                 ws = PyObject_CallFunction(a[8], "nO", (Py_ssize_t)s4c_lm_head_topk_workspace_bytes(R, V, H, k ? k : 1), a[0]);
@@ -245,7 +263,8 @@ PyObject* lm_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
             int32_t* status = i32(made[2], "status");
             const Scratch scratch(ws ? ws : a[6]);
             void* stream = stream_of(a[7]);
-            const int rc = s4c_lm_head_topk(hidden, weight, R, V, H, k ? k : 1, token, logit, status, scratch.p, scratch.bytes, stream);
+            const int rc = unlocked(
+                [&] { return s4c_lm_head_topk(hidden, weight, R, V, H, k ? k : 1, token, logit, status, scratch.p, scratch.bytes, stream); });
             Py_XDECREF(ws);
             PyObject* t = PyTuple_New(3);
             for (int i = 0; i < 3; ++i) PyTuple_SET_ITEM(t, i, made[i]);
@@ -275,7 +294,10 @@ PyObject* accept_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
                 if (a[6 + i] != Py_None)
                     Py_INCREF(made[i] = a[6 + i]);
                 else
-                    made[i] = THPVariable_Wrap(i == 1 ? at::empty({B, max_depth + 1}, t.options().dtype(at::kInt)) : at::empty({B}, t.options().dtype(at::kInt)));
+                    made[i] = THPVariable_Wrap(unlocked([&] {
+                        const auto opt = t.options().dtype(at::kInt);
+                        return i == 1 ? at::empty({B, max_depth + 1}, opt) : at::empty({B}, opt);
+                    }));
             }
             const int32_t* target = static_cast<const int32_t*>(ptr(t, at::kInt, "target_token"));
             const int32_t *tokens = i32(a[1], "tokens"), *parent = i32(a[2], "parent"), *n_nodes = i32(a[4], "n_nodes");
@@ -283,7 +305,9 @@ PyObject* accept_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
             int32_t *accept_len = i32(made[0], "accept_len"), *path = i32(made[1], "path"), *next_token = i32(made[2], "next_token");
             int32_t* status = i32(made[3], "status");
             void* stream = stream_of(a[10]);
-            const int rc = s4c_tree_accept_tokens(target, tokens, parent, n_nodes, B, T, V, max_depth, accept_len, path, next_token, status, stream);
+            const int rc = unlocked([&] {
+                return s4c_tree_accept_tokens(target, tokens, parent, n_nodes, B, T, V, max_depth, accept_len, path, next_token, status, stream);
+            });
             PyObject* r = PyTuple_New(4);
             for (int i = 0; i < 4; ++i) PyTuple_SET_ITEM(r, i, made[i]);
             return answer(rc, r);
