@@ -1,5 +1,5 @@
 """Binding of ``libs4c.so`` -- argument marshalling only; every step runs in the library's CUDA kernels.  The calls a program
-makes eagerly per layer or step go through ``_bind.so`` (native marshalling), the others through ctypes.
+makes eagerly per layer or step go through native marshalling (``csrc/bind.cpp``), the others through ctypes.
 
 The functions mirror the C ABI declared in ``include/s4c.h`` (same names, same argument meaning).  Tensors are
 torch CUDA tensors used purely as device buffers: the binding checks dtype / contiguity / device, passes raw
@@ -9,12 +9,13 @@ CPU fallback: importing this module fails if the library has not been built, and
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Sequence
 
 import torch
 
-from ._build import lib_path
+from ._build import bind_path, lib_path
 
 F32, BF16 = 0, 1
 SEQ_OK, SEQ_BAD_PARENT, SEQ_TOKEN_RANGE, SEQ_CAPACITY, SEQ_DEPTH, SEQ_BAD_PATH, SEQ_TIMEOUT, SEQ_NONFINITE = 0, 1, 2, 4, 8, 16, 32, 64
@@ -106,10 +107,20 @@ def _load() -> ctypes.CDLL:
 
 _lib = None
 _lib = _load()
-try:
-    from . import _bind
-except ImportError as e:
-    raise ImportError(f"_bind.so is missing or does not load ({e}): build it with `python -c 'import __graft_entry__ as g; g.build()'`") from e
+
+
+def _load_bind():
+    path = bind_path()
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing (its name holds the torch and Python it is built for): build it with "
+                          "`python -c 'import __graft_entry__ as g; g.build()'`")
+    spec = importlib.util.spec_from_file_location(__package__ + "._bind", path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
+
+
+_bind = _load_bind()
 
 
 def version() -> int:

@@ -41,3 +41,29 @@ def test_of_several_wrong_arguments_the_first_is_named(s4c_lib):
         s4c.tree_attention(q, kv, kv, i, par, rows=torch.ones(2))
     with pytest.raises(IndexError):
         s4c.kv_compact(None, None, 0, (1, 2, 128, 64), torch.float32, i, i, i, 8, status=i)
+
+
+def test_a_binary_of_another_torch_is_neither_kept_nor_loaded(s4c_lib, monkeypatch, tmp_path):
+    import os
+    import subprocess
+    import sys
+
+    from paper_2506_14158_b200 import _build
+
+    ran = []
+
+    def compiler(cmd, check):
+        ran.append(cmd)
+        open(cmd[cmd.index("-o") + 1], "w").close()
+
+    monkeypatch.setattr(_build, "_HERE", str(tmp_path))
+    monkeypatch.setattr(_build.subprocess, "run", compiler)
+    build = lambda: (ran.clear(), _build._build_bind(), len(ran))[-1]
+    assert build() == 1 and build() == 0
+    monkeypatch.setattr(torch, "__version__", "0.0.0")  # the sources are older than the binary all the same
+    assert build() == 1 and build() == 0
+    monkeypatch.undo()
+    assert os.path.exists(_build.bind_path())
+    code = "import torch; torch.__version__ = '0.0.0'; import paper_2506_14158_b200.s4c"
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=os.path.dirname(_build._HERE))
+    assert r.returncode != 0 and "ImportError" in r.stderr and "0_0_0" in r.stderr
