@@ -149,7 +149,10 @@ tree_attention_simt_kernel(const T_* __restrict__ q, const T_* __restrict__ kc, 
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
                 mn = fmaxf(mn, m);
-                if (mn > -INFINITY) {  // (a tile of other branches' slots only leaves the row as it is)
+                const uint32_t visible = __ballot_sync(0xffffffffu, seen);
+                // (a tile of other branches' slots only leaves the row as it is; one whose visible scores are all NaN, which the
+                // maximum passes over, does not)
+                if (mn > -INFINITY || __any_sync(0xffffffffu, s != s)) {
                     const float corr = exp2f(m - mn);  // m = -inf on the first visible slot: corr = 0
                     const float p = exp2f(s - mn);
                     float sum = p;
@@ -159,11 +162,17 @@ tree_attention_simt_kernel(const T_* __restrict__ q, const T_* __restrict__ kc, 
                     m = mn;
 #pragma unroll
                     for (int c = 0; c < DPL; ++c) acc[c] *= corr;
-#pragma unroll 8
-                    for (int jj = 0; jj < kSimtTile; ++jj) {
+                    auto add = [&](int jj) {
                         const float pj = __shfl_sync(0xffffffffu, p, jj);
 #pragma unroll
                         for (int c = 0; c < DPL; ++c) acc[c] = fmaf(pj, vs[jj][lane * DPL + c], acc[c]);
+                    };
+                    // Slots the row does not see are left out, not multiplied by zero: another branch's values may be Inf or NaN.
+                    if (visible == 0xffffffffu) {
+#pragma unroll 8
+                        for (int jj = 0; jj < kSimtTile; ++jj) add(jj);
+                    } else {
+                        for (uint32_t left = visible; left; left &= left - 1u) add(__ffs(left) - 1);
                     }
                 }
             }
