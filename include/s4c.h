@@ -385,7 +385,8 @@ s4c_status s4c_qkv_rope_at(const void* x, const void* w_qkv, const int32_t* cach
  * one tree): the tree checks, the rows' cache positions and the rotary table depend on cache_len,
  * parent, n_nodes, T, d and rope_theta alone, so the layers after the first reuse what s4c_qkv_rope
  * left in `workspace` (same B, T, d, C; cache_len unchanged since; the workspace untouched since)
- * and skip that kernel.  Arguments as s4c_qkv_rope.  status [B] or NULL is NOT rewritten: it keeps
+ * and skip that kernel.  w_qkv must not be the output of the call or kernel directly in front (as w of
+ * s4c_linear).  Arguments as s4c_qkv_rope.  status [B] or NULL is NOT rewritten: it keeps
  * what it holds (the first call's flags, when the same array is passed) and gets S4C_SEQ_TIMEOUT
  * OR-ed in; sequences the first call flagged are skipped here too. */
 s4c_status s4c_qkv_rope_same_tree(const void* x, const void* w_qkv, void* q_out, void* k_cache, void* v_cache, int B,
@@ -410,10 +411,10 @@ s4c_status s4c_qkv_rope_same_tree(const void* x, const void* w_qkv, void* q_out,
  *                   timing): workspace must hold s4c_linear_workspace_bytes(R, K1, K2, N, gate)
  *                   bytes (0 for shapes that need none; then NULL is accepted), 256-byte aligned;
  *                   S4C_ERR_WORKSPACE otherwise.  Stream order: the kernels are launched programmatically
- *                   dependent; inputs, bias, residual and outputs are touched only after the kernel
- *                   in front has completed, but tiles of w are requested earlier -- w must not be
- *                   the output of the kernel enqueued directly in front on the same stream (a
- *                   weight written earlier than that, or by a copy, is fine).
+ *                   dependent; inputs, bias, residual, norm weights and outputs are touched only after
+ *                   what is in front has completed, but tiles of w are requested earlier -- w must
+ *                   not be the output of the call or kernel enqueued directly in front on the same
+ *                   stream (a weight written by the one before that, or by a copy, is fine).
  *   s4c_linear_rmsnorm  the ungated s4c_linear followed by norm_out[r, :] = rmsnorm(out[r, :]) with
  *                   norm_weight [N] and eps >= 0 (norm_out [R, N] bf16, 16-byte aligned): the decoder
  *                   layer's "projection + residual, then the next block's normalisation".  Both out

@@ -94,8 +94,8 @@ kv_compact_rows_kernel(void* const* __restrict__ k_caches, void* const* __restri
     __shared__ PathInfo info;
     __shared__ int32_t spath[S4C_MAX_T];
     __shared__ int pages[kMaxTreeBlocks];
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();
     if (threadIdx.x < 32) {
         PathInfo r = check_path(cache_len, path, accept_len, b, max_depth, T, C, spath);
         if (threadIdx.x == 0) {

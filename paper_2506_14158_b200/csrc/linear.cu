@@ -92,7 +92,6 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_cta = (uint32_t)*tmem_slot;
     const uint32_t tmem = tmem_cta;
-    griddep_launch_dependents();  // the kernel behind may set itself up; it waits for this one's results on its own
 
     // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: what such
     // a thread computes per slice is time the stream waits, so the two operands have a producer each.
@@ -122,6 +121,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
         // ================= input producer =================
         if (elect_one()) {
             griddep_wait();
+            griddep_launch_dependents();  // (after the wait: see ln_launch)
             int s = 0, ks = k_first, fill = 0;
             uint32_t ph = 0, at = base;
             const int row = mtile * kLnBM * prm.nm, k1 = prm.k1_steps;
@@ -335,9 +335,11 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
                      const __nv_bfloat16* __restrict__ norm_weight, float norm_eps, __nv_bfloat16* __restrict__ norm_out,
                      float* __restrict__ out_f32) {
     __shared__ float red[kRowThreads / 32];
-    griddep_launch_dependents();  // (the next product sets itself up and requests weights meanwhile)
+    // The next product sets itself up and requests its weights meanwhile.  Ahead of the wait, for the product in front has triggered
+    // after its own: whatever came before this call has ended.
+    griddep_launch_dependents();
     const int r = blockIdx.x, first = threadIdx.x * 8;
-    uint4 g = make_uint4(0, 0, 0, 0);  // the norm weight, which no kernel in front writes, under way before the wait
+    uint4 g = make_uint4(0, 0, 0, 0);  // the norm weight, which the product in front does not write, under way before the wait
     if (norm_weight && first < N) g = __ldg(reinterpret_cast<const uint4*>(norm_weight + first));
     griddep_wait();
     const int w_rows = gate ? 2 * N : N;
@@ -417,8 +419,8 @@ rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restr
     __shared__ float red[kRowThreads / 32];
     const size_t row = blockIdx.x;
     const __nv_bfloat16* xr = x + row * H;
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();
     float ss = 0.f;
     for (int i = threadIdx.x * 8; i < H; i += blockDim.x * 8)  // H is a multiple of 8
         ss = sumsq8(ss, __ldg(reinterpret_cast<const uint4*>(xr + i)));
@@ -435,8 +437,8 @@ __global__ void __launch_bounds__(256)
 embed_gather_kernel(const __nv_bfloat16* __restrict__ table, const int32_t* __restrict__ tokens, int V, int H,
                     __nv_bfloat16* __restrict__ out) {
     const size_t row = blockIdx.x;
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();
     const int t = tokens[row];
     const bool ok = t >= 0 && t < V;
     for (int i = threadIdx.x * 8; i < H; i += blockDim.x * 8) {
@@ -449,6 +451,10 @@ embed_gather_kernel(const __nv_bfloat16* __restrict__ table, const int32_t* __re
 // ----------------------------------------------------------------------------- host side
 // A launch that may begin while the kernel in front of it on the stream is still running (programmatic dependent
 // launch): every kernel of this file waits (griddepcontrol.wait) before it reads what that kernel wrote or writes anything.
+// What follows may be launched (griddepcontrol.launch_dependents) only after the wait in the first kernel of a call: a kernel that
+// has started then knows that all calls but the one directly in front have ended, and may read ahead of its own wait what they
+// wrote -- a product its weights.  (Triggered before the wait, starts run through several calls: a weight written two calls
+// earlier could still be in the making.)
 template <typename... KArgs, typename... Args>
 static cudaError_t ln_launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     cudaLaunchAttribute pdl;

@@ -95,8 +95,8 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = (uint32_t)*tmem_slot;
-    griddep_launch_dependents();
     griddep_wait();  // the set-up above ran beside the kernel in front
+    griddep_launch_dependents();  // (after the wait, as in every call's first kernel: what follows may read ahead of its own)
     auto TM = [&](int buf, int t) { return tmem + (uint32_t)((buf * NM + t) * Cfg::kMaxBN); };
 
     // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: such a
@@ -360,8 +360,8 @@ accept_tokens_kernel(const int32_t* __restrict__ target_token, const int32_t* __
                      int32_t* __restrict__ accept_len, int32_t* __restrict__ path, int32_t* __restrict__ next_token,
                      int32_t* __restrict__ status) {
     __shared__ TokWalkShared sh;
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();
     const int b = blockIdx.x, tid = threadIdx.x;
     const int n = n_nodes ? n_nodes[b] : T;
     int32_t* pth = path + (size_t)b * (max_depth + 1);

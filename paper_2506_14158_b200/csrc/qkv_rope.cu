@@ -113,7 +113,6 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     tc_fence_after();
     const uint32_t tmem = (uint32_t)*tmem_slot;
 
-    griddep_launch_dependents();
     // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: what such
     // a thread computes per slice is time the stream waits, so the two operands have a producer each.
     // Every CTA walks the K slices from a start of its own: the CTAs of a row tile all read the same state tiles, and in step
@@ -121,7 +120,7 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int k_steps = prm.k_steps, k_first = (int)((blockIdx.x * 7u + blockIdx.y * 3u) % (uint32_t)k_steps);
     if (warp == 0 || warp == 6) {
         // ================= producers: weights (warp 0), states (warp 6) =================
-        // The weights, which no kernel of the step writes, fill the first ring while the kernel in front is still running;
+        // The weights, which the call in front does not write, fill the first ring while the kernel in front is still running;
         // the states follow once it has ended.
         if (elect_one()) {
             const bool states = warp == 6;
@@ -132,7 +131,12 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             const int tx = states ? x_bytes : stage_bytes - x_bytes, row = states ? mtile * kQkBM : head * d;
             const CUtensorMap* map = states ? &map_x : &map_w;
             const bool wait_x = prm.wait_x != 0;  // (else the table kernel is in front, and the states were there before it)
-            if (states && wait_x) griddep_wait();
+            if (states) {
+                if (wait_x) griddep_wait();
+                // (after the wait, or behind the table kernel, which is launched plainly: the calls before this one have ended, and a
+                // product behind may read its weights ahead of its own wait)
+                griddep_launch_dependents();
+            }
             for (; fill < k_steps; ++fill) {
                 if (fill == S && wait_x) griddep_wait();  // (a stage is freed only after its states have come: the bounded waits start here)
                 if (fill >= S && !mbar_wait(EMPTY(s), ph ^ 1, dead)) break;

@@ -242,8 +242,8 @@ draft_level_kernel(const int32_t* __restrict__ choice, int k, const __grid_const
                    int32_t* __restrict__ position, int32_t* __restrict__ n_nodes, const uint4* __restrict__ embedding, int V,
                    const uint4* __restrict__ features, int words, uint4* __restrict__ e_out, uint4* __restrict__ f_out,
                    int32_t* __restrict__ tok_out, int32_t* __restrict__ pos_out) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (after the wait: the product behind reads its weights ahead of its own)
     const int b = blockIdx.y, tid = threadIdx.x;
     const int base = root_position ? root_position[b] : 0;
     const int32_t* mine = choice + (size_t)b * from_count * k;
