@@ -122,7 +122,7 @@ class MultiHeadDrafter:
     A row's rotary position is root_position + depth (`position_base` of `s4c_qkv_rope_at`); its cache slot counts the
     head's own entries.
 
-    Only buffers, the static row maps and the order of the calls live here; the per-row work is `DrafterHead`'s chain of
+    Only buffers and the order of the calls live here; the per-row work is `DrafterHead`'s chain of
     library calls.
     """
 
@@ -165,8 +165,9 @@ class MultiHeadDrafter:
         Returns dict(tokens, parent, position, n_nodes) of the tree and the heads' features per level."""
         B, k = self.B, self.k
         choice = target_topk
-        if choice.dtype != torch.int32 or choice.shape != (B, k) or not choice.is_contiguous():
-            choice = torch.empty(B, k, dtype=torch.int32, device=self.topk_all.device).copy_(target_topk)
+        dev = self.topk_all.device
+        if choice.dtype != torch.int32 or choice.device != dev or choice.shape != (B, k) or not choice.is_contiguous():
+            choice = torch.empty(B, k, dtype=torch.int32, device=dev).copy_(target_topk)
         tree = self.tree
         feats_prev, level = f0, (0, 1)  # the root's feature is shared by all its candidates
         features = []

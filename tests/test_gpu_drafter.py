@@ -154,3 +154,21 @@ def test_three_heads_fill_the_tree_level_by_level():
                            c0[j][0], c0[j][1], r, position_base=pos, min_clear=0.0)
         np.testing.assert_array_equal(topk_all[:, s:e], head.token.cpu().numpy().reshape(B, nj, k))
         feats_prev, n_prev, s_prev = _f64(head.f_out), nj, s
+
+
+def test_the_candidates_of_a_round_may_come_in_any_form_that_can_be_copied():
+    from paper_2506_14158_b200 import drafter
+
+    B, T, V, Hq, Hkv, d, inter, C, k = 2, 7, 500, 2, 1, 64, 128, 24, 3
+    H = Hq * d
+    mh = drafter.MultiHeadDrafter([drafter.random_weights(V, H, Hq, Hkv, d, inter, "cuda", seed=3)], B, T, [3, 1], Hq, Hkv, d, C, k)
+    g = torch.Generator().manual_seed(4)
+    cand = torch.randint(0, V, (B, k), generator=g, dtype=torch.int32)
+    f0 = torch.randn(B, H, generator=g).to(torch.bfloat16).cuda()
+    kc, vc = (torch.randn(3 * B, Hkv, C, d, generator=g).to(torch.bfloat16).cuda() for _ in range(2))
+    i32 = lambda *x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    run = lambda c: {n: t.clone() for n, t in mh.draft(i32(1, 2), f0, c, i32(9, 5), [(kc, vc, i32(*[10] * 3 * B))]).items() if n != "features"}
+    want = run(cand.cuda())
+    for form in (cand, cand.long(), cand.cuda().long(), cand.t().contiguous().cuda().t()):  # host memory, other types, strides
+        got = run(form)
+        assert all(torch.equal(got[n], want[n]) for n in want)
