@@ -504,21 +504,23 @@ static bool ln_make_map(CUtensorMap* map, const void* ptr, uint64_t rows, int H,
 //   * per K slice of 64 elements a CTA needs the longest of: the issuing thread's fixed ~0.3 us (four tcgen05.mma, a
 //     commit, a wait -- whatever the tile's width, so narrow tiles move few bytes per issue); the tensor pipe's time for
 //     128 x bn x 64 products; its share of the weight stream from HBM (what one SM pulls, ~55 GB/s, or HBM divided
-//     among the CTAs of the wave; row tiles of one column tile share the weights through L2); the stage's bytes over
-//     what an SM takes in from L2 (~100 GB/s); and the ring's turn-round (a slot is refilled ~1.3 us after its
-//     products retire, so few deep stages starve the issuer);
+//     among the CTAs of the wave; row tiles of one column tile share the weights through L2 -- above 128 rows the next
+//     term is always the longer one); the stage's bytes over what an SM takes in from L2 (~100 GB/s); and the ring's
+//     turn-round (a slot is refilled ~1.3 us after its products retire, so few deep stages starve the issuer);
 //   * a shared-out K range writes and re-reads float32 partial sums and runs the finishing kernel.
-// The constants are measurements of this kernel on 7B- and 8B-shaped projections (26 and 256 rows), rounded; against
-// 70 measured (shape, columns, splits) points the model's choice was within 4 % of the best measured one.
+// The constants were fitted to 70 points of this kernel on 7B- and 8B-shaped projections (26 and 256 rows).  Against 2812
+// measured points -- eleven shapes from 2048 x 2560 to 13824 x 5120, plain and gated, 2 to 512 rows, the candidates that
+// the model holds for the best -- its choice takes 1.5 % longer than the best one on average up to 128 rows (12.7 % at worst:
+// 2048 x 2560 at 48 rows, 8.7 against 7.7 us; with 80 GB/s per SM 2.7 % on average), and 3.7 % above (24 % at worst:
+// 2048 x 2560 at 160 rows, 13.5 against 10.8 us; 13824 x 5120 at 256 rows 53.9 against 46.1 us: shares of 112 columns
+// and two row tiles are dearer in the model than on the GPU).
 struct LnPlan {
     int bn, splits, x_rows, stages, cols_per_tile, m_tiles, n_tiles, nm;
 };
 static LnPlan ln_plan(int R, int K1, int K2, int N, int gate) {
-    constexpr double kIssueUs = 0.30, kMmaUsPerCol = 0.27 / 256.0, kHbmBytesPerUs = 6.4e6, kL2BytesPerUs = 100e3,
+    constexpr double kIssueUs = 0.30, kMmaUsPerCol = 0.27 / 256.0, kSmBytesPerUs = 55e3, kHbmBytesPerUs = 6.4e6, kL2BytesPerUs = 100e3,
                      kTurnUs = 1.3, kWaveUs = 2.5, kFinishUs = 3.0, kPartialBytesPerUs = 4.0e6, kIssueTwo = 1.5;
     constexpr int kSms = 148;
-    // (what one SM pulls of the weight stream: with two row tiles per CTA the ring is deeper in time, and waves of few CTAs pay)
-    const double kSmBytesPerUs = R > kLnBM ? 80e3 : 55e3;
     const int k_steps = (K1 + K2) / kLnBK;
     const int w_rows = gate ? 2 * N : N;
     LnPlan best = {};
