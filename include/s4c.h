@@ -93,7 +93,9 @@ const char* s4c_status_string(s4c_status code);
  * query head h is h / (Hq/Hkv).  Scores are scale * <q,k>; softmax statistics and accumulation
  * are fp32; for S4C_BF16 the probabilities are rounded to bf16 before the PV product, and partial
  * results of the splits of a long cache are exchanged as normalised fp16 rows: output entries
- * beyond +-65504 (possible only with V entries of that size) are clamped there.
+ * beyond +-65504 (possible only with V entries of that size) are clamped there.  A NaN or Inf in K of a
+ * tree slot stays with the rows that see the slot; one in V does so for S4C_F32, while for S4C_BF16 the
+ * PV product multiplies it by the other rows' probability 0.  Slots past the sequence may hold anything.
  *
  *   q          [B,Hq,T,d]   dt     queries of the tree tokens (after positional encoding)
  *   k_cache    [B,Hkv,C,d]  dt     keys; the tree tokens' own keys already sit at slots L_b..L_b+T-1
@@ -301,19 +303,6 @@ size_t s4c_lm_head_greedy_workspace_bytes(int R, int V, int H);
  * Section 3.2 with the same shape and numbering; child j of node n carries topk[b, n, j]
  * (topk [B, T, k] int32, device; k >= every branching factor).  No workspace.  With s4c_lm_head_topk
  * in front, a drafting round needs no [B, T, V] array of probabilities at all. */
-/* s4c_draft_level -- what a drafting round does between two heads, in one launch: `choice` [B, from_count, k] are the
- * ranked choices of the nodes from_first .. from_first + from_count - 1 (one depth of the tree).  They are stored in
- * topk_all [B, T, k], the tree is written as s4c_tree_build_topk writes it from topk_all, and for the nodes to_first ..
- * to_first + to_count - 1 (their children; to_count may be 0) come out, one row per node and sequence, the token
- * (tok_out), root_position + depth (pos_out), the row of `embedding` [V, H] at the token (e_out; zeros outside [0, V))
- * and the parent's row of `features` [B * from_count, H] (f_out).  embedding .. pos_out are not read when to_count = 0.
- * bf16 rows, H a multiple of 8. */
-s4c_status s4c_draft_level(const int32_t* choice, int k, const int32_t* branching, int depth, int from_first, int from_count,
-                           int to_first, int to_count, const int32_t* root_token, const int32_t* root_position, int B,
-                           int T, int32_t* topk_all, int32_t* tokens, int32_t* parent, int32_t* position,
-                           int32_t* n_nodes, const void* embedding, int V, const void* features, int H, void* e_out,
-                           void* f_out, int32_t* tok_out, int32_t* pos_out, s4c_stream_t stream);
-
 size_t s4c_lm_head_topk_workspace_bytes(int R, int V, int H, int k);
 
 s4c_status s4c_lm_head_topk(const void* hidden, const void* weight, int R, int V, int H, int k, int32_t* token,
@@ -331,6 +320,19 @@ s4c_status s4c_lm_head_greedy(const void* hidden, const void* weight, int R, int
 s4c_status s4c_tree_accept_tokens(const int32_t* target_token, const int32_t* tokens, const int32_t* parent,
                                   const int32_t* n_nodes, int B, int T, int V, int max_depth, int32_t* accept_len,
                                   int32_t* path, int32_t* next_token, int32_t* status, s4c_stream_t stream);
+
+/* s4c_draft_level -- what a drafting round does between two heads, in one launch: `choice` [B, from_count, k] are the
+ * ranked choices of the nodes from_first .. from_first + from_count - 1 (one depth of the tree).  They are stored in
+ * topk_all [B, T, k], the tree is written as s4c_tree_build_topk writes it from topk_all, and for the nodes to_first ..
+ * to_first + to_count - 1 (their children; to_count may be 0) come out, one row per node and sequence, the token
+ * (tok_out), root_position + depth (pos_out), the row of `embedding` [V, H] at the token (e_out; zeros outside [0, V))
+ * and the parent's row of `features` [B * from_count, H] (f_out).  embedding .. pos_out are not read when to_count = 0.
+ * bf16 rows, H a multiple of 8. */
+s4c_status s4c_draft_level(const int32_t* choice, int k, const int32_t* branching, int depth, int from_first, int from_count,
+                           int to_first, int to_count, const int32_t* root_token, const int32_t* root_position, int B,
+                           int T, int32_t* topk_all, int32_t* tokens, int32_t* parent, int32_t* position,
+                           int32_t* n_nodes, const void* embedding, int V, const void* features, int H, void* e_out,
+                           void* f_out, int32_t* tok_out, int32_t* pos_out, s4c_stream_t stream);
 
 /* s4c_lm_head_logits -- the LM head when the logits themselves are wanted: verification by speculative
  * sampling (Eq. 11-12, temperature > 0) needs the target's distribution at the walked nodes, so

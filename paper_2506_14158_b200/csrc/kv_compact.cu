@@ -5,9 +5,9 @@
 // row set and moves it for j = 1..a in ascending order.  Because a path is strictly increasing
 // (path[j] >= j), a destination slot j is never a source of a later copy, so the ascending order is
 // race-free in place without a snapshot; loads are issued in batches ahead of their stores for
-// memory-level parallelism.  cache_len is read by the copy kernel and rewritten by a second, tiny
-// kernel ordered after it on the stream (which also gathers the features), so no CTA can observe the
-// new length.
+// memory-level parallelism.  Further blocks of the same launch gather the features.  cache_len is read
+// by this kernel and rewritten by a second, tiny one ordered after it on the stream, so no CTA can
+// observe the new length.
 #include <algorithm>
 
 #include "s4c_common.cuh"

@@ -1,8 +1,8 @@
-// Tree-masked attention on CUDA cores (Section 3.2 tree mask; Figure 3): the float32 path and the
-// generic fallback.
+// Tree-masked attention on CUDA cores (Section 3.2 tree mask; Figure 3): the float32 path, and the merge of
+// partial results that the tensor-core kernel leaves in the workspace.
 //
-// Used for S4C_F32 inputs (fp32 FMA keeps the 1e-4 accuracy that tf32 tensor-core products would lose)
-// and for bf16 shapes the tensor-core kernel does not take.  Split-KV: grid (splits, Hq, B); a CTA stages
+// Used for S4C_F32 inputs (fp32 FMA keeps the 1e-4 accuracy that tf32 tensor-core products would lose); every
+// bf16 shape goes to the tensor-core kernel.  Split-KV: grid (splits, Hq, B); a CTA stages
 // 32 cache slots at a time in shared memory and its 16 warps take the query rows in turn.  Scores: a lane per slot, the
 // whole dot product in one thread; one warp maximum and one sum per 32 slots; then the lanes spread over the head
 // dimension for P V.  (With the lanes over the head dimension throughout, every slot cost a chain of five shuffles and
@@ -22,7 +22,7 @@ constexpr int kSimtWarps = kSimtThreads / 32;
 constexpr float kLog2e = 1.4426950408889634f;
 
 template <typename T>
-struct Elem;
+struct Elem;  // (bf16 only leaves: the merge writes it)
 template <>
 struct Elem<float> {
     template <int N>
@@ -43,19 +43,6 @@ struct Elem<float> {
 };
 template <>
 struct Elem<__nv_bfloat16> {
-    template <int N>
-    static __device__ __forceinline__ void load(const __nv_bfloat16* p, float (&v)[N]) {
-        if (N == 4) {
-            const uint2 t = __ldg(reinterpret_cast<const uint2*>(p));
-            const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&t.x);
-            const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&t.y);
-            v[0] = __low2float(a), v[1] = __high2float(a), v[2] = __low2float(b), v[3] = __high2float(b);
-        } else {
-            const uint32_t t = __ldg(reinterpret_cast<const uint32_t*>(p));
-            const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&t);
-            v[0] = __low2float(a), v[1] = __high2float(a);
-        }
-    }
     template <int N>
     static __device__ __forceinline__ void store(__nv_bfloat16* p, const float (&v)[N]) {
 #pragma unroll
@@ -223,7 +210,7 @@ tree_attention_combine_kernel(const float* __restrict__ ws, const int32_t* __res
 }
 
 int simt_splits(int B, int Hq, int C) {
-    int s = ceil_div(4 * 148, B * Hq);  // ~4 CTAs of 4 warps per SM
+    int s = ceil_div(4 * 148, B * Hq);  // ~4 CTAs of 16 warps per SM
     s = s < 1 ? 1 : s;
     const int cap = ceil_div(C, kSimtTile);  // a staged tile of slots per split at least
     return s > cap ? cap : (s > 64 ? 64 : s);
@@ -279,17 +266,9 @@ s4c_status tree_attention_simt(const void* q, const void* k, const void* v, cons
                                const int32_t* parent, const int32_t* n_nodes, void* out, int B, int T, int Hq, int Hkv,
                                int d, int C, int span, s4c_dtype dt, float scale, int32_t* status, void* ws,
                                cudaStream_t stream) {
-#define S4C_SIMT(TYPE, DD) \
-    launch_simt<TYPE, DD>(q, k, v, cache_len, parent, n_nodes, out, B, T, Hq, Hkv, C, span, scale, status, ws, stream)
-    if (dt == S4C_F32) {
-        if (d == 64) return S4C_SIMT(float, 64);
-        if (d == 128) return S4C_SIMT(float, 128);
-    } else {
-        if (d == 64) return S4C_SIMT(__nv_bfloat16, 64);
-        if (d == 128) return S4C_SIMT(__nv_bfloat16, 128);
-    }
-#undef S4C_SIMT
-    return S4C_ERR_UNSUPPORTED;
+    if (dt != S4C_F32 || (d != 64 && d != 128)) return S4C_ERR_UNSUPPORTED;
+    return (d == 64 ? launch_simt<float, 64> : launch_simt<float, 128>)(q, k, v, cache_len, parent, n_nodes, out, B, T, Hq, Hkv, C, span, scale,
+                                                                        status, ws, stream);
 }
 
 }  // namespace s4c
