@@ -29,6 +29,8 @@
 #include <cuda_fp16.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "s4c_common.cuh"
 #include "tree_attention.cuh"
 
@@ -258,9 +260,6 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float a, float b, float c, float d) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
 __device__ __forceinline__ void st_cluster_f2(uint32_t addr, float a, float b) {
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }
@@ -269,22 +268,12 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-    return v;
-}
 __device__ __forceinline__ void st_cluster_u4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-__device__ __forceinline__ uint2 ld_cluster_u2(uint32_t addr) {
-    uint2 v;
-    asm volatile("ld.shared::cluster.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_cluster_u1(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr));
+__device__ __forceinline__ uint4 ld_cluster_u4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
     return v;
 }
 // Two floats to fp16 (a in the low half), saturating at the largest finite value: a normalised output row is a convex
@@ -296,6 +285,17 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
     return r;
 }
 __device__ __forceinline__ float2 unpack_half2(uint32_t v) { return __half22float2(*reinterpret_cast<const __half2*>(&v)); }
+// plain shared memory, by the same 32-bit addresses
+__device__ __forceinline__ uint4 ld_shared_u4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ float2 ld_shared_f2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
 __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
     float2 v;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
@@ -402,6 +402,17 @@ __device__ __forceinline__ size_t out_row_offset(const TcParams& prm, int b, int
     if (!ROWS) return ((size_t)(b * prm.Hq + first_head) * T + gr) * D;
     const int g = gr / T, t = gr - g * T;
     return (((size_t)b * T + t) * prm.Hq + first_head + g) * D;
+}
+
+// eight columns of an output row: v * scale, rounded to bf16, one 16-byte store
+__device__ __forceinline__ void store_row8(__nv_bfloat16* dst, const float (&v)[8], float scale) {
+    uint32_t pk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j] * scale, v[2 * j + 1] * scale);
+        pk[j] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
 }
 
 // Tile range of a split: tiles are dealt out as evenly as whole tiles allow, the odd ones to the FIRST splits -- the last
@@ -916,7 +927,26 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 uint32_t hx[CPT / 2];
 #pragma unroll
                 for (int k = 0; k < CPT; k += 2) hx[k >> 1] = pack_half2(acc[k] * inv_den, acc[k + 1] * inv_den);
-                if (PUSH == 1) {
+                if (splits == 1) {
+                    // ... and, with no other split to merge it with, the output: the steps of the merge below with one partial
+                    // (192 pairs of one row, two CTAs per SM, L=1024: 25.5 -> 22.4 us per launch; 320 pairs of 26 rows: 49.9 -> 43.3)
+                    if (mine && run && !*dead) {  // (a CTA that gave up a wait stores nothing; every warp has passed its waits here)
+                        const int gr = mt0 * kBM + r;
+                        const bool valid = n == T || gr % T < n;
+                        const float w = exp2f(M - M) * den, inv = (valid && w > 0.f) ? 1.f / w : 0.f;
+                        __nv_bfloat16* dst = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + col0;
+#pragma unroll
+                        for (int k = 0; k < CPT / 2; k += 4) {
+                            float v[8];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float2 a = unpack_half2(hx[k + j]);
+                                v[2 * j] = w * a.x, v[2 * j + 1] = w * a.y;
+                            }
+                            store_row8(dst + 2 * k, v, inv);
+                        }
+                    }
+                } else if (PUSH == 1) {
                     // ... stored to CTA r % splits, slot (r / splits) * splits + split of its receive area
                     if (mine && run) {
                         const uint32_t recv = base + (uint32_t)(Cfg::kQBytes + 2 * S * Cfg::kTileBytes);
@@ -981,7 +1011,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         tc_fence_before();
     }
 
-    if (PUSH == 1 && prm.mode == kModeCluster) {
+    if (PUSH == 1 && prm.mode == kModeCluster && splits > 1) {
         // ---- every split's partial of this CTA's rows (rank, rank + splits, ...) has been stored into its receive area
         __syncwarp();
         cluster_sync_all();
@@ -1026,98 +1056,108 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 }
             }
         __syncthreads();  // warp 1 frees the tensor memory below: every warp is done
-    } else if (prm.mode == kModeCluster) {
-        // ---- merge the splits (and turns) through distributed shared memory: this CTA owns the output rows
-        //      rank, rank + splits, ... of every row tile.  One warp per row, two rows at a time: lane i fetches
-        //      (offset, sum) of partial i, every lane its 4 (d = 64: 2) output columns of up to 8 partials of both rows,
-        //      all requests in flight before the first use -- a remote read takes about a microsecond
+    } else if (PUSH != 2 && prm.mode == kModeCluster && !(REP > 1 && splits == 1)) {
+        // ---- merge the splits (and turns): this CTA owns the output rows rank, rank + splits, ... of its row tiles.  A thread takes
+        //      16 bytes of an exchange row at a time (8 columns) and finds the weights of the row's partials itself, so nothing is
+        //      exchanged between lanes; all requests of U such items go out before the first use.  (A warp per row, four columns a
+        //      lane, offsets and weights by shuffles: 2 us for every two to four rows of a warp, most of it instructions.)  The
+        //      partials of this CTA come from its own shared memory, the others through distributed shared memory, whose path is
+        //      slow: about a microsecond a read, 7 to 12 bytes per clock for an SM when all pull at once.  16 x 8 pairs of 104 rows in
+        //      two turns, L=2000: 34.3 -> 28.2 us per launch; 4 x 8 pairs of 256 rows, four splits, L=4096: 27.7 -> 26.8 us.
         __syncwarp();
-        cluster_sync_all();
+        if (splits > 1) {
+            cluster_sync_all();
+        } else {
+            __syncthreads();  // (the turns of an unsplit launch: everything to be merged is this CTA's own)
+        }
         // the same in every CTA of the cluster: it depends on the sequence only
         const bool run = (flags | *bad_s) == 0;
         const int gave_up = *dead;  // a CTA that gave up a wait stores nothing; only the stores wait for this word
-        const uint32_t rank = cluster_ctarank();
+        const uint32_t rank = splits > 1 ? cluster_ctarank() : 0u;
         // row copies were merged inside their CTA (one exchange row per row, behind the parked copies); turns are
         // merged here with the splits
         const uint32_t part = base + (uint32_t)(REP > 1 ? Cfg::kXBytes : 0);
-        constexpr int EPL = D / 32;  // output elements per lane
+        constexpr int CH = D / 8;    // 16-byte pieces of a row
         constexpr int NC = TC;       // partials per split
-        constexpr int U = 2;         // output rows in flight per warp
         const int np = splits * NC;  // partials per output row (<= 16)
-        // exchange row of partial i of output row (t, lr): i / NC is the split, i % NC the turn
-        auto part_addr = [&](int t, int lr, int i) {
-            return map_to_cta(part + (uint32_t)(((t * TC + i % NC) * kBM + lr) * XS), (uint32_t)(i / NC));
-        };
-        const int stride = splits * (Cfg::kThreads / 32);
-        if (run)
-            for (int idx0 = (int)rank + splits * warp; idx0 < NM * RB; idx0 += U * stride) {
-                int tt[U], lr[U];
-                bool ok[U];
-                float2 ml[U];
+        int n_rows = 0;              // valid rows: the first ones of the row tiles
+#pragma unroll
+        for (int t = 0; t < NM; ++t) n_rows += rows_in(t);
+        const int n_items = n_rows > (int)rank ? (n_rows - (int)rank + splits - 1) / splits * CH : 0;
+        // U pieces in flight per thread, K >= np partials
+        auto merge_rows = [&](auto U_, auto K_) {
+            constexpr int U = decltype(U_)::value, K = decltype(K_)::value;
+            for (int it0 = threadIdx.x; it0 < n_items; it0 += U * Cfg::kThreads) {
+                float2 ml[U][K];
+                uint4 h[U][K];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int idx = idx0 + u * stride;
-                    tt[u] = idx / RB, lr[u] = idx % RB;
-                    ok[u] = idx < NM * RB && lr[u] < rows_in(tt[u]);
-                    ml[u] = make_float2(-INFINITY, 0.f);
-                    if (ok[u] && lane < np) ml[u] = ld_cluster_f2(part_addr(tt[u], lr[u], lane) + (uint32_t)(2 * D));
-                }
-                float num[U][4], den[U], w_mine[U];
+                    const int it = it0 + u * Cfg::kThreads;
+                    const int idx = (int)rank + splits * (it / CH);
+                    const int tt = NM == 2 ? idx / kBM : 0, lr = idx - tt * kBM;
+                    const uint32_t at = part + (uint32_t)((tt * TC * kBM + lr) * XS);  // the same place in every CTA; turn c: c * kBM rows on
 #pragma unroll
-                for (int u = 0; u < U; ++u) num[u][0] = num[u][1] = num[u][2] = num[u][3] = 0.f, den[u] = 0.f;
-                for (int i0 = 0; i0 < np; i0 += 8) {
-                    uint2 h[U][8];
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            h[u][k] = make_uint2(0u, 0u);
-                            if (ok[u] && i0 + k < np) {
-                                const uint32_t a = part_addr(tt[u], lr[u], i0 + k) + (uint32_t)(lane * EPL * 2);
-                                if (EPL == 4) {
-                                    h[u][k] = ld_cluster_u2(a);
-                                } else {
-                                    h[u][k].x = ld_cluster_u1(a);
-                                }
+                    for (int k = 0; k < K; ++k) {
+                        ml[u][k] = make_float2(-INFINITY, 0.f);
+                        h[u][k] = make_uint4(0u, 0u, 0u, 0u);
+                        if (it < n_items && k < np) {
+                            const uint32_t a = at + (uint32_t)((k % NC) * kBM * XS), src = (uint32_t)(k / NC);
+                            if (src == rank) {
+                                ml[u][k] = ld_shared_f2(a + 2 * D);
+                                h[u][k] = ld_shared_u4(a + (uint32_t)(it % CH) * 16);
+                            } else {
+                                const uint32_t ra = map_to_cta(a, src);
+                                ml[u][k] = ld_cluster_f2(ra + 2 * D);
+                                h[u][k] = ld_cluster_u4(ra + (uint32_t)(it % CH) * 16);
                             }
                         }
-                    if (i0 == 0) {
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            float M = -INFINITY;  // independent shuffles, not a butterfly: they overlap
-                            for (int i = 0; i < np; ++i) M = fmaxf(M, __shfl_sync(0xffffffffu, ml[u].x, i));
-                            w_mine[u] = lane < np ? exp2f(ml[u].x - M) * ml[u].y : 0.f;  // the partial's share of the sum
-                        }
                     }
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const float w = __shfl_sync(0xffffffffu, w_mine[u], (i0 + k) & 31);  // 0 past the last partial
-                            den[u] += w;  // partial order: the same on every run
-                            const float2 a = unpack_half2(h[u][k].x), c = unpack_half2(h[u][k].y);
-                            num[u][0] = fmaf(w, a.x, num[u][0]), num[u][1] = fmaf(w, a.y, num[u][1]);
-                            num[u][2] = fmaf(w, c.x, num[u][2]), num[u][3] = fmaf(w, c.y, num[u][3]);
-                        }
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (!ok[u] || gave_up) continue;
-                    const int gr = (mt0 + tt[u]) * kBM + lr[u];
-                    const float inv = ((gr % T) < n && den[u] > 0.f) ? 1.f / den[u] : 0.f;
-                    __nv_bfloat16* dst = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + lane * EPL;
-                    const __nv_bfloat162 h0 = __floats2bfloat162_rn(num[u][0] * inv, num[u][1] * inv);
-                    if (EPL == 4) {
-                        const __nv_bfloat162 h1 = __floats2bfloat162_rn(num[u][2] * inv, num[u][3] * inv);
-                        *reinterpret_cast<uint2*>(dst) =
-                            make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-                    } else {
-                        *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(&h0);
+                    const int it = it0 + u * Cfg::kThreads;
+                    float M = -INFINITY, den = 0.f, num[8];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) M = fmaxf(M, ml[u][k].x);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) num[c] = 0.f;
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {  // partial order: the same on every run
+                        if (k >= np) break;
+                        const float w = exp2f(ml[u][k].x - M) * ml[u][k].y;  // the partial's share of the softmax sum
+                        den += w;
+                        const float2 a0 = unpack_half2(h[u][k].x), a1 = unpack_half2(h[u][k].y), a2 = unpack_half2(h[u][k].z),
+                                     a3 = unpack_half2(h[u][k].w);
+                        num[0] = fmaf(w, a0.x, num[0]), num[1] = fmaf(w, a0.y, num[1]);
+                        num[2] = fmaf(w, a1.x, num[2]), num[3] = fmaf(w, a1.y, num[3]);
+                        num[4] = fmaf(w, a2.x, num[4]), num[5] = fmaf(w, a2.y, num[5]);
+                        num[6] = fmaf(w, a3.x, num[6]), num[7] = fmaf(w, a3.y, num[7]);
                     }
+                    if (it >= n_items || gave_up) continue;
+                    const int gr = mt0 * kBM + (int)rank + splits * (it / CH);
+                    const bool valid = n == T || gr % T < n;  // (rows of nodes past the tree's are zero)
+                    const float inv = (valid && den > 0.f) ? 1.f / den : 0.f;
+                    store_row8(prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + (it % CH) * 8, num, inv);
                 }
             }
+        };
+        if (run) {
+            if (TC == 2 && np == 2) {
+                merge_rows(std::integral_constant<int, 4>(), std::integral_constant<int, 2>());
+            } else if (np <= 4) {
+                merge_rows(std::integral_constant<int, 3>(), std::integral_constant<int, 4>());
+            } else if (TC == 1 || np <= 8) {
+                merge_rows(std::integral_constant<int, 2>(), std::integral_constant<int, 8>());
+            } else {
+                merge_rows(std::integral_constant<int, 1>(), std::integral_constant<int, 16>());
+            }
+        }
         __syncwarp();
-        cluster_sync_all();  // nobody leaves while a peer may still read its shared memory
+        if (splits > 1) {
+            cluster_sync_all();  // nobody leaves while a peer may still read its shared memory
+        } else {
+            __syncthreads();
+        }
     } else {
         __syncthreads();
     }
@@ -1329,7 +1369,7 @@ static s4c_status launch_tc_layout(const void* q, const void* k, const void* v, 
     attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attrs[na].val.programmaticStreamSerializationAllowed = 1;
     ++na;
-    if (prm.mode == kModeCluster) {
+    if (prm.mode == kModeCluster && prm.splits > 1) {
         attrs[na].id = cudaLaunchAttributeClusterDimension;
         attrs[na].val.clusterDim.x = prm.splits;
         attrs[na].val.clusterDim.y = 1;
