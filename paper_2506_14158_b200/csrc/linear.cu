@@ -4,10 +4,10 @@
 // s4c_rmsnorm and s4c_embed_gather: the layer's two small row operations (root-mean-square normalisation; Eq. 6,
 // e = Embedding(t)).
 //
-// One CTA per (column tile of the output, row tile, share of the K range): the pipeline of the q/k/v kernel -- warp 0
-// requests 64-element K slices by TMA (128-byte swizzle; slices of the first input, then of the second, against consecutive
-// column ranges of the weight), warp 1 issues the products into an f32 accumulator in tensor memory, warps 2-5 read it
-// (one row per thread), apply the epilogue and store 16 bytes at a time.  Gated form: a tile's accumulator holds its gate
+// One CTA per (column tile of the output, row tile, share of the K range): the pipeline of the q/k/v kernel -- warps 0 and 2
+// request 64-element K slices by TMA (128-byte swizzle; the weight; slices of the first input, then of the second, against
+// consecutive column ranges of it), warp 1 issues the products into an f32 accumulator in tensor memory, warps 4-11 read it
+// (one row per thread), apply the epilogue and store whole runs of a row.  Gated form: a tile's accumulator holds its gate
 // columns beside the same outputs' up columns (two boxes of the weight), as the q/k/v kernel keeps a rotary pair in one row.
 // The launch shape -- tile width (a multiple of 16 columns), one or two 128-row accumulators per CTA, the number of CTAs
 // that share a tile's K range -- is chosen per call (ln_plan); shared-out K ranges meet again in linear_finish_kernel, in
@@ -29,7 +29,9 @@ constexpr int kLnBN = 256;       // most accumulator columns per CTA (the launch
 constexpr int kLnBK = 64;        // K elements per stage (one 128-byte swizzled row)
 constexpr int kLnMaxStages = 12;
 constexpr int kLnRingBytes = 192 * 1024;
-constexpr int kLnThreads = 224;  // weight producer, issuer, four epilogue warps, input producer
+constexpr int kLnRoleWarps = 4;  // weight producer, issuer, input producer, one without a role: the epilogue warps start at a multiple of four
+constexpr int kLnEpiGroups = 2;  // epilogue warps per tensor-memory quarter (32 rows), which share the tile's columns
+constexpr int kLnThreads = 32 * (kLnRoleWarps + 4 * kLnEpiGroups);
 constexpr int kLnBars = 2 * kLnMaxStages + 2;  // full[], empty[], acc_full, drain
 constexpr int kLnSmemBytes = 1024 + kLnRingBytes + kLnBars * 8 + 32;
 
@@ -51,7 +53,9 @@ struct LnParams {
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
 
-__global__ void __launch_bounds__(kLnThreads, 1)
+// (at most half the registers of an SM, as if two CTAs were to share it: the finishing kernel of one product and the CTAs of the next
+// one, which request their weights meanwhile, are resident together)
+__global__ void __launch_bounds__(kLnThreads, 2)
 linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
               const __grid_constant__ CUtensorMap map_w, const LnParams prm) {
     constexpr int SM = kLnMaxStages;
@@ -78,19 +82,26 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
     const int k_steps = k_end - k_begin;  // this CTA's share of the K slices (>= 1: the launch keeps splits <= slices)
     const int cols = prm.cols;
     const int n0 = ntile * cols;  // first output column of this tile
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 2), mbar_init(EMPTY(s), 1);
-        mbar_init(ACC_FULL, 1), mbar_init(DRAIN, 1);
+    // Warp 0 sets the barriers up and goes straight on to its copies: the first weights are requested before the other warps have
+    // met (tensor memory may still be with the CTA in front on this SM; the copies do not need it).
+    if (warp == 0) {
+        if (lane < S) mbar_init(FULL(lane), 2), mbar_init(EMPTY(lane), 1);
+        if (lane == S) mbar_init(ACC_FULL, 1), mbar_init(DRAIN, 1);
         mbar_fence_init();
-        *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
-        tma_prefetch_desc(&map_x1), tma_prefetch_desc(&map_w);
-        if (prm.k2_steps) tma_prefetch_desc(&map_x2);
+        if (lane == 0) *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
+        __syncwarp();
+        named_bar_arrive(1, kLnThreads);
+    } else {
+        if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), kLnBN * prm.nm);
+        if (warp == 2 && lane == 0) {
+            tma_prefetch_desc(&map_x1);
+            if (prm.k2_steps) tma_prefetch_desc(&map_x2);
+        }
+        tc_fence_before();
+        named_bar_sync(1, kLnThreads);
+        tc_fence_after();
     }
-    if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), kLnBN * prm.nm);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_cta = (uint32_t)*tmem_slot;
+    const uint32_t tmem_cta = warp == 0 ? 0u : (uint32_t)*tmem_slot;  // (warp 0 has not waited for it and does not use it)
     const uint32_t tmem = tmem_cta;
 
     // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: what such
@@ -117,7 +128,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
             issued_s[0] = fill;
         }
         __syncwarp();
-    } else if (warp == 6) {
+    } else if (warp == 2) {
         // ================= input producer =================
         if (elect_one()) {
             griddep_wait();
@@ -170,95 +181,124 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
             if (ok) tc_commit(ACC_FULL);
         }
         __syncwarp();
-    } else {
+    } else if (warp >= kLnRoleWarps) {
         // ================= epilogue =================
+        // A thread reads one row of the accumulator, 32 columns at a time; stored from there a warp's store would touch 32 rows.  The
+        // runs are turned around in shared memory (in the ring, which nothing uses any more) so that eight lanes hold a run of one
+        // row: 128 bytes of float32 in one piece.  Two warps per 32 rows share the columns (one, with 16-byte stores of a row each and a
+        // branch per element in the gate: 4096 x 4096 shared out four ways 19.7 -> 15.5 us at 256 rows and 11.4 -> 10.3 at 26,
+        // 14336 x 4096 seven ways 43.2 -> 41.4 at 256, gate/up of 4096 x 14336 55.2 -> 54.3; three warps, whose CTAs no longer
+        // leave the finishing kernel its registers: 19.9 us at 256 rows and 12.6 at 26 for the first).
         const int q = warp & 3;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
+        const int grp = (warp - kLnRoleWarps) >> 2;
         griddep_wait();  // (the residual may be the result of the kernel in front, and nothing is written before that kernel has ended)
-        bool ok = mbar_wait(ACC_FULL, 0, dead);
-        ok = __all_sync(0xffffffffu, ok);
+        bool ok = true;
+        if (lane == 0) ok = mbar_wait(ACC_FULL, 0, dead);
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         if (ok) tc_fence_after();
+        const uint32_t stage = base + (uint32_t)(warp - kLnRoleWarps) * 4096u;  // 32 rows x 128 bytes, 16-byte pieces XOR-swizzled
+        const int w_rows = prm.gate ? 2 * prm.N : prm.N;
+        const bool shares = prm.splits > 1;
+        // shares of the K slices go out raw, column = weight row (linear_finish_kernel adds them in split order and applies what
+        // follows the product); else runs of 32 output columns, the last may be short
+        const int runs = ((shares ? bn : cols) + 31) / 32;
+        const int rr0 = lane >> 3, piece = lane & 7;  // after the turn: this lane's rows rr0 + 4 i, and its four columns of the run
         for (int rt = 0; ok && rt < prm.nm; ++rt) {
-            const int r = (mtile * prm.nm + rt) * kLnBM + q * 32 + lane;
-            const uint32_t tmem = tmem_cta + (uint32_t)(rt * kLnBN);  // this row tile's accumulator
-            const bool live = r < prm.R;
-            __nv_bfloat16* orow = prm.out + (size_t)(live ? r : 0) * prm.N;
-            const __nv_bfloat16* rrow = prm.residual ? prm.residual + (size_t)(live ? r : 0) * prm.N : nullptr;
-            if (prm.splits > 1) {
-                // a share of the K slices: the raw sums go out as float32, column = weight row; linear_finish_kernel adds the
-                // shares in split order and applies what follows the product
-                const int w_rows = prm.gate ? 2 * prm.N : prm.N;
-                float* prow = prm.partial + ((size_t)blockIdx.z * prm.R + (live ? r : 0)) * w_rows;
-                for (int c = 0; c < (bn + 31) / 32; ++c) {
-                    uint32_t a[32];
-                    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + c * 32, a);
+            const int r0 = (mtile * prm.nm + rt) * kLnBM + q * 32, live = min(32, prm.R - r0);  // this warp's rows r0 .. r0 + live - 1
+            if (live <= 0) break;  // (the later row tiles have none either)
+            for (int c = (grp + rt) % kLnEpiGroups; c < runs; c += kLnEpiGroups) {
+                const uint32_t acc = tmem_cta + (uint32_t)(rt * kLnBN) + ((uint32_t)(q * 32) << 16) + c * 32;
+                uint32_t a[32];
+                __syncwarp();  // (the lanes may have left the run before at different places; the load is warp-wide)
+                tmem_ld32(acc, a);
+                if (!shares && prm.gate) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t u[16];
+                        tmem_ld16(acc + cols + h * 16, u);
+                        tmem_wait_ld();
+                        if (prm.bias) {  // (apart from the products below: a branch per element would run them one after the other)
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                const int col = min(n0 + c * 32 + h * 16 + j, prm.N - 1);
+                                a[h * 16 + j] = __float_as_uint(__uint_as_float(a[h * 16 + j]) + __bfloat162float(prm.bias[col]));
+                                u[j] = __float_as_uint(__uint_as_float(u[j]) + __bfloat162float(prm.bias[prm.N + col]));
+                            }
+                        }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            a[h * 16 + j] = __float_as_uint(silu(__uint_as_float(a[h * 16 + j])) * __uint_as_float(u[j]));
+                    }
+                } else {
                     tmem_wait_ld();
-                    if (live) {
+                }
 #pragma unroll
-                        for (int v4 = 0; v4 < 8; ++v4) {
-                            // accumulator column -> weight row: plain n0 + column; gated: the first cols are gate rows n0..,
-                            // the others up rows N + n0.. (cols is a multiple of 16: four columns never straddle)
-                            const int tc = c * 32 + v4 * 4;
-                            const bool up_part = prm.gate && tc >= cols;
-                            const int wrow = up_part ? prm.N + n0 + tc - cols : n0 + tc;
-                            if (tc + 4 <= bn && wrow + 4 <= (up_part ? 2 * prm.N : prm.N))
-                                *reinterpret_cast<float4*>(prow + wrow) =
-                                    make_float4(__uint_as_float(a[v4 * 4]), __uint_as_float(a[v4 * 4 + 1]), __uint_as_float(a[v4 * 4 + 2]),
-                                                __uint_as_float(a[v4 * 4 + 3]));
+                for (int v = 0; v < 8; ++v)
+                    st_shared_u4(stage + (uint32_t)(lane * 128 + ((v ^ (lane & 7)) << 4)), a[4 * v], a[4 * v + 1], a[4 * v + 2], a[4 * v + 3]);
+                __syncwarp();
+                float4 f[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = rr0 + 4 * i;
+                    f[i] = ld_shared_f4(stage + (uint32_t)(rr * 128 + ((piece ^ (rr & 7)) << 4)));
+                }
+                __syncwarp();  // the run is in registers: the next one may take its place
+                const int tc = c * 32 + piece * 4;
+                if (shares) {
+                    // accumulator column -> weight row: plain n0 + column; gated: the first cols are gate rows n0..,
+                    // the others up rows N + n0.. (cols is a multiple of 16: four columns never straddle)
+                    const bool up_part = prm.gate && tc >= cols;
+                    const int wrow = up_part ? prm.N + n0 + tc - cols : n0 + tc;
+                    if (tc + 4 > bn || wrow + 4 > (up_part ? 2 * prm.N : prm.N)) continue;
+                    float* dst = prm.partial + ((size_t)blockIdx.z * prm.R + r0 + rr0) * w_rows + wrow;
+                    const size_t step4 = (size_t)w_rows * 4;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i, dst += step4)
+                        if (rr0 + 4 * i < live) *reinterpret_cast<float4*>(dst) = f[i];
+                    continue;
+                }
+                if (tc + 4 > cols || n0 + tc + 4 > prm.N) continue;  // (cols and N are multiples of 8)
+                const size_t at = (size_t)(r0 + rr0) * prm.N + n0 + tc, step4 = (size_t)prm.N * 4;
+                if (prm.bias && !prm.gate) {
+                    float bias[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) bias[j] = __bfloat162float(prm.bias[n0 + tc + j]);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) f[i].x += bias[0], f[i].y += bias[1], f[i].z += bias[2], f[i].w += bias[3];
+                }
+                if (prm.residual) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint2 rv[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            rv[i] = make_uint2(0u, 0u);
+                            if (rr0 + 4 * (h * 4 + i) < live) rv[i] = __ldg(reinterpret_cast<const uint2*>(prm.residual + at + (h * 4 + i) * step4));
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float2 e0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&rv[i].x)),
+                                         e1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&rv[i].y));
+                            float4& g = f[h * 4 + i];
+                            g.x += e0.x, g.y += e0.y, g.z += e1.x, g.w += e1.y;
                         }
                     }
-                    __syncwarp();
                 }
-            }
-            // runs of 32 output columns; the last may be short (loads past the tile's columns stay inside the allocation)
-            const int n_chunks = prm.splits > 1 ? 0 : (cols + 31) / 32;
-            for (int c = 0; c < n_chunks; ++c) {
-                uint32_t a[32], u[32];
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + c * 32, a);
-                if (prm.gate) tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + cols + c * 32, u);
-                tmem_wait_ld();
-                if (live) {
+                if (prm.out_f32) {  // the sums as they are (logits)
+                    float* dst = prm.out_f32 + at;
 #pragma unroll
-                    for (int v8 = 0; v8 < 4; ++v8) {  // eight output columns = one 16-byte store
-                        const int col = n0 + c * 32 + v8 * 8;
-                        if (c * 32 + v8 * 8 + 8 > cols || col + 8 > prm.N) continue;  // (cols and N are multiples of 8)
-                        float y[8];
+                    for (int i = 0; i < 8; ++i, dst += step4)
+                        if (rr0 + 4 * i < live) *reinterpret_cast<float4*>(dst) = f[i];
+                } else {
+                    __nv_bfloat16* dst = prm.out + at;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            y[j] = __uint_as_float(a[v8 * 8 + j]);
-                            if (prm.bias) y[j] += __bfloat162float(prm.bias[col + j]);
-                        }
-                        if (prm.gate) {
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                float up = __uint_as_float(u[v8 * 8 + j]);
-                                if (prm.bias) up += __bfloat162float(prm.bias[prm.N + col + j]);
-                                y[j] = silu(y[j]) * up;
-                            }
-                        }
-                        if (rrow) {
-                            const uint4 rv = __ldg(reinterpret_cast<const uint4*>(rrow + col));
-                            const __nv_bfloat162* rp = reinterpret_cast<const __nv_bfloat162*>(&rv);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const float2 f = __bfloat1622float2(rp[j]);
-                                y[2 * j] += f.x, y[2 * j + 1] += f.y;
-                            }
-                        }
-                        if (prm.out_f32) {  // the sums as they are (logits)
-                            float4* dst = reinterpret_cast<float4*>(prm.out_f32 + (size_t)r * prm.N + col);
-                            dst[0] = make_float4(y[0], y[1], y[2], y[3]), dst[1] = make_float4(y[4], y[5], y[6], y[7]);
-                            continue;
-                        }
-                        uint32_t pk[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const __nv_bfloat162 p = __floats2bfloat162_rn(y[2 * j], y[2 * j + 1]);
-                            pk[j] = *reinterpret_cast<const uint32_t*>(&p);
-                        }
-                        *reinterpret_cast<uint4*>(orow + col) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    for (int i = 0; i < 8; ++i, dst += step4) {
+                        const __nv_bfloat162 p0 = __floats2bfloat162_rn(f[i].x, f[i].y), p1 = __floats2bfloat162_rn(f[i].z, f[i].w);
+                        if (rr0 + 4 * i < live)
+                            *reinterpret_cast<uint2*>(dst) =
+                                make_uint2(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1));
                     }
                 }
-                __syncwarp();  // the lanes took different ways; the next tensor-memory load is warp-wide
             }
         }
         if (ok) tc_fence_before();
@@ -329,8 +369,9 @@ __device__ __forceinline__ uint4 scale8(const uint4& v, const uint4& g, float sc
 // holds the whole row, also writes its root-mean-square normalisation (of the rounded row, as a separate call would).
 // Nothing here is work, everything is latency between two products: the shares' loads go out together, four at a time (one
 // after the other, with 256 threads and two passes, a 4096-wide row of four shares took 6 us).
-__global__ void __launch_bounds__(kRowThreads)
-linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N, int gate, const __nv_bfloat16* __restrict__ bias,
+template <bool kGate>
+__global__ void __launch_bounds__(kRowThreads, 2)
+linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N, const __nv_bfloat16* __restrict__ bias,
                      const __nv_bfloat16* __restrict__ residual, __nv_bfloat16* __restrict__ out,
                      const __nv_bfloat16* __restrict__ norm_weight, float norm_eps, __nv_bfloat16* __restrict__ norm_out,
                      float* __restrict__ out_f32) {
@@ -342,6 +383,7 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
     uint4 g = make_uint4(0, 0, 0, 0);  // the norm weight, which the product in front does not write, under way before the wait
     if (norm_weight && first < N) g = __ldg(reinterpret_cast<const uint4*>(norm_weight + first));
     griddep_wait();
+    constexpr int gate = kGate ? 1 : 0;
     const int w_rows = gate ? 2 * N : N;
     const size_t share = (size_t)R * w_rows;
     float ss = 0.f;
@@ -353,10 +395,11 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
 #pragma unroll
         for (int j = 0; j < 8; ++j) y[j] = 0.f, up[j] = 0.f;
         const float* p = partial + (size_t)r * w_rows + col;
-        for (int z0 = 0; z0 < splits; z0 += 4) {
-            float4 a[4][2], u[4][2];
+        constexpr int kZ = kGate ? 2 : 4;  // (the registers of 64 a thread)
+        for (int z0 = 0; z0 < splits; z0 += kZ) {
+            float4 a[kZ][2], u[kZ][2];
 #pragma unroll
-            for (int z = 0; z < 4; ++z) {
+            for (int z = 0; z < kZ; ++z) {
                 a[z][0] = a[z][1] = u[z][0] = u[z][1] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (z0 + z < splits) {
                     const float4* q = reinterpret_cast<const float4*>(p + (z0 + z) * share);
@@ -365,7 +408,7 @@ linear_finish_kernel(const float* __restrict__ partial, int splits, int R, int N
                 }
             }
 #pragma unroll
-            for (int z = 0; z < 4; ++z) {  // (a share that does not exist adds zero)
+            for (int z = 0; z < kZ; ++z) {  // (a share that does not exist adds zero)
                 y[0] += a[z][0].x, y[1] += a[z][0].y, y[2] += a[z][0].z, y[3] += a[z][0].w;
                 y[4] += a[z][1].x, y[5] += a[z][1].y, y[6] += a[z][1].z, y[7] += a[z][1].w;
                 if (gate) {
@@ -620,8 +663,8 @@ static s4c_status ln_run(const void* x1, const void* x2, const void* w, const vo
     bool ok = ln_launch(linear_kernel, dim3(pl.n_tiles, pl.m_tiles, pl.splits), kLnThreads, kLnSmemBytes, stream, map_x1, map_x2, map_w,
                         prm) == cudaSuccess;
     if (ok && pl.splits > 1)  // the finishing kernel holds whole rows: it normalises them as well
-        ok = ln_launch(linear_finish_kernel, dim3(R, 1, 1), kRowThreads, 0, stream, (const float*)prm.partial, pl.splits, R, N, gate ? 1 : 0,
-                       prm.bias, prm.residual, prm.out, nw, norm_eps, no, prm.out_f32) == cudaSuccess;
+        ok = ln_launch(gate ? linear_finish_kernel<true> : linear_finish_kernel<false>, dim3(R, 1, 1), kRowThreads, 0, stream,
+                       (const float*)prm.partial, pl.splits, R, N, prm.bias, prm.residual, prm.out, nw, norm_eps, no, prm.out_f32) == cudaSuccess;
     else if (ok && nw)
         ok = ln_launch(rmsnorm_kernel, dim3(R, 1, 1), kRowThreads, 0, stream, (const __nv_bfloat16*)prm.out, nw, norm_eps, N, no) == cudaSuccess;
     if (!ok) {

@@ -6,9 +6,9 @@
 //
 // [B*T, H] x [(Hq+2Hkv)*d, H]^T is a dense contraction: bf16 operands on the tcgen05 tensor cores, f32 accumulator in tensor
 // memory.  One CTA per (head, 128-row tile): a head's d output columns are one MMA tile, so both halves of every rotary pair
-// (j, j + d/2) sit in the same accumulator row.  Roles as in the LM-head kernel: warp 0 requests 64-element K slices by TMA
-// (128-byte swizzle, a ring of 192 KB cut into 6 to 12 stages), warp 1 issues the products, warps 2-5 read the finished accumulator (one row per
-// thread), rotate, round to bf16 and store 16 bytes at a time.  A small kernel in front checks the trees and the capacity
+// (j, j + d/2) sit in the same accumulator row.  Roles as in the LM-head kernel: warps 0 (weights) and 2 (states) request 64-element
+// K slices by TMA (128-byte swizzle, a ring of 192 KB cut into 6 to 12 stages), warp 1 issues the products, warps 4-11 read the finished
+// accumulator (one row per thread), rotate, round to bf16 and store whole runs of a row.  A small kernel in front checks the trees and the capacity
 // and tabulates cos / sin per (node, pair) in float64; the contraction is launched programmatically dependent on it and
 // only its epilogue waits for it.  Every wait on a barrier is bounded.
 #include <cuda.h>
@@ -27,7 +27,8 @@ constexpr int kQkBM = 128;       // rows per CTA (tensor-memory lanes)
 constexpr int kQkBK = 64;        // hidden elements per stage (one 128-byte swizzled row)
 constexpr int kQkMaxStages = 12;
 constexpr int kQkRingBytes = 192 * 1024;  // cut into stages at launch: a stage holds the rows that exist and the head's d weight rows
-constexpr int kQkThreads = 224;  // weight producer, issuer, four epilogue warps, state producer
+constexpr int kQkRoleWarps = 4;  // weight producer, issuer, state producer, one without a role: the epilogue warps start at a multiple of four
+constexpr int kQkThreads = 32 * (kQkRoleWarps + 8);  // two epilogue warps per tensor-memory quarter (32 rows)
 constexpr int kQkBars = 2 * kQkMaxStages + 2;  // full[], empty[], acc_full, drain
 constexpr int kQkSmemBytes = 1024 + kQkRingBytes + kQkBars * 8 + 32;
 
@@ -100,30 +101,34 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int head = blockIdx.x, mtile = blockIdx.y, d = prm.d;
     const uint32_t tmem_cols = d <= 64 ? 64u : 128u;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 2), mbar_init(EMPTY(s), 1);
-        mbar_init(ACC_FULL, 1), mbar_init(DRAIN, 1);
+    // Warp 0 sets the barriers up and goes straight on to its copies: the first weights are requested before the other warps have met.
+    if (warp == 0) {
+        if (lane < S) mbar_init(FULL(lane), 2), mbar_init(EMPTY(lane), 1);
+        if (lane == S) mbar_init(ACC_FULL, 1), mbar_init(DRAIN, 1);
         mbar_fence_init();
-        *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
-        tma_prefetch_desc(&map_x), tma_prefetch_desc(&map_w);
+        if (lane == 0) *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
+        __syncwarp();
+        named_bar_arrive(1, kQkThreads);
+    } else {
+        if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), tmem_cols);
+        if (warp == 2 && lane == 0) tma_prefetch_desc(&map_x);
+        tc_fence_before();
+        named_bar_sync(1, kQkThreads);
+        tc_fence_after();
     }
-    if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), tmem_cols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = (uint32_t)*tmem_slot;
+    const uint32_t tmem = warp == 0 ? 0u : (uint32_t)*tmem_slot;  // (warp 0 has not waited for it and does not use it)
 
     // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: what such
     // a thread computes per slice is time the stream waits, so the two operands have a producer each.
     // Every CTA walks the K slices from a start of its own: the CTAs of a row tile all read the same state tiles, and in step
     // they would all ask the same L2 lines at the same moment (the order of a sum's terms is free).
     const int k_steps = prm.k_steps, k_first = (int)((blockIdx.x * 7u + blockIdx.y * 3u) % (uint32_t)k_steps);
-    if (warp == 0 || warp == 6) {
-        // ================= producers: weights (warp 0), states (warp 6) =================
+    if (warp == 0 || warp == 2) {
+        // ================= producers: weights (warp 0), states (warp 2) =================
         // The weights, which the call in front does not write, fill the first ring while the kernel in front is still running;
         // the states follow once it has ended.
         if (elect_one()) {
-            const bool states = warp == 6;
+            const bool states = warp == 2;
             int s = 0, ks = k_first, fill = 0;
             uint32_t ph = 0;
             const uint32_t first = base + (states ? 0 : x_bytes);
@@ -175,58 +180,85 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             if (ok) tc_commit(ACC_FULL);
         }
         __syncwarp();
-    } else {
+    } else if (warp >= kQkRoleWarps) {
         // ================= epilogue: rotate, round, store =================
-        const int q = warp & 3;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
-        const int r = mtile * kQkBM + q * 32 + lane;
+        // A thread reads one row of the accumulator, 32 columns and their partners half a head on; turned around in shared memory (in
+        // the ring, which nothing uses any more), eight lanes hold a run of one row, so that tables and stores are read and written
+        // in whole pieces.  Two warps per 32 rows take every other run.  What does not depend on the products -- the rows'
+        // destinations, half of the table -- is fetched before them.
+        const int q = warp & 3, grp = (warp - kQkRoleWarps) >> 2;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
+        const int r0 = mtile * kQkBM + q * 32, live = min(32, prm.R - r0), half = d >> 1;
         griddep_wait();  // the rows' bases and the rotary table are complete; the bounded wait starts here
-        bool ok = mbar_wait(ACC_FULL, 0, dead);
-        ok = __all_sync(0xffffffffu, ok);
-        if (ok) {
-            tc_fence_after();
-            const int Lb = r < prm.R ? prm.row_base[r] : -1;
-            const int b = r / prm.T, t = r - b * prm.T, half = d >> 1;
-            __nv_bfloat16* dst = nullptr;
-            bool rotate = true;
-            if (Lb >= 0) {
-                if (head < prm.Hq)
-                    dst = prm.q_out + (((size_t)b * prm.Hq + head) * prm.T + t) * d;
-                else if (head < prm.Hq + prm.Hkv)
-                    dst = prm.k_cache + (((size_t)b * prm.Hkv + (head - prm.Hq)) * prm.C + Lb + t) * d;
-                else
-                    dst = prm.v_cache + (((size_t)b * prm.Hkv + (head - prm.Hq - prm.Hkv)) * prm.C + Lb + t) * d, rotate = false;
+        if (live > 0 && grp * 32 < half) {
+            const int rr0 = lane >> 3, piece = lane & 7, c = grp * 32;  // this lane's rows rr0 + 4 i, and its four pairs c + 4 piece ..
+            const bool rotate = head < prm.Hq + prm.Hkv;
+            __nv_bfloat16* out = head < prm.Hq ? prm.q_out : (rotate ? prm.k_cache : prm.v_cache);
+            long long row_at = -1;  // where row r0 + lane goes (elements), -1: nowhere
+            if (lane < live) {
+                const int r = r0 + lane, Lb = prm.row_base[r], b = r / prm.T, t = r - b * prm.T;
+                if (Lb >= 0)
+                    row_at = head < prm.Hq ? (((long long)b * prm.Hq + head) * prm.T + t) * d
+                                           : (((long long)b * prm.Hkv + (head - prm.Hq) % prm.Hkv) * prm.C + Lb + t) * d;
             }
-            const float2* cs = prm.rope + (size_t)(r < prm.R ? r : 0) * half;
-            for (int c = 0; c < half / 32; ++c) {  // columns [32c, 32c+32) and their partners half further on
-                uint32_t lo[32], hi[32];
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + c * 32, lo);
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + half + c * 32, hi);
-                tmem_wait_ld();
-                if (dst) {
-                    uint32_t plo[16], phi[16];
+            const float2* cs = prm.rope + (size_t)(r0 + rr0) * half + c + piece * 4;
+            float4 w[4][2];  // (cos, sin) of four pairs of four rows
+            auto fetch = [&](int i0) {
 #pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        float a0 = __uint_as_float(lo[j]), a1 = __uint_as_float(lo[j + 1]);
-                        float b0 = __uint_as_float(hi[j]), b1 = __uint_as_float(hi[j + 1]);
-                        if (rotate) {
-                            const float4 w = __ldg(reinterpret_cast<const float4*>(cs + c * 32 + j));  // (cos, sin) of two pairs
-                            const float x0 = a0, x1 = a1;
-                            a0 = x0 * w.x - b0 * w.y, b0 = b0 * w.x + x0 * w.y;
-                            a1 = x1 * w.z - b1 * w.w, b1 = b1 * w.z + x1 * w.w;
-                        }
-                        const __nv_bfloat162 pa = __floats2bfloat162_rn(a0, a1), pb = __floats2bfloat162_rn(b0, b1);
-                        plo[j >> 1] = *reinterpret_cast<const uint32_t*>(&pa), phi[j >> 1] = *reinterpret_cast<const uint32_t*>(&pb);
-                    }
-                    uint4* o_lo = reinterpret_cast<uint4*>(dst + c * 32);
-                    uint4* o_hi = reinterpret_cast<uint4*>(dst + half + c * 32);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        o_lo[v] = make_uint4(plo[4 * v], plo[4 * v + 1], plo[4 * v + 2], plo[4 * v + 3]);
-                        o_hi[v] = make_uint4(phi[4 * v], phi[4 * v + 1], phi[4 * v + 2], phi[4 * v + 3]);
+                for (int i = 0; i < 4; ++i) {
+                    w[i][0] = w[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (rotate && rr0 + 4 * (i0 + i) < live) {
+                        const float4* p = reinterpret_cast<const float4*>(cs + (size_t)(4 * (i0 + i)) * half);
+                        w[i][0] = __ldg(p), w[i][1] = __ldg(p + 1);
                     }
                 }
+            };
+            fetch(0);
+            bool ok = true;
+            if (lane == 0) ok = mbar_wait(ACC_FULL, 0, dead);
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (ok) {
+                tc_fence_after();
+                const uint32_t stage = base + (uint32_t)(warp - kQkRoleWarps) * 8192u;  // twice 32 rows x 128 bytes, 16-byte pieces XOR-swizzled
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t a[32];
+                    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + h * half + c, a);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int v = 0; v < 8; ++v)
+                        st_shared_u4(stage + (uint32_t)(h * 4096 + lane * 128 + ((v ^ (lane & 7)) << 4)), a[4 * v], a[4 * v + 1], a[4 * v + 2],
+                                     a[4 * v + 3]);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i0 = 0; i0 < 8; i0 += 4) {
+                    if (i0) fetch(i0);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int rr = rr0 + 4 * (i0 + i);
+                        const long long to = __shfl_sync(0xffffffffu, row_at, rr);
+                        const uint32_t at = stage + (uint32_t)(rr * 128 + ((piece ^ (rr & 7)) << 4));
+                        const float4 x = ld_shared_f4(at), y = ld_shared_f4(at + 4096);
+                        float a0 = x.x, a1 = x.y, a2 = x.z, a3 = x.w, b0 = y.x, b1 = y.y, b2 = y.z, b3 = y.w;
+                        if (rotate) {
+                            a0 = x.x * w[i][0].x - y.x * w[i][0].y, b0 = y.x * w[i][0].x + x.x * w[i][0].y;
+                            a1 = x.y * w[i][0].z - y.y * w[i][0].w, b1 = y.y * w[i][0].z + x.y * w[i][0].w;
+                            a2 = x.z * w[i][1].x - y.z * w[i][1].y, b2 = y.z * w[i][1].x + x.z * w[i][1].y;
+                            a3 = x.w * w[i][1].z - y.w * w[i][1].w, b3 = y.w * w[i][1].z + x.w * w[i][1].w;
+                        }
+                        const __nv_bfloat162 p0 = __floats2bfloat162_rn(a0, a1), p1 = __floats2bfloat162_rn(a2, a3);
+                        const __nv_bfloat162 p2 = __floats2bfloat162_rn(b0, b1), p3 = __floats2bfloat162_rn(b2, b3);
+                        if (to >= 0) {  // (rows past the last have no place either)
+                            __nv_bfloat16* dst = out + to + c + piece * 4;
+                            *reinterpret_cast<uint2*>(dst) =
+                                make_uint2(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1));
+                            *reinterpret_cast<uint2*>(dst + half) =
+                                make_uint2(*reinterpret_cast<const uint32_t*>(&p2), *reinterpret_cast<const uint32_t*>(&p3));
+                        }
+                    }
+                }
+                tc_fence_before();
             }
-            tc_fence_before();
         }
     }
     __syncthreads();
