@@ -5,10 +5,10 @@
 // logits[r, v] = sum_h hidden[r, h] * weight[v, h] is a dense contraction: bf16 operands on the tcgen05 tensor cores, f32
 // accumulators in tensor memory.  One persistent CTA per SM walks over 128-token tiles of the vocabulary (tile = CTA index,
 // + grid size, ...): every weight tile leaves HBM once and meets all rows (up to 256: two 128-row accumulators side by
-// side on one weight stream); the hidden states (a few MB) are re-read from L2.  Roles: warps 0 and 6 request weight
+// side on one weight stream); the hidden states (a few MB) are re-read from L2.  Roles: warps 0 and 2 request weight
 // and hidden-state tiles by TMA (64-element K slices, 128-byte swizzle, a ring of 192 KB cut into 4 to 12 stages), warp 1 issues the products and commits them to the
-// ring's "empty" barriers and to the accumulator's "full" barrier, warps 2-5 read a finished accumulator (one row per
-// thread), keep the running (maximum, first token that reaches it) per row across the CTA's tiles while the next tile's
+// ring's "empty" barriers and to the accumulator's "full" barrier, warps 4-11 read a finished accumulator (one row per
+// thread, every other run of 32 columns), keep the best (logit, token) of the row across the CTA's tiles while the next tile's
 // products fill the other accumulator.  A second small kernel merges the CTAs' candidates per row (greater logit, then
 // lower token).  Every wait on a barrier is bounded; a CTA that gives up waits for what it set in motion, frees its
 // tensor memory and flags the call.
@@ -28,7 +28,9 @@ using namespace tcp;
 constexpr int kLmBM = 128;        // rows per accumulator (tensor-memory lanes)
 constexpr int kLmBK = 64;         // hidden elements per stage (one 128-byte swizzled row)
 constexpr int kLmTileBytes = kLmBM * kLmBK * 2;  // 16 KB: one 128 x 64 bf16 operand tile
-constexpr int kLmThreads = 224;   // weight producer, issuer, four epilogue warps, hidden-state producer
+constexpr int kLmRoleWarps = 4;   // weight producer, issuer, hidden-state producer, one without a role: the epilogue warps start at a multiple of four
+constexpr int kLmEpiGroups = 2;   // epilogue warps per tensor-memory quarter (32 rows); they take every other run of 32 columns
+constexpr int kLmThreads = 32 * (kLmRoleWarps + 4 * kLmEpiGroups);
 constexpr int kLmRowsPerLaunch = 2 * kLmBM;
 constexpr int kLmMaxParts = 160;  // CTAs of a launch: one per SM, at most this many
 
@@ -82,15 +84,24 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int bn = prm.bn;
     const int n_tiles = (prm.V + bn - 1) / bn;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(FULL(s), 2), mbar_init(EMPTY(s), 1);
-        for (int b = 0; b < 2; ++b) mbar_init(ACC_FULL(b), 1), mbar_init(ACC_EMPTY(b), 4);
-        mbar_init(DRAIN, 1);
+    if (warp == 0) {
+        if (lane < S) mbar_init(FULL(lane), 2), mbar_init(EMPTY(lane), 1);
+        if (lane == S) {
+            for (int b = 0; b < 2; ++b) mbar_init(ACC_FULL(b), 1), mbar_init(ACC_EMPTY(b), 4 * kLmEpiGroups);
+            mbar_init(DRAIN, 1);
+        }
         mbar_fence_init();
-        *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
-        tma_prefetch_desc(&map_h), tma_prefetch_desc(&map_w);
+        if (lane == 0) *dead = 0, issued_s[0] = 0, issued_s[1] = 0;
+        // The first ring of weights on its way into L2 while the kernel in front still runs: a prefetch reads nothing that the copies
+        // below, which wait for that kernel, would not see anew.
+        if (elect_one()) {
+            const int first = min(S, prm.k_steps);
+            for (int ks = 0; ks < first; ++ks) tma_prefetch_2d(&map_w, ks * kLmBK, blockIdx.x * bn);
+        }
+        __syncwarp();
     }
     if (warp == 1) tmem_alloc(smem_u32(const_cast<int*>(tmem_slot)), Cfg::kTmemCols);
+    if (warp == 2 && lane == 0) tma_prefetch_desc(&map_h);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -101,10 +112,10 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
 
     // Producers and issuer are one elected thread each, with addresses and descriptors stepped from slice to slice: such a
     // thread's instructions per slice are time the stream waits, so the two operands have a producer each.
-    if (warp == 0 || warp == 6) {
-        // ================= producers: weight tiles (warp 0) and hidden-state tiles (warp 6) into the ring =================
+    if (warp == 0 || warp == 2) {
+        // ================= producers: weight tiles (warp 0) and hidden-state tiles (warp 2) into the ring =================
         if (elect_one()) {
-            const bool states = warp == 6;
+            const bool states = warp == 2;
             const int tx = states ? NM * a_bytes : stage_bytes - NM * a_bytes;
             int fill = 0, s = 0;
             uint32_t ph = 1, at = base + (states ? 0 : NM * a_bytes);  // the ring pass's parity; the stage's address
@@ -162,9 +173,9 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
             }
         }
         __syncwarp();
-    } else {
-        // ================= epilogue: running (maximum, first token) per row over this CTA's tiles =================
-        const int q = warp & 3;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
+    } else if (warp >= kLmRoleWarps) {
+        // ================= epilogue: the row's best (logit, token) over this CTA's tiles =================
+        const int q = warp & 3, grp = (warp - kLmRoleWarps) >> 2;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
         float best_v[NM][KT];  // the KT best of the row so far, best first; equal logits: the lower token first
         int best_t[NM][KT];
 #pragma unroll
@@ -175,79 +186,103 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
         bool ok = true;
         for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++it) {
             const int buf = it & 1;
-            ok = mbar_wait(ACC_FULL(buf), (it >> 1) & 1, dead);
-            ok = __all_sync(0xffffffffu, ok);
+            if (lane == 0) ok = mbar_wait(ACC_FULL(buf), (it >> 1) & 1, dead);
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
             tc_fence_after();
-            const int col0 = tile * bn;
+            const int col0 = tile * bn, n_cols = min(bn, prm.V - col0);
 #pragma unroll
             for (int t = 0; t < NM; ++t) {
-#pragma unroll
-                for (int c = 0; c < Cfg::kMaxBN / 32; ++c) {
-                    if (c * 32 >= bn) break;
+                if (t * kLmBM + q * 32 >= prm.rows) break;  // none of this warp's rows exists
+                const bool mine = t * kLmBM + q * 32 + lane < prm.rows;  // (the accumulator holds whatever lay behind the last row's states)
+                for (int c = grp * 32; c < n_cols; c += 32 * kLmEpiGroups) {
                     uint32_t r[32];
-                    tmem_ld32(TM(buf, t) + ((uint32_t)(q * 32) << 16) + c * 32, r);
+                    __syncwarp();  // (the lanes take different ways through a run; the load is warp-wide)
+                    tmem_ld32(TM(buf, t) + ((uint32_t)(q * 32) << 16) + c, r);
                     tmem_wait_ld();
-                    if (KT == 1) {
-                        // one candidate per row: compare and keep (tokens ascend within a CTA and the comparison is strict:
-                        // of equal logits the lower token stays)
-                        // (most runs of 32 hold nothing above the row's maximum so far: one maximum over the run settles that)
-                        float run_max = -INFINITY;
+                    if (n_cols - c < 32) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j)
-                            if (col0 + c * 32 + j < prm.V) run_max = fmaxf(run_max, __uint_as_float(r[j]));
-                        if (run_max > best_v[t][0]) {
+                            if (c + j >= n_cols) r[j] = 0xff800000u;  // -inf: past the vocabulary, never enters
+                    }
+                    // The run's maximum enters the list if it beats the list's last entry, then the maximum of the rest, at most KT
+                    // times; most runs hold nothing any more.  Of equal logits the lower token comes first and stays ahead (tokens
+                    // ascend within a warp and the comparisons are strict); NaN never enters.  All from registers, 32 independent
+                    // steps at a time.  (A bit per candidate and the values by run-time index, from local memory: the first run, all
+                    // of whose 32 bits are set, took 1.7 us.)
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const float v = __uint_as_float(r[j]);
-                                const int col = col0 + c * 32 + j;
-                                if (col < prm.V && v > best_v[t][0]) best_v[t][0] = v, best_t[t][0] = col;
-                            }
-                        }
-                    } else {
-                        // a ranked list per row: which of the 32 logits beat the list's last entry is one bit each; only
-                        // those (a few per run once the list has settled) are looked at again, in token order, and enter by
-                        // strict comparisons, so that of equal logits the lower token stays ahead.  NaN and columns past
-                        // the vocabulary never enter.  (The values are indexed by a run-time bit position: the compiler
-                        // keeps this copy in local memory, which the L1 serves.)
-                        float lv[32];
-                        uint32_t m = 0;
+                    for (int round = 0; round < KT; ++round) {
+                        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            lv[j] = __uint_as_float(r[j]);
-                            m |= (col0 + c * 32 + j < prm.V && lv[j] > best_v[t][KT - 1]) ? (1u << j) : 0u;
-                        }
-                        while (m) {
-                            const int j = __ffs(m) - 1;
-                            m &= m - 1;
-                            const float v = lv[j];
-                            if (v > best_v[t][KT - 1]) {
-                                best_v[t][KT - 1] = v, best_t[t][KT - 1] = col0 + c * 32 + j;
+                        for (int j = 0; j < 32; ++j) mx[j & 3] = fmaxf(mx[j & 3], __uint_as_float(r[j]));
+                        const float v = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                        const bool enters = mine && v > best_v[t][KT - 1];
+                        if (!__any_sync(0xffffffffu, enters)) break;
+                        uint32_t at = 0;
 #pragma unroll
-                                for (int jj = KT - 1; jj > 0; --jj)
-                                    if (best_v[t][jj] > best_v[t][jj - 1]) {
-                                        const float fv = best_v[t][jj];
-                                        best_v[t][jj] = best_v[t][jj - 1], best_v[t][jj - 1] = fv;
-                                        const int ft = best_t[t][jj];
-                                        best_t[t][jj] = best_t[t][jj - 1], best_t[t][jj - 1] = ft;
-                                    }
-                            }
+                        for (int j = 0; j < 32; ++j) at |= __uint_as_float(r[j]) == v ? 1u << j : 0u;
+                        const int j_max = __ffs(at) - 1;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            if (j == j_max) r[j] = 0xff800000u;
+                        if (enters) {
+                            best_v[t][KT - 1] = v, best_t[t][KT - 1] = col0 + c + j_max;
+#pragma unroll
+                            for (int jj = KT - 1; jj > 0; --jj)
+                                if (best_v[t][jj] > best_v[t][jj - 1]) {
+                                    const float fv = best_v[t][jj];
+                                    best_v[t][jj] = best_v[t][jj - 1], best_v[t][jj - 1] = fv;
+                                    const int ft = best_t[t][jj];
+                                    best_t[t][jj] = best_t[t][jj - 1], best_t[t][jj - 1] = ft;
+                                }
                         }
                     }
-                    __syncwarp();  // the lanes took different ways through the run; the next tensor-memory load is warp-wide
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(ACC_EMPTY(buf));
         }
+        // The groups' lists of a row become one: the second group leaves its own in shared memory (in the ring, which nothing uses
+        // any more once every group is through the last tile), the first one takes its entries in.  (A group that gave up a wait
+        // leaves the lists as they are; the call is flagged.)
+        float* left_v = reinterpret_cast<float*>(gen);
+        int* left_t = reinterpret_cast<int*>(gen) + NM * kLmBM * KT;
+        named_bar_sync(1, 128 * kLmEpiGroups);
+        const bool whole = !*dead;  // (nothing of the ring is in flight then)
+        const int row = q * 32 + lane;
+        if (grp == 1 && whole) {
 #pragma unroll
-        for (int t = 0; t < NM; ++t) {
-            const int r = t * kLmBM + q * 32 + lane;
+            for (int t = 0; t < NM; ++t)
 #pragma unroll
-            for (int j = 0; j < KT; ++j) {
-                prm.part_v[((size_t)r * kLmMaxParts + blockIdx.x) * KT + j] = best_v[t][j];
-                prm.part_t[((size_t)r * kLmMaxParts + blockIdx.x) * KT + j] = best_t[t][j];
+                for (int j = 0; j < KT; ++j)
+                    left_v[(t * KT + j) * kLmBM + row] = best_v[t][j], left_t[(t * KT + j) * kLmBM + row] = best_t[t][j];
+        }
+        named_bar_sync(1, 128 * kLmEpiGroups);
+        if (grp == 0) {
+#pragma unroll
+            for (int t = 0; t < NM; ++t) {
+                const int r = t * kLmBM + row;
+                if (r >= prm.rows) break;
+                if (whole) {
+#pragma unroll
+                    for (int j = 0; j < KT; ++j) {
+                        float v = left_v[(t * KT + j) * kLmBM + row];
+                        int tk = left_t[(t * KT + j) * kLmBM + row];
+#pragma unroll
+                        for (int jj = 0; jj < KT; ++jj) {  // sinks to its place: greater logit first, then the lower token
+                            const bool ahead = v > best_v[t][jj] || (v == best_v[t][jj] && tk < best_t[t][jj]);
+                            const float fv = best_v[t][jj];
+                            const int ft = best_t[t][jj];
+                            if (ahead) best_v[t][jj] = v, best_t[t][jj] = tk, v = fv, tk = ft;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < KT; ++j) {
+                    prm.part_v[((size_t)r * kLmMaxParts + blockIdx.x) * KT + j] = best_v[t][j];
+                    prm.part_t[((size_t)r * kLmMaxParts + blockIdx.x) * KT + j] = best_t[t][j];
+                }
             }
         }
     }
