@@ -5,8 +5,7 @@
 // so K/V stream from HBM once per KV head (NM = 2 covers G*T up to 256 rows, the GQA case, with one pass).
 // Warp-specialised:
 //   warp 0        TMA producer: Q once, then K and V tiles of 64 slots into 128B-swizzled shared-memory rings
-//   next NM + 1   MMA issuers (the loops run warp-uniformly, so that descriptors stay in uniform registers; an
-//                 elected lane issues): one QK issuer warp per row tile sends S = Q K^T (tcgen05.mma kind::f16,
+//   next NM + 1   MMA issuers (an elected lane issues; see kOneIssuer for who runs the loop): one QK issuer warp per row tile sends S = Q K^T (tcgen05.mma kind::f16,
 //                 M128 N64 K16 x d/16) into one of the TMEM score buffers of its row tile, one PV issuer warp sends
 //                 O += P V (M128 N=d K16 x 4, P read from tensor memory) into each row tile's TMEM accumulator;
 //                 warp 1 owns the TMEM allocation
@@ -449,6 +448,13 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     constexpr int XS = Cfg::kXRowBytes;
     constexpr int RB = kBM / REP;  // rows per copy
     constexpr int CW = kBN / REP;  // columns of a tile per copy
+    // Who issues the products.  Rows without copies (65 and more): one elected thread of the issuing warp runs its loop, with descriptors
+    // stepped from tile to tile -- the loop turns in 750 cycles, most of them the tensor pipe's (QK 384 + PV 256 per tile); run by the
+    // whole warp, all lanes polling and the leader issuing, it took 1000, and that was the rate of a sequence whose neighbours are done
+    // (16 x 8 pairs of 104 rows, lengths 1000 to 2000: 26.4 -> 25.3 us; two row tiles, L = 4096: 26.8 -> 26.6).  Row copies: the whole
+    // warp runs the loop, descriptors in uniform registers -- the products of a tile go out faster, and a launch of few tiles ends
+    // earlier (40 heads of 26 rows, L = 2048: 13.0 against 13.4 us; 32 heads, L = 1024: 9.36 against 9.46).
+    constexpr bool kOneIssuer = REP == 1;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128B swizzle atoms need 1024-byte alignment
@@ -621,75 +627,152 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     } else if (warp <= NM) {
         // ================= QK issuer of row tile t: S = Q K^T =================
         // (one issuing warp per product and row tile: a single thread spends more time issuing a tile's
-        //  instructions and polling its barriers than the tile takes to arrive; the whole warp runs the loop so
-        //  that the descriptor arithmetic is warp-uniform, one elected lane issues)
+        //  instructions and polling its barriers than the tile takes to arrive; see kOneIssuer for who issues)
         const int t = warp - 1;
-        if (nt > 0 && t < nm_act) {
-            constexpr uint32_t idesc_qk = instr_desc_bf16(kBM, kBN, false);
-            uint64_t a_desc[D / 16];  // the Q operand never moves: one descriptor per K step, made once
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)  // 64-element halves along d, 32 bytes per K step inside a half
-                a_desc[kk] = smem_desc_sw128(sQ + t * Cfg::kQBytes + (kk >> 2) * (kBM * 128) + (kk & 3) * 32, 16, 1024);
-            // `ok` is this lane's own record: once one of its waits has been given up it never issues again.  (The lanes
-            // poll on their own and need not agree at the moment of giving up; the elected lane acts on what it saw
-            // itself, and every later wait of every lane ends at once.)
-            bool ok = mbar_wait(BAR(Q_FULL), 0, dead, limit);
-            for (int j = 0; j < nt; ++j) {
-                const int s = j % S, it = j / S;
-                ok &= mbar_wait(BAR(K_FULL + s), it & 1, dead, limit);
-                const uint64_t k_desc = smem_desc_sw128(sK + s * Cfg::kTileBytes, 16, 1024);
-                ok &= mbar_wait(S_EMPTY(t, j % NB), ((j / NB) & 1) ^ 1, dead, limit);
-                tc_fence_after();
-                if (elect_one() && ok) {
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)  // the start-address field counts 16-byte units
-                        tc_mma_bf16(TM_S(t, j % NB), a_desc[kk], k_desc + (uint64_t)(((kk >> 2) * (kBN * 128) + (kk & 3) * 32) >> 4),
-                                    idesc_qk, kk > 0 ? 1u : 0u);
+        if constexpr (kOneIssuer) {
+            if (nt > 0 && t < nm_act && elect_one()) {
+                constexpr uint32_t idesc_qk = instr_desc_bf16(kBM, kBN, false);
+                constexpr uint64_t kStep = Cfg::kTileBytes >> 4;  // the start-address field counts 16-byte units
+                const uint64_t q_desc = smem_desc_sw128(sQ + t * Cfg::kQBytes, 16, 1024), k_first = smem_desc_sw128(sK, 16, 1024);
+                uint64_t k_desc = k_first;
+                uint32_t ph = 0;  // the ring pass's parity
+                int s = 0;
+                bool ok = mbar_wait(BAR(Q_FULL), 0, dead, limit);
+                for (int j = 0; j < nt && ok; ++j) {
+                    ok = mbar_wait(BAR(K_FULL + s), ph, dead, limit) && mbar_wait(S_EMPTY(t, j % NB), ((j / NB) & 1) ^ 1, dead, limit);
+                    if (!ok) break;
+                    tc_fence_after();
+    #pragma unroll
+                    for (int kk = 0; kk < D / 16; ++kk)  // 64-element halves along d, 32 bytes per K step inside a half
+                        tc_mma_bf16(TM_S(t, j % NB), q_desc + (uint64_t)(((kk >> 2) * (kBM * 128) + (kk & 3) * 32) >> 4),
+                                    k_desc + (uint64_t)(((kk >> 2) * (kBN * 128) + (kk & 3) * 32) >> 4), idesc_qk, kk > 0 ? 1u : 0u);
                     tc_commit(S_FULL(t, j % NB));
                     tc_commit(BAR(K_EMPTY + s));
+                    k_desc += kStep;
+                    if (++s == S) s = 0, ph ^= 1, k_desc = k_first;
                 }
-                __syncwarp();
+            }
+            __syncwarp();
+        } else {
+            if (nt > 0 && t < nm_act) {
+                constexpr uint32_t idesc_qk = instr_desc_bf16(kBM, kBN, false);
+                uint64_t a_desc[D / 16];  // the Q operand never moves: one descriptor per K step, made once
+    #pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk)  // 64-element halves along d, 32 bytes per K step inside a half
+                    a_desc[kk] = smem_desc_sw128(sQ + t * Cfg::kQBytes + (kk >> 2) * (kBM * 128) + (kk & 3) * 32, 16, 1024);
+                // `ok` is this lane's own record: once one of its waits has been given up it never issues again.  (The lanes
+                // poll on their own and need not agree at the moment of giving up; the elected lane acts on what it saw
+                // itself, and every later wait of every lane ends at once.)
+                bool ok = mbar_wait(BAR(Q_FULL), 0, dead, limit);
+                for (int j = 0; j < nt; ++j) {
+                    const int s = j % S, it = j / S;
+                    ok &= mbar_wait(BAR(K_FULL + s), it & 1, dead, limit);
+                    const uint64_t k_desc = smem_desc_sw128(sK + s * Cfg::kTileBytes, 16, 1024);
+                    ok &= mbar_wait(S_EMPTY(t, j % NB), ((j / NB) & 1) ^ 1, dead, limit);
+                    tc_fence_after();
+                    if (elect_one() && ok) {
+    #pragma unroll
+                        for (int kk = 0; kk < D / 16; ++kk)  // the start-address field counts 16-byte units
+                            tc_mma_bf16(TM_S(t, j % NB), a_desc[kk], k_desc + (uint64_t)(((kk >> 2) * (kBN * 128) + (kk & 3) * 32) >> 4),
+                                        idesc_qk, kk > 0 ? 1u : 0u);
+                        tc_commit(S_FULL(t, j % NB));
+                        tc_commit(BAR(K_EMPTY + s));
+                    }
+                    __syncwarp();
+                }
             }
         }
     } else if (warp == NM + 1) {
         // ================= PV issuer: O += P V, for every row tile in turn =================
         // (the row tiles' softmax groups finish a tile one after the other, so one warp serves them in that order)
-        if (nt > 0) {
+        if constexpr (kOneIssuer) {
             constexpr uint32_t idesc_pv = instr_desc_bf16(kBM, D, true);
-            bool ok = true;  // this lane's own record, as in the QK issuer
-            for (int j = 0; j < nt; ++j) {
-                const int s = j % S, it = j / S;
-                ok &= mbar_wait(BAR(V_FULL + s), it & 1, dead, limit);
-                if ((t0 + j) * kBN + kBN > Ltot) {
-                    // last, partial tile of the sequence: rows past the end may hold anything (even NaN); P is 0 there
-                    // but 0 * NaN would poison O, so those V rows are cleared before the product reads them -- here, by
-                    // the warp that waits for P anyway
-                    const int first = Ltot - (t0 + j) * kBN;  // 1..63
-                    unsigned char* vt = base_ptr + (sV - base) + s * Cfg::kTileBytes;
-                    constexpr int CPR = 8 * NH;  // 16-byte chunks per slot: a lane keeps its chunk and walks down the slots
-                    for (int r = first + lane / CPR; r < kBN; r += 32 / CPR)
-                        *reinterpret_cast<uint4*>(vt + ((lane % CPR) >> 3) * (kBN * 128) + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
-                    fence_async_smem();  // generic-proxy stores, read by the tensor core through the async proxy
-                    __syncwarp();
-                }
+            // the products of tile j with the V tile in slot s, by one thread; false: a wait was given up, nothing further is issued
+            auto issue = [&](int j, int s) -> bool {
                 // B = V [64 slots][d], MN-major: 16 slots (K step) = 2048 bytes; d halves kBN*128 bytes apart
                 const uint64_t v_desc = smem_desc_sw128(sV + s * Cfg::kTileBytes, kBN * 128, 1024);
-#pragma unroll
+    #pragma unroll
                 for (int t = 0; t < NM; ++t) {
                     if (t >= nm_act) break;
-                    ok &= mbar_wait(P_FULL(t, j % NB), (j / NB) & 1, dead, limit);
+                    if (!mbar_wait(P_FULL(t, j % NB), (j / NB) & 1, dead, limit)) return false;
                     tc_fence_after();
-                    if (elect_one() && ok) {
-#pragma unroll
-                        for (int kk = 0; kk < kBN / 16; ++kk)
-                            // A = P in tensor memory, over the first 32 columns of the score buffer: 8 columns per K step
-                            tc_mma_bf16_ts(TM_O(t, TC == 2 ? (j & 1) : 0), TM_S(t, j % NB) + kk * 8, v_desc + (uint64_t)((kk * 2048) >> 4),
-                                           idesc_pv, (j >= TC || kk > 0) ? 1u : 0u);
-                        tc_commit(PV_DONE(t, TC == 2 ? (j & 1) : 0));
-                        tc_commit(S_EMPTY(t, j % NB));  // the score buffer (and the P inside it) may be overwritten
-                        tc_commit(BAR(V_EMPTY + s));    // (one arrival per row tile)
+    #pragma unroll
+                    for (int kk = 0; kk < kBN / 16; ++kk)
+                        // A = P in tensor memory, over the first 32 columns of the score buffer: 8 columns per K step
+                        tc_mma_bf16_ts(TM_O(t, TC == 2 ? (j & 1) : 0), TM_S(t, j % NB) + kk * 8, v_desc + (uint64_t)((kk * 2048) >> 4), idesc_pv,
+                                       (j >= TC || kk > 0) ? 1u : 0u);
+                    tc_commit(PV_DONE(t, TC == 2 ? (j & 1) : 0));
+                    tc_commit(S_EMPTY(t, j % NB));  // the score buffer (and the P inside it) may be overwritten
+                    tc_commit(BAR(V_EMPTY + s));    // (one arrival per row tile)
+                }
+                return true;
+            };
+            const bool short_end = nt > 0 && t1 * kBN > Ltot;  // the last tile is the sequence's last, partial one
+            const int n_whole = nt - (short_end ? 1 : 0);
+            int ok = 1;
+            if (n_whole > 0 && elect_one()) {
+                uint32_t ph = 0;
+                int s = 0;
+                for (int j = 0; j < n_whole && ok; ++j) {
+                    ok = mbar_wait(BAR(V_FULL + s), ph, dead, limit) && issue(j, s);
+                    if (++s == S) s = 0, ph ^= 1;
+                }
+            }
+            ok = __all_sync(0xffffffffu, ok);
+            if (short_end && ok) {
+                const int j = nt - 1, s = j % S;
+                ok = mbar_wait(BAR(V_FULL + s), (j / S) & 1, dead, limit);
+                // rows past the end may hold anything (even NaN); P is 0 there but 0 * NaN would poison O, so those V rows are cleared
+                // before the product reads them -- here, by the warp that waits for P anyway
+                const int first = Ltot - (t0 + j) * kBN;  // 1..63
+                unsigned char* vt = base_ptr + (sV - base) + s * Cfg::kTileBytes;
+                constexpr int CPR = 8 * NH;  // 16-byte chunks per slot: a lane keeps its chunk and walks down the slots
+                if (ok)
+                    for (int r = first + lane / CPR; r < kBN; r += 32 / CPR)
+                        *reinterpret_cast<uint4*>(vt + ((lane % CPR) >> 3) * (kBN * 128) + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
+                fence_async_smem();  // generic-proxy stores, read by the tensor core through the async proxy
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok && elect_one()) issue(j, s);
+            }
+            __syncwarp();
+        } else {
+            if (nt > 0) {
+                constexpr uint32_t idesc_pv = instr_desc_bf16(kBM, D, true);
+                bool ok = true;  // this lane's own record, as in the QK issuer
+                for (int j = 0; j < nt; ++j) {
+                    const int s = j % S, it = j / S;
+                    ok &= mbar_wait(BAR(V_FULL + s), it & 1, dead, limit);
+                    if ((t0 + j) * kBN + kBN > Ltot) {
+                        // last, partial tile of the sequence: rows past the end may hold anything (even NaN); P is 0 there
+                        // but 0 * NaN would poison O, so those V rows are cleared before the product reads them -- here, by
+                        // the warp that waits for P anyway
+                        const int first = Ltot - (t0 + j) * kBN;  // 1..63
+                        unsigned char* vt = base_ptr + (sV - base) + s * Cfg::kTileBytes;
+                        constexpr int CPR = 8 * NH;  // 16-byte chunks per slot: a lane keeps its chunk and walks down the slots
+                        for (int r = first + lane / CPR; r < kBN; r += 32 / CPR)
+                            *reinterpret_cast<uint4*>(vt + ((lane % CPR) >> 3) * (kBN * 128) + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
+                        fence_async_smem();  // generic-proxy stores, read by the tensor core through the async proxy
+                        __syncwarp();
                     }
-                    __syncwarp();
+                    // B = V [64 slots][d], MN-major: 16 slots (K step) = 2048 bytes; d halves kBN*128 bytes apart
+                    const uint64_t v_desc = smem_desc_sw128(sV + s * Cfg::kTileBytes, kBN * 128, 1024);
+    #pragma unroll
+                    for (int t = 0; t < NM; ++t) {
+                        if (t >= nm_act) break;
+                        ok &= mbar_wait(P_FULL(t, j % NB), (j / NB) & 1, dead, limit);
+                        tc_fence_after();
+                        if (elect_one() && ok) {
+    #pragma unroll
+                            for (int kk = 0; kk < kBN / 16; ++kk)
+                                // A = P in tensor memory, over the first 32 columns of the score buffer: 8 columns per K step
+                                tc_mma_bf16_ts(TM_O(t, TC == 2 ? (j & 1) : 0), TM_S(t, j % NB) + kk * 8, v_desc + (uint64_t)((kk * 2048) >> 4),
+                                               idesc_pv, (j >= TC || kk > 0) ? 1u : 0u);
+                            tc_commit(PV_DONE(t, TC == 2 ? (j & 1) : 0));
+                            tc_commit(S_EMPTY(t, j % NB));  // the score buffer (and the P inside it) may be overwritten
+                            tc_commit(BAR(V_EMPTY + s));    // (one arrival per row tile)
+                        }
+                        __syncwarp();
+                    }
                 }
             }
         }
