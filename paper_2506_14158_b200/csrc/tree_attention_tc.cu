@@ -611,14 +611,25 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             __syncwarp();
             if (lane == 0) {
                 int issued = nt < S ? nt : S;
-                // (paged: the page of the next tile is looked up before this tile's ring slot is waited for)
-                int page_next = (paged && issued < nt) ? fetch_page(t0 + issued) : 0, page_after = 0;
-                if (paged && issued + 1 < nt) page_after = fetch_page(t0 + issued + 1);
-                for (; issued < nt; ++issued) {  // table entries are fetched two tiles ahead and looked at when needed
-                    const int page = paged ? check_page(page_next) : 0;
-                    page_next = page_after;
-                    if (paged && issued + 2 < nt) page_after = fetch_page(t0 + issued + 2);
-                    if (!load_tile(issued, paged ? paged_row(t0 + issued, page) : kv_row0 + (t0 + issued) * kBN)) break;
+                if (!paged) {
+                    for (; issued < nt; ++issued)
+                        if (!load_tile(issued, kv_row0 + (t0 + issued) * kBN)) break;
+                } else if (issued < nt) {
+                    // pages are counted off tile by tile (two divisions a tile otherwise); table entries are fetched two pages ahead
+                    // and looked at when needed
+                    const int per = prm.page_tiles, last = (t1 - 1) / per;
+                    int block = (t0 + issued) / per, at = t0 + issued - block * per;  // the tile's page of the sequence, its place in the page
+                    const int32_t* table = prm.block_table + (size_t)b * prm.max_blocks;
+                    auto fetch = [&](int i) -> int { return i <= last ? __ldg(table + i) : 0; };
+                    int page = fetch(block), page_next = fetch(block + 1), page_after = fetch(block + 2);
+                    page = check_page(page);
+                    for (; issued < nt; ++issued) {
+                        if (!load_tile(issued, ((page * prm.Hkv + hk) * per + at) * kBN)) break;
+                        if (++at == per && issued + 1 < nt) {
+                            at = 0, ++block;
+                            page = check_page(page_next), page_next = page_after, page_after = fetch(block + 2);
+                        }
+                    }
                 }
                 *issued_s = issued;  // tiles requested: what a CTA that gives up has to see in before it leaves
             }
