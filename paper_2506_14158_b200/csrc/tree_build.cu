@@ -7,10 +7,12 @@
 // kernels as a launch parameter.  What depends on the data is which tokens the children carry: child j of node n takes
 // the j-th most probable token of draft row n.  That is a top-k selection over the vocabulary per expanded node -- a
 // streaming pass over the draft probabilities, bound by HBM bandwidth (every row of an expanded node is read once):
-//   tree_topk_segments_kernel  grid (vocabulary segments of 4096, expanded nodes, B): the segment sits in registers;
-//                              k rounds of a warp-wide (maximum, lowest index) reduction, each round restricted to
-//                              entries that rank strictly after the previous winner, give each warp's k best, and one
-//                              warp selects the segment's k best among those the same way
+//   tree_topk_segments_kernel  grid (vocabulary segments of 4096, expanded nodes, B): the segment sits in registers; the
+//                              k-th greatest of the warps' maxima bounds the segment's k best from below, the few
+//                              entries that reach it are collected, and each finds its rank among them.  Where too many
+//                              reach it (plateaus, more children than warps) every warp first selects its own k best in k
+//                              rounds of a warp-wide (maximum, lowest index) reduction, each round restricted to entries
+//                              that rank strictly after the previous winner
 //   tree_emit_kernel           grid (B): one warp per expanded node merges the segments' candidates the same way and
 //                              writes the children's tokens; the CTA also writes parent[], position ids and n_nodes
 // Ranking is (probability descending, token index ascending): ties go to the lower index, every run gives the same tree.
@@ -26,6 +28,8 @@ constexpr int kTbThreads = 256;
 constexpr int kTbElems = 16;
 constexpr int kTbSeg = kTbThreads * kTbElems;  // 4096 probabilities per CTA
 constexpr int kMaxBranch = 16;                 // most children a node may get
+constexpr int kTbWarps = kTbThreads / 32;
+constexpr int kTbListed = kTbWarps * kMaxBranch;  // candidates of a segment that are kept for the selection
 
 struct TreeShape {  // breadth-first numbering; filled on the host
     int n;                          // nodes in use (<= T)
@@ -57,33 +61,74 @@ __device__ __forceinline__ void warp_best(float& p, int& tok) {
 }
 
 template <bool VEC>
-__global__ void __launch_bounds__(kTbThreads)
+__global__ void __launch_bounds__(kTbThreads, VEC ? 6 : 5)
 tree_topk_segments_kernel(const float* __restrict__ probs, const __grid_constant__ TreeShape shape, int T, int V,
                           int max_branch, Cand* __restrict__ cand) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (launched plainly: all that came before has ended)
     const int seg = blockIdx.x, u = shape.expanded[blockIdx.y], b = blockIdx.z;
     const int k = shape.n_child[u];
     const float* row = probs + ((size_t)b * T + u) * V;
     const int s0 = seg * kTbSeg;
     float x[kTbElems];
-    int e[kTbElems];
-#pragma unroll
-    for (int i = 0; i < kTbElems; ++i) e[i] = VEC ? s0 + ((i >> 2) * kTbThreads + threadIdx.x) * 4 + (i & 3) : s0 + i * kTbThreads + threadIdx.x;
+    // entry i's token, made anew where it is needed: sixteen registers more would halve the CTAs of an SM
+    auto tok = [&](int i) { return VEC ? s0 + ((i >> 2) * kTbThreads + (int)threadIdx.x) * 4 + (i & 3) : s0 + i * kTbThreads + (int)threadIdx.x; };
     if (VEC) {
 #pragma unroll
         for (int i = 0; i < kTbElems / 4; ++i) {
             float4 v = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if (e[4 * i] < V) v = __ldg(reinterpret_cast<const float4*>(row + e[4 * i]));  // V % 4 == 0 here
+            if (tok(4 * i) < V) v = __ldg(reinterpret_cast<const float4*>(row + tok(4 * i)));  // V % 4 == 0 here
             x[4 * i + 0] = v.x, x[4 * i + 1] = v.y, x[4 * i + 2] = v.z, x[4 * i + 3] = v.w;
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < kTbElems; ++i) x[i] = e[i] < V ? __ldg(row + e[i]) : -INFINITY;
+        for (int i = 0; i < kTbElems; ++i) x[i] = tok(i) < V ? __ldg(row + tok(i)) : -INFINITY;
     }
-    // Every warp first selects the k best of its own 512 entries (k rounds of shuffles, no CTA barrier), leaves them in
-    // shared memory, and after the one barrier warp 0 selects the segment's k best among the 8 k candidates.
-    __shared__ Cand wc[kTbThreads / 32][kMaxBranch];
+    __shared__ Cand wc[kTbListed];
+    __shared__ float top_s[kTbWarps];
+    __shared__ int listed_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    {
+    // Two operations per entry: k warps hold an entry of at least the k-th greatest warp maximum, so nothing below it is among the k
+    // best.  (k rounds over all entries, about nine instructions per entry and round, then k rounds of one warp over the candidates: the
+    // call took 57 us for 16 x 11 rows of 128256 with one to four children each, whose 90 MB take 14; with the bound 47, with ranks
+    // counted instead of rounds and six CTAs per SM 39.)
+    float mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < kTbElems; ++i) mx = fmaxf(mx, x[i]);  // (NaN never ranks, here or below)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) top_s[warp] = mx;
+    if (threadIdx.x == 0) listed_s = 0;
+    __syncthreads();
+    int n_listed = kTbListed + 1;
+    if (k <= kTbWarps) {  // (uniform over the CTA)
+        float bound = -INFINITY;  // the k-th greatest of the maxima
+#pragma unroll
+        for (int w = 0; w < kTbWarps; ++w) {
+            int above = 0;
+#pragma unroll
+            for (int v = 0; v < kTbWarps; ++v) above += top_s[v] > top_s[w] || (v < w && top_s[v] == top_s[w]) ? 1 : 0;
+            if (above == k - 1) bound = top_s[w];
+        }
+        if (bound > -INFINITY) {  // (else: entries of -inf rank as well, by their index)
+            uint32_t reach = 0;
+#pragma unroll
+            for (int i = 0; i < kTbElems; ++i) reach |= x[i] >= bound && tok(i) < V ? 1u << i : 0u;
+            if (reach) {
+                int at = atomicAdd(&listed_s, __popc(reach));
+#pragma unroll
+                for (int i = 0; i < kTbElems; ++i)
+                    if (reach >> i & 1u) {
+                        if (at < kTbListed) wc[at].p = x[i], wc[at].tok = tok(i);
+                        ++at;
+                    }
+            }
+            __syncthreads();
+            n_listed = listed_s;
+        }
+    }
+    if (n_listed > kTbListed) {
+        // every warp selects the k best of its own 512 entries (k rounds of shuffles)
+        __syncthreads();  // (nobody adds to the list any more)
         float pp = INFINITY;  // previous winner: nothing ranks before (+inf, -1)
         int pt = -1;
         for (int r = 0; r < k; ++r) {
@@ -91,32 +136,33 @@ tree_topk_segments_kernel(const float* __restrict__ probs, const __grid_constant
             int bt = INT_MAX;  // "no entry left": ranks after every real entry
 #pragma unroll
             for (int i = 0; i < kTbElems; ++i)
-                if (e[i] < V && ranks_after(x[i], e[i], pp, pt) && ranks_before(x[i], e[i], bp, bt)) bp = x[i], bt = e[i];
+                if (tok(i) < V && ranks_after(x[i], tok(i), pp, pt) && ranks_before(x[i], tok(i), bp, bt)) bp = x[i], bt = tok(i);
             warp_best(bp, bt);
             pp = bp, pt = bt;
-            if (lane == 0) wc[warp][r].p = bp, wc[warp][r].tok = bt;
+            if (lane == 0) wc[warp * k + r].p = bp, wc[warp * k + r].tok = bt;
         }
+        n_listed = kTbWarps * k;
+        __syncthreads();
     }
-    __syncthreads();
-    if (warp == 0) {
+    // A candidate's rank is the number of candidates that rank before it: a thread per candidate, no rounds.  (Fewer than k entries
+    // in the segment: (-inf, INT_MAX) in the remaining places.)
+    if (threadIdx.x < kTbListed) {
         Cand* out = cand + (((size_t)b * shape.n_expanded + blockIdx.y) * gridDim.x + seg) * max_branch;
-        constexpr int NW = kTbThreads / 32;
-        float pp = INFINITY;
-        int pt = -1;
-        for (int r = 0; r < k; ++r) {
-            float bp = -INFINITY;
-            int bt = INT_MAX;
-            for (int s = lane; s < NW * k; s += 32) {  // candidate (warp s / k, rank s % k)
-                const Cand v = wc[s / k][s % k];
-                if (v.tok != INT_MAX && ranks_after(v.p, v.tok, pp, pt) && ranks_before(v.p, v.tok, bp, bt)) bp = v.p, bt = v.tok;
-            }
-            warp_best(bp, bt);
-            pp = bp, pt = bt;
-            if (lane == 0) {  // an exhausted segment (fewer than k entries) leaves (-inf, INT_MAX) in the remaining slots
-                Cand c;
-                c.p = bt == INT_MAX ? -INFINITY : bp, c.tok = bt;
-                out[r] = c;
-            }
+        const int c = threadIdx.x;
+        Cand mine;
+        mine.p = -INFINITY, mine.tok = INT_MAX;
+        if (c < n_listed) mine = wc[c];
+        int rank = 0, entries = 0;
+        for (int j = 0; j < n_listed; ++j) {
+            const Cand v = wc[j];
+            if (v.tok == INT_MAX) continue;
+            ++entries;
+            rank += ranks_before(v.p, v.tok, mine.p, mine.tok) ? 1 : 0;
+        }
+        if (mine.tok != INT_MAX && rank < k) out[rank] = mine;
+        if (c < k && c >= entries) {
+            mine.p = -INFINITY, mine.tok = INT_MAX;
+            out[c] = mine;
         }
     }
 }
@@ -138,6 +184,9 @@ tree_emit_kernel(const Cand* __restrict__ cand, const __grid_constant__ TreeShap
         if (!used) tokens[(size_t)b * T + i] = 0;
     }
     if (threadIdx.x == 0) n_nodes[b] = shape.n;
+    // (launched dependent on the selection, whose candidates are all it waits for; without a selection, plainly)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // children's tokens: one warp per expanded node, k rounds over the segments' candidates, which the warp first brings
     // into shared memory (the rounds depend on one another: from global memory each would cost a round trip)
     __shared__ Cand stage[kEmitThreads / 32][kStageCands];
@@ -319,9 +368,17 @@ extern "C" s4c_status s4c_tree_build(const float* draft_probs, const int32_t* br
             tree_topk_segments_kernel<false><<<grid, kTbThreads, 0, stream>>>(draft_probs, shape, T, V, max_branch, cand);
         S4C_RETURN_IF_CUDA_ERROR();
     }
-    tree_emit_kernel<<<B, kEmitThreads, 0, stream>>>(cand, shape, root_token, cache_len, T, segs, max_branch, tokens, parent, position,
-                                            n_nodes);
-    S4C_RETURN_IF_CUDA_ERROR();
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(B, 1, 1), cfg.blockDim = dim3(kEmitThreads, 1, 1), cfg.stream = stream;
+    cfg.attrs = &pdl, cfg.numAttrs = shape.n_expanded > 0 ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, tree_emit_kernel, (const Cand*)cand, shape, root_token, cache_len, T, segs, max_branch, tokens, parent,
+                           position, n_nodes) != cudaSuccess) {
+        cudaGetLastError();
+        return S4C_ERR_CUDA;
+    }
     return S4C_OK;
 }
 
