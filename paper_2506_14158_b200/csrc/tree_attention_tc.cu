@@ -414,6 +414,26 @@ __device__ __forceinline__ void store_row8(__nv_bfloat16* dst, const float (&v)[
     *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
 }
 
+// The weighted sum of np <= K partials of eight columns of a row (offset and sum; the normalised values in fp16), in their order.
+template <int K>
+__device__ __forceinline__ void weigh_partials(const float2 (&ml)[K], const uint4 (&h)[K], int np, float& den, float (&num)[8]) {
+    float M = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < K; ++k) M = fmaxf(M, ml[k].x);  // (-inf past the last)
+    den = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) num[c] = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {  // partial order: the same on every run
+        if (k >= np) break;
+        const float w = exp2f(ml[k].x - M) * ml[k].y;  // the partial's share of the softmax sum
+        den += w;
+        const float2 a0 = unpack_half2(h[k].x), a1 = unpack_half2(h[k].y), a2 = unpack_half2(h[k].z), a3 = unpack_half2(h[k].w);
+        num[0] = fmaf(w, a0.x, num[0]), num[1] = fmaf(w, a0.y, num[1]), num[2] = fmaf(w, a1.x, num[2]), num[3] = fmaf(w, a1.y, num[3]);
+        num[4] = fmaf(w, a2.x, num[4]), num[5] = fmaf(w, a2.y, num[5]), num[6] = fmaf(w, a3.x, num[6]), num[7] = fmaf(w, a3.y, num[7]);
+    }
+}
+
 // Tile range of a split: tiles are dealt out as evenly as whole tiles allow, the odd ones to the FIRST splits -- the last
 // split holds the tree's own tiles, which cost more than a tile of the prefix (they are masked), and every split of a
 // cluster waits for the slowest.
@@ -825,6 +845,14 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     anc_hi |= 1ull << (u - 64);
             }
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
+        // where this thread will push its piece of a merged row: CTA r % splits, slot (r / splits) * splits + split (divided here, where
+        // the first tile is still on its way, rather than behind the last one)
+        uint32_t push_to = 0;
+        if (PUSH == 1) {
+            const int r = ((int)threadIdx.x - 32 * Cfg::kRoleWarps) % RB, o = r / splits;
+            push_to = map_to_cta(base + (uint32_t)(Cfg::kQBytes + 2 * S * Cfg::kTileBytes) + (uint32_t)((o * splits + split) * XS),
+                                 (uint32_t)(r - o * splits));
+        }
         float m = -1e30f, l = 0.f;  // m: offset in use (scaled, log2 units); never -inf so that exp2(-inf - m) = 0
         const float sc = prm.scale_log2;
         bool alive = true;  // false once this warp has seen a wait of the CTA given up
@@ -990,73 +1018,66 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 const int tid = (int)threadIdx.x - 32 * Cfg::kRoleWarps;
                 const int r = tid % RB, col0 = (tid / RB) * CPT;
                 const bool mine = r < rows_t && alive;
-                float acc[CPT], M = -INFINITY, den = 0.f;
-#pragma unroll
-                for (int k = 0; k < CPT; ++k) acc[k] = 0.f;
                 if (mine) {
-                    float2 ml[REP];
+                    float M = -INFINITY, den = 0.f, w[REP];
+#pragma unroll
+                    for (int c = 0; c < REP; ++c) M = fmaxf(M, *reinterpret_cast<const float*>(base_ptr + (size_t)(c * RB + r) * XS + 2 * D));
 #pragma unroll
                     for (int c = 0; c < REP; ++c) {
-                        ml[c] = *reinterpret_cast<const float2*>(base_ptr + (size_t)(c * RB + r) * XS + 2 * D);
-                        M = fmaxf(M, ml[c].x);
+                        const float2 ml = *reinterpret_cast<const float2*>(base_ptr + (size_t)(c * RB + r) * XS + 2 * D);
+                        w[c] = exp2f(ml.x - M) * ml.y;  // the copy's share of the softmax sum
+                        den += w[c];
                     }
+                    const float inv_den = den > 0.f ? 1.f / den : 0.f;
+                    // With no other split to merge it with, the merged partial is written as output (the steps of the merge below, with
+                    // one partial; 192 pairs of one row, two CTAs per SM, L=1024: 25.5 -> 22.4 us per launch; 320 pairs of 26 rows:
+                    // 49.9 -> 43.3); else it becomes one exchange row, pushed to the row's owner or left behind the parked copies, where
+                    // the peers will fetch it.  (A CTA that gave up a wait stores no output; every warp has passed its waits here.)
+                    const int gr = mt0 * kBM + r;
+                    const bool valid = n == T || gr % T < n;
+                    const float w1 = exp2f(M - M) * den, inv = (valid && w1 > 0.f) ? 1.f / w1 : 0.f;
+                    __nv_bfloat16* out = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + col0;
+                    const bool store_out = run && !*dead;
+                    const unsigned char* src = base_ptr + (size_t)r * XS + col0 * 2;
+                    unsigned char* xo = base_ptr + Cfg::kXBytes + (size_t)r * XS;
+#pragma unroll 1
+                    for (int k = 0; k < CPT; k += 8) {  // (as fast as unrolled, and a fraction of the code)
+                        float acc[8];
 #pragma unroll
-                    for (int c = 0; c < REP; ++c) {
-                        const float w = exp2f(ml[c].x - M) * ml[c].y;  // the copy's share of the softmax sum
-                        den += w;
-                        const unsigned char* src = base_ptr + (size_t)(c * RB + r) * XS + col0 * 2;
+                        for (int j = 0; j < 8; ++j) acc[j] = 0.f;
 #pragma unroll
-                        for (int k = 0; k < CPT; k += 8) {
-                            const uint4 v = *reinterpret_cast<const uint4*>(src + k * 2);
+                        for (int c = 0; c < REP; ++c) {
+                            const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)c * RB * XS + k * 2);
                             const float2 a0 = unpack_half2(v.x), a1 = unpack_half2(v.y), a2 = unpack_half2(v.z), a3 = unpack_half2(v.w);
-                            acc[k] = fmaf(w, a0.x, acc[k]), acc[k + 1] = fmaf(w, a0.y, acc[k + 1]);
-                            acc[k + 2] = fmaf(w, a1.x, acc[k + 2]), acc[k + 3] = fmaf(w, a1.y, acc[k + 3]);
-                            acc[k + 4] = fmaf(w, a2.x, acc[k + 4]), acc[k + 5] = fmaf(w, a2.y, acc[k + 5]);
-                            acc[k + 6] = fmaf(w, a3.x, acc[k + 6]), acc[k + 7] = fmaf(w, a3.y, acc[k + 7]);
+                            acc[0] = fmaf(w[c], a0.x, acc[0]), acc[1] = fmaf(w[c], a0.y, acc[1]);
+                            acc[2] = fmaf(w[c], a1.x, acc[2]), acc[3] = fmaf(w[c], a1.y, acc[3]);
+                            acc[4] = fmaf(w[c], a2.x, acc[4]), acc[5] = fmaf(w[c], a2.y, acc[5]);
+                            acc[6] = fmaf(w[c], a3.x, acc[6]), acc[7] = fmaf(w[c], a3.y, acc[7]);
                         }
-                    }
-                }
-                // the merged partial becomes one exchange row, straight from the registers
-                const float inv_den = den > 0.f ? 1.f / den : 0.f;
-                uint32_t hx[CPT / 2];
+                        uint32_t hx[4];
 #pragma unroll
-                for (int k = 0; k < CPT; k += 2) hx[k >> 1] = pack_half2(acc[k] * inv_den, acc[k + 1] * inv_den);
-                if (splits == 1) {
-                    // ... and, with no other split to merge it with, the output: the steps of the merge below with one partial
-                    // (192 pairs of one row, two CTAs per SM, L=1024: 25.5 -> 22.4 us per launch; 320 pairs of 26 rows: 49.9 -> 43.3)
-                    if (mine && run && !*dead) {  // (a CTA that gave up a wait stores nothing; every warp has passed its waits here)
-                        const int gr = mt0 * kBM + r;
-                        const bool valid = n == T || gr % T < n;
-                        const float w = exp2f(M - M) * den, inv = (valid && w > 0.f) ? 1.f / w : 0.f;
-                        __nv_bfloat16* dst = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + col0;
-#pragma unroll
-                        for (int k = 0; k < CPT / 2; k += 4) {
+                        for (int j = 0; j < 4; ++j) hx[j] = pack_half2(acc[2 * j] * inv_den, acc[2 * j + 1] * inv_den);
+                        if (splits == 1) {
                             float v[8];
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                const float2 a = unpack_half2(hx[k + j]);
-                                v[2 * j] = w * a.x, v[2 * j + 1] = w * a.y;
+                                const float2 a = unpack_half2(hx[j]);
+                                v[2 * j] = w1 * a.x, v[2 * j + 1] = w1 * a.y;
                             }
-                            store_row8(dst + 2 * k, v, inv);
+                            if (store_out) store_row8(out + k, v, inv);
+                        } else if (PUSH == 1) {
+                            if (run) st_cluster_u4(push_to + (uint32_t)((col0 + k) * 2), hx[0], hx[1], hx[2], hx[3]);
+                        } else {
+                            *reinterpret_cast<uint4*>(xo + (col0 + k) * 2) = make_uint4(hx[0], hx[1], hx[2], hx[3]);
                         }
                     }
-                } else if (PUSH == 1) {
-                    // ... stored to CTA r % splits, slot (r / splits) * splits + split of its receive area
-                    if (mine && run) {
-                        const uint32_t recv = base + (uint32_t)(Cfg::kQBytes + 2 * S * Cfg::kTileBytes);
-                        const uint32_t dst = map_to_cta(recv + (uint32_t)(((r / splits) * splits + split) * XS), (uint32_t)(r % splits));
-#pragma unroll
-                        for (int k = 0; k < CPT / 2; k += 4)
-                            st_cluster_u4(dst + (uint32_t)(col0 * 2 + k * 4), hx[k], hx[k + 1], hx[k + 2], hx[k + 3]);
-                        if (col0 == 0) st_cluster_f2(dst + (uint32_t)(2 * D), M, den);
+                    if (splits > 1 && col0 == 0) {
+                        if (PUSH == 1) {
+                            if (run) st_cluster_f2(push_to + (uint32_t)(2 * D), M, den);
+                        } else {
+                            *reinterpret_cast<float2*>(xo + 2 * D) = make_float2(M, den);
+                        }
                     }
-                } else if (mine) {
-                    // ... left behind the parked copies, where the peers will fetch it
-                    unsigned char* xo = base_ptr + Cfg::kXBytes + (size_t)r * XS;
-#pragma unroll
-                    for (int k = 0; k < CPT / 2; k += 4)
-                        *reinterpret_cast<uint4*>(xo + col0 * 2 + k * 4) = make_uint4(hx[k], hx[k + 1], hx[k + 2], hx[k + 3]);
-                    if (col0 == 0) *reinterpret_cast<float2*>(xo + 2 * D) = make_float2(M, den);
                 }
             }
         } else if (warp_active && run && alive) {
@@ -1112,43 +1133,39 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         const bool run = (flags | *bad_s) == 0;
         const int gave_up = *dead;  // (a CTA that gave up stores nothing; only the stores wait for this word)
         const uint32_t rank = cluster_ctarank();
-        const unsigned char* recv = base_ptr + Cfg::kQBytes + 2 * S * Cfg::kTileBytes;
-        constexpr int EPL = D / 32;
-        const int rows = rows_in(0);
-        if (run)
-            for (int k = warp; (int)rank + splits * k < rows; k += Cfg::kThreads / 32) {
-                const int lr = (int)rank + splits * k;
-                const unsigned char* prow = recv + (size_t)k * splits * XS;
-                // every lane reads all (offset, sum) pairs itself (broadcast reads of this CTA's own shared memory):
-                // no chain of shuffles between the barrier and the stores
-                float M = -INFINITY;
-                for (int i = 0; i < splits; ++i) M = fmaxf(M, *reinterpret_cast<const float*>(prow + (size_t)i * XS + 2 * D));
-                float den = 0.f, num[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int i = 0; i < splits; ++i) {  // split order: the same on every run
-                    const float2 ml = *reinterpret_cast<const float2*>(prow + (size_t)i * XS + 2 * D);
-                    const float w = exp2f(ml.x - M) * ml.y;  // the partial's share of the softmax sum
-                    den += w;
-                    const unsigned char* src = prow + (size_t)i * XS + lane * (EPL * 2);
-                    const float2 a = unpack_half2(*reinterpret_cast<const uint32_t*>(src));
-                    num[0] = fmaf(w, a.x, num[0]), num[1] = fmaf(w, a.y, num[1]);
-                    if (EPL == 4) {
-                        const float2 c = unpack_half2(*reinterpret_cast<const uint32_t*>(src + 4));
-                        num[2] = fmaf(w, c.x, num[2]), num[3] = fmaf(w, c.y, num[3]);
-                    }
+        const uint32_t recv = base + (uint32_t)(Cfg::kQBytes + 2 * S * Cfg::kTileBytes);
+        // a thread takes 16 bytes of a row's partials at a time, as in the merge below (a warp per row: 1.2 us for
+        // the 20 rows of a CTA of 40 heads x 60 rows in three splits, whose launch at L = 2048 took 14.2 us, now 13.3)
+        constexpr int CH = D / 8;
+        const int rows = rows_in(0), n_items = rows > (int)rank ? (rows - (int)rank + splits - 1) / splits * CH : 0;
+        auto merge_rows = [&](auto K_) {
+            constexpr int K = decltype(K_)::value;
+            for (int it = threadIdx.x; it < n_items; it += Cfg::kThreads) {
+                const int o = it / CH;
+                const uint32_t at = recv + (uint32_t)(o * splits * XS), col = (uint32_t)(it % CH) * 16;
+                float2 ml[K];
+                uint4 h[K];
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    ml[k] = make_float2(-INFINITY, 0.f);
+                    h[k] = make_uint4(0u, 0u, 0u, 0u);
+                    if (k < splits) ml[k] = ld_shared_f2(at + (uint32_t)(k * XS + 2 * D)), h[k] = ld_shared_u4(at + (uint32_t)(k * XS) + col);
                 }
-                const int gr = mt0 * kBM + lr;
-                const float inv = ((gr % T) < n && den > 0.f) ? 1.f / den : 0.f;
-                __nv_bfloat16* dst = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + lane * EPL;
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(num[0] * inv, num[1] * inv);
-                if (gave_up) break;
-                if (EPL == 4) {
-                    const __nv_bfloat162 h1 = __floats2bfloat162_rn(num[2] * inv, num[3] * inv);
-                    *reinterpret_cast<uint2*>(dst) =
-                        make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-                } else {
-                    *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(&h0);
-                }
+                const int gr = mt0 * kBM + (int)rank + splits * o;
+                const bool valid = n == T || gr % T < n;
+                float den, num[8];
+                weigh_partials<K>(ml, h, splits, den, num);
+                const float inv = (valid && den > 0.f) ? 1.f / den : 0.f;
+                if (!gave_up) store_row8(prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + (it % CH) * 8, num, inv);
             }
+        };
+        if (run) {
+            if (splits <= 4) {
+                merge_rows(std::integral_constant<int, 4>());
+            } else {
+                merge_rows(std::integral_constant<int, 8>());
+            }
+        }
         __syncthreads();  // warp 1 frees the tensor memory below: every warp is done
     } else if (PUSH != 2 && prm.mode == kModeCluster && !(REP > 1 && splits == 1)) {
         // ---- merge the splits (and turns): this CTA owns the output rows rank, rank + splits, ... of its row tiles.  A thread takes
@@ -1210,23 +1227,8 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int it = it0 + u * Cfg::kThreads;
-                    float M = -INFINITY, den = 0.f, num[8];
-#pragma unroll
-                    for (int k = 0; k < K; ++k) M = fmaxf(M, ml[u][k].x);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) num[c] = 0.f;
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {  // partial order: the same on every run
-                        if (k >= np) break;
-                        const float w = exp2f(ml[u][k].x - M) * ml[u][k].y;  // the partial's share of the softmax sum
-                        den += w;
-                        const float2 a0 = unpack_half2(h[u][k].x), a1 = unpack_half2(h[u][k].y), a2 = unpack_half2(h[u][k].z),
-                                     a3 = unpack_half2(h[u][k].w);
-                        num[0] = fmaf(w, a0.x, num[0]), num[1] = fmaf(w, a0.y, num[1]);
-                        num[2] = fmaf(w, a1.x, num[2]), num[3] = fmaf(w, a1.y, num[3]);
-                        num[4] = fmaf(w, a2.x, num[4]), num[5] = fmaf(w, a2.y, num[5]);
-                        num[6] = fmaf(w, a3.x, num[6]), num[7] = fmaf(w, a3.y, num[7]);
-                    }
+                    float den, num[8];
+                    weigh_partials<K>(ml[u], h[u], np, den, num);
                     if (it >= n_items || gave_up) continue;
                     const int gr = mt0 * kBM + (int)rank + splits * (it / CH);
                     const bool valid = n == T || gr % T < n;  // (rows of nodes past the tree's are zero)
