@@ -316,6 +316,7 @@ __device__ __forceinline__ void chain_eval(double p0, double q0, int v, int r, c
 constexpr int kCl = 8;             // CTAs per cluster
 constexpr int kClEpt = 16;         // row elements per thread
 constexpr int kClMaxThreads = 1024;
+constexpr int kWalkMaxCl = 16;     // most CTAs of a walk (see the launch)
 constexpr int kWalkGroup = 128;    // vocabulary entries that a warp of the walk takes at once: four per lane
 constexpr int kClMaxV = kCl * kClMaxThreads * kClEpt;
 constexpr size_t kSegStatsMinElems = (size_t)8 << 20;  // B*T*V above which the segment kernels win (measured)
@@ -512,7 +513,7 @@ struct WalkClShared {
     WalkShared w;
     double tab[32];
     double slots[2][2];  // two alternating sets of (sum a, sum b): set k is rewritten two cluster barriers later
-    double gab[2][kCl];
+    double gab[2][kWalkMaxCl];
     double tp0[S4C_MAX_T], tq0[S4C_MAX_T];  // node i's token under its parent's row: target and draft probability
     double ratio0[S4C_MAX_T];               // ... and what its test compares with while no sibling has been rejected
     uint32_t kids[S4C_MAX_T][S4C_MASK_WORDS];  // node i's children
@@ -535,6 +536,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.y, tid = threadIdx.x;
     const uint32_t rank = STOCH ? cl_rank() : 0u;
+    const int n_cl = (int)gridDim.x;  // CTAs of the cluster: 8 or 16
     const bool writer = rank == 0;  // CTA 0 writes everything except the final token, which its finder writes
     const int n = n_nodes ? n_nodes[b] : T;
     int32_t* pth = path + (size_t)b * (max_depth + 1);
@@ -652,7 +654,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
 
     // ---- speculative-sampling walk: every thread of every CTA follows the same control flow on the same scalars; only the
     //      passes over the vocabulary are split, CTA `rank` owning the entries [c0, c1).  What bounds it is a chain of a few
-    //      dependent passes over one row, each on 8 SMs: instructions per entry, code met for the first time, barriers.  So
+    //      dependent passes over one row, each on 8 or 16 SMs: instructions per entry, code met for the first time, barriers.  So
     //      there is one pass in the code, for the residual masses and for the draw; an entry stays with its thread through
     //      all passes at a node (no barrier for the kept values); a pass takes the kept p one rejection further instead of
     //      starting from the logits; siblings come from bitmasks.  Batch of 4, V = 128256, up to four passes: 82 -> 54 us;
@@ -670,7 +672,8 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
     // two values per CTA (at set[0], set[1] before the barrier) to cs.gab in every CTA, in rank order
     auto exchange = [&](double* set) {
         cl_sync();
-        if (tid < 2 * kCl) cs.gab[tid / kCl][tid % kCl] = cl_peer_f64(&set[tid / kCl], tid % kCl);
+        const int field = tid >= n_cl ? 1 : 0, from = tid - field * n_cl;
+        if (tid < 2 * n_cl) cs.gab[field][from] = cl_peer_f64(&set[field], from);
         __syncthreads();
         ++round;
     };
@@ -808,7 +811,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
             }
             exchange(set);
             double Z = 0.0, s = 0.0;
-            for (int k = 0; k < kCl; ++k) Z += cs.gab[0][k], s += cs.gab[1][k];
+            for (int k = 0; k < n_cl; ++k) Z += cs.gab[0][k], s += cs.gab[1][k];
             if (tid == 0) sh.cx[r] = x, sh.cinvZ[r] = Z > 0.0 ? 1.0 / Z : 0.0;  // (entry r has had no reader since the barriers above)
             if (tid == 32) sh.cinvs[r] = s > 0.0 ? 1.0 / s : 0.0;
             __syncthreads();
@@ -838,11 +841,11 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         exchange(set);
         double total = 0.0;
         int lastpos = 0;
-        for (int k = 0; k < kCl; ++k) total += cs.gab[0][k], lastpos = max(lastpos, (int)cs.gab[1][k]);
+        for (int k = 0; k < n_cl; ++k) total += cs.gab[0][k], lastpos = max(lastpos, (int)cs.gab[1][k]);
         const double target = (double)sh.uni[0] * total;
         double before = 0.0;  // mass of the ranks before the one that holds the crossing
         int rstar = -1;
-        for (int k = 0; k < kCl; ++k) {
+        for (int k = 0; k < n_cl; ++k) {
             if (before + cs.gab[0][k] > target) {
                 rstar = k;
                 break;
@@ -898,6 +901,36 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
         cl_sync();  // nobody leaves while a peer may still read its slots
         return;
     }
+}
+
+constexpr int kWalkWideV = 65536;  // rows from here on: 16 entries and more for each thread of 8 CTAs
+constexpr size_t kWalkState = ((sizeof(WalkClShared) + 15) / 16) * 16, kWalkSmemMax = 227 * 1024;
+
+// How many walks of 16 CTAs run at once (0: clusters of that size are not to be had here), asked of the device once: a cluster
+// of more than 8 is not portable, and clusters do not straddle GPCs.
+static int walk_wide_clusters() {
+    static int known[64] = {};  // answer + 1
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (!known[dev]) {
+        int clusters = 0;
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = kWalkMaxCl, attr.val.clusterDim.y = 1, attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kWalkMaxCl, 1, 1), cfg.blockDim = dim3(1024, 1, 1), cfg.dynamicSmemBytes = kWalkSmemMax;
+        cfg.attrs = &attr, cfg.numAttrs = 1;
+        const bool ok =
+            cudaFuncSetAttribute(accept_walk_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkSmemMax) == cudaSuccess &&
+            cudaFuncSetAttribute(accept_walk_cluster_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, accept_walk_cluster_kernel<true>, &cfg) == cudaSuccess;
+        cudaGetLastError();
+        known[dev] = (ok && clusters > 0 ? clusters : 0) + 1;
+    }
+    return known[dev] - 1;
 }
 
 }  // namespace s4c
@@ -986,22 +1019,26 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
     const NodeSummary* summary = seg_stats ? nullptr : ws.summary;
     const RowPartial* seg_row = seg_stats ? ws.row : nullptr;
     if (stoch) {
-        cfg.gridDim = dim3(kCl, B, 1);
+        // A pass over one row is what the walk consists of, so a long row goes to 16 CTAs where as many clusters of 16 run at once as
+        // there are sequences (4 x 64 rows of 128256, cold L2: the call 98 -> 88 us; 32000 entries are four for a thread of 8 CTAs
+        // already).
+        const int n_cl = V >= kWalkWideV && B <= walk_wide_clusters() ? kWalkMaxCl : kCl;
+        const int chunk = (int)round_up((size_t)ceil_div(V, n_cl), 4);
+        attr[0].val.clusterDim.x = n_cl;
+        cfg.gridDim = dim3(n_cl, B, 1);
         cfg.blockDim = dim3(1024, 1, 1);
         // room for the range's target probabilities (8 bytes per vocabulary entry of a CTA), and for its draft
         // probabilities too (4 more), next to the walk's state?
-        const size_t walk_state = ((sizeof(WalkClShared) + 15) / 16) * 16;
-        const size_t walk_smem_max = 227 * 1024;
         const size_t held = round_up((size_t)chunk, kWalkGroup);
-        const int keep = walk_state + held * 12 <= walk_smem_max ? 2 : (walk_state + held * 8 <= walk_smem_max ? 1 : 0);
-        cfg.dynamicSmemBytes = walk_state + held * (keep == 2 ? 12 : (keep == 1 ? 8 : 0));
+        const int keep = kWalkState + held * 12 <= kWalkSmemMax ? 2 : (kWalkState + held * 8 <= kWalkSmemMax ? 1 : 0);
+        cfg.dynamicSmemBytes = kWalkState + held * (keep == 2 ? 12 : (keep == 1 ? 8 : 0));
         {
             static bool configured[64] = {};  // the opt-in to more than 48 KB of dynamic shared memory is per device
             int dev = 0;
             if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return S4C_ERR_CUDA;
             if (!configured[dev]) {
                 if (cudaFuncSetAttribute(accept_walk_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)walk_smem_max) != cudaSuccess)
+                                         (int)kWalkSmemMax) != cudaSuccess)
                     return S4C_ERR_CUDA;
                 configured[dev] = true;
             }
