@@ -536,7 +536,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.y, tid = threadIdx.x;
     const uint32_t rank = STOCH ? cl_rank() : 0u;
-    const int n_cl = (int)gridDim.x;  // CTAs of the cluster: 8 or 16
+    const int n_cl = (int)gridDim.x;  // CTAs of the cluster: 1, 8 or 16
     const bool writer = rank == 0;  // CTA 0 writes everything except the final token, which its finder writes
     const int n = n_nodes ? n_nodes[b] : T;
     int32_t* pth = path + (size_t)b * (max_depth + 1);
@@ -671,9 +671,14 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
     int round = 0;  // cluster-wide exchanges so far (selects the slot set)
     // two values per CTA (at set[0], set[1] before the barrier) to cs.gab in every CTA, in rank order
     auto exchange = [&](double* set) {
-        cl_sync();
-        const int field = tid >= n_cl ? 1 : 0, from = tid - field * n_cl;
-        if (tid < 2 * n_cl) cs.gab[field][from] = cl_peer_f64(&set[field], from);
+        if (n_cl == 1) {
+            __syncthreads();
+            if (tid < 2) cs.gab[tid][0] = set[tid];
+        } else {
+            cl_sync();
+            const int field = tid >= n_cl ? 1 : 0, from = tid - field * n_cl;
+            if (tid < 2 * n_cl) cs.gab[field][from] = cl_peer_f64(&set[field], from);
+        }
         __syncthreads();
         ++round;
     };
@@ -898,7 +903,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
                 }
             }
         }
-        cl_sync();  // nobody leaves while a peer may still read its slots
+        if (n_cl > 1) cl_sync();  // nobody leaves while a peer may still read its slots
         return;
     }
 }
@@ -965,8 +970,10 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
     dim3 grid(splits, T, B);
 
     // ---- per-node statistics: row-in-registers clusters for small problems (one launch, latency-bound), vocabulary
-    //      segments of 4096 with many CTAs per SM for large ones (two launches, throughput-bound)
-    const bool seg_stats = !(vec && V <= kClMaxV) || (size_t)B * T * V > kSegStatsMinElems;
+    //      segments of 4096 with many CTAs per SM for large ones (two launches, throughput-bound).  A row that is one segment goes
+    //      that way too: there is nothing to share out over a cluster, whose four barriers are most of the time (15 rows of 1000 with
+    //      the walk by one CTA as well, see below: 16.4 -> 12.3 us).
+    const bool seg_stats = !(vec && V <= kClMaxV) || (size_t)B * T * V > kSegStatsMinElems || splits == 1;
     const int chunk = (int)round_up((size_t)ceil_div(V, kCl), 4);
     const float floor_span = kExpFloorSpan * (stoch ? temperature : 1.f);
     cudaLaunchAttribute attr[2];
@@ -1022,7 +1029,8 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
         // A pass over one row is what the walk consists of, so a long row goes to 16 CTAs where as many clusters of 16 run at once as
         // there are sequences (4 x 64 rows of 128256, cold L2: the call 98 -> 88 us; 32000 entries are four for a thread of 8 CTAs
         // already).
-        const int n_cl = V >= kWalkWideV && B <= walk_wide_clusters() ? kWalkMaxCl : kCl;
+        // Up to 4096 entries are four for a thread of one CTA, and then nothing has to be exchanged.
+        const int n_cl = splits == 1 ? 1 : (V >= kWalkWideV && B <= walk_wide_clusters() ? kWalkMaxCl : kCl);
         const int chunk = (int)round_up((size_t)ceil_div(V, n_cl), 4);
         attr[0].val.clusterDim.x = n_cl;
         cfg.gridDim = dim3(n_cl, B, 1);
