@@ -194,7 +194,9 @@ template <bool STOCH, bool VEC>
 __global__ void __launch_bounds__(kRowThreads)
 accept_rowstats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ n_nodes, int T, int V,
                        double inv_tau, float floor_span, RowPartial* __restrict__ out) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk's set-up runs beside this)
+    // (the walk's set-up runs beside this; after the wait, so that what came before this call has ended when the walk starts)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int split = blockIdx.x, node = blockIdx.y, b = blockIdx.z;
     if (n_nodes && node >= n_nodes[b]) return;
     const float* row = logits + ((size_t)b * T + node) * V;
@@ -364,7 +366,9 @@ accept_stats_cluster_kernel(const float* __restrict__ logits, const float* __res
                             const int32_t* __restrict__ tokens, const int32_t* __restrict__ parent,
                             const int32_t* __restrict__ n_nodes, int T, int V, int chunk, double inv_tau,
                             float floor_span, NodeSummary* __restrict__ out) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the walk's set-up runs beside this)
+    // (the walk's set-up runs beside this; after the wait, so that what came before this call has ended when the walk starts)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int node = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
     const int n = n_nodes ? n_nodes[b] : T;
     if (node >= n || n > T) return;  // the whole cluster leaves together: nobody is left waiting at a barrier
@@ -566,7 +570,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
             cs.tp0[i] = (double)__ldg(logits + at);  // turned into a probability below, once the parent's statistics are in
             atomicOr(&cs.kids[sh.par[i]][i >> 5], 1u << (i & 31));
         }
-    // Everything above reads the caller's inputs only, which were complete before the statistics kernel began; from here on
+    // Everything above reads the caller's inputs only, which were complete before the statistics kernel let this one start; from here on
     // its results are needed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!(flags & S4C_SEQ_BAD_PARENT)) {
@@ -981,21 +985,23 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
     attr[0].val.clusterDim.x = kCl, attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = stream;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr, cfg.numAttrs = 1;
     cudaError_t err = cudaSuccess;
     if (seg_stats) {
-        if (stoch) {
-            if (vec)
-                accept_rowstats_kernel<true, true><<<grid, kRowThreads, 0, stream>>>(target_logits, n_nodes, T, V, inv_tau, floor_span, ws.row);
-            else
-                accept_rowstats_kernel<true, false><<<grid, kRowThreads, 0, stream>>>(target_logits, n_nodes, T, V, inv_tau, floor_span, ws.row);
-        } else {
-            if (vec)
-                accept_rowstats_kernel<false, true><<<grid, kRowThreads, 0, stream>>>(target_logits, n_nodes, T, V, inv_tau, floor_span, ws.row);
-            else
-                accept_rowstats_kernel<false, false><<<grid, kRowThreads, 0, stream>>>(target_logits, n_nodes, T, V, inv_tau, floor_span, ws.row);
+        cudaLaunchConfig_t rows = {};
+        rows.gridDim = grid, rows.blockDim = dim3(kRowThreads, 1, 1), rows.stream = stream, rows.attrs = &attr[1];
+        // Dependent where a row is one segment: a small step is a chain of launches (15 rows of 1000 in a one-layer step, eager: 29.1 -> 26.0
+        // us).  With more, what overlaps is nothing beside the kernel, and its CTAs come in the way of the launch in front (four of 64 rows of
+        // 128256: 0.998x).
+        rows.numAttrs = splits == 1 ? 1 : 0;
+        auto kernel = stoch ? (vec ? accept_rowstats_kernel<true, true> : accept_rowstats_kernel<true, false>)
+                            : (vec ? accept_rowstats_kernel<false, true> : accept_rowstats_kernel<false, false>);
+        if (cudaLaunchKernelEx(&rows, kernel, target_logits, n_nodes, T, V, inv_tau, floor_span, ws.row) != cudaSuccess) {
+            cudaGetLastError();
+            return S4C_ERR_CUDA;
         }
-        S4C_RETURN_IF_CUDA_ERROR();
     } else {
         cfg.gridDim = dim3(kCl, T, B);
 #define S4C_LAUNCH_STATS(THREADS)                                                                                      \
@@ -1019,10 +1025,7 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
         }
     }
     // ---- the walk: one cluster per sequence (greedy: one CTA, no vocabulary pass), launched dependent on the statistics
-    cudaLaunchAttribute& pdl = attr[stoch ? 1 : 0];
-    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl.val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = stoch ? 2 : 1;
+    cfg.attrs = stoch ? attr : attr + 1, cfg.numAttrs = stoch ? 2 : 1;
     const NodeSummary* summary = seg_stats ? nullptr : ws.summary;
     const RowPartial* seg_row = seg_stats ? ws.row : nullptr;
     if (stoch) {
