@@ -5,9 +5,10 @@
 // so K/V stream from HBM once per KV head (NM = 2 covers G*T up to 256 rows, the GQA case, with one pass).
 // Warp-specialised:
 //   warp 0        TMA producer: Q once, then K and V tiles of 64 slots into 128B-swizzled shared-memory rings
-//   next NM + 1   MMA issuers (an elected lane issues; see kOneIssuer for who runs the loop): one QK issuer warp per row tile sends S = Q K^T (tcgen05.mma kind::f16,
-//                 M128 N64 K16 x d/16) into one of the TMEM score buffers of its row tile, one PV issuer warp sends
-//                 O += P V (M128 N=d K16 x 4, P read from tensor memory) into each row tile's TMEM accumulator;
+//   next NM + 1   MMA issuers (an elected lane issues; see kOneIssuer for who runs the loop): one QK issuer
+//                 warp per row tile sends S = Q K^T (tcgen05.mma kind::f16, M128 N64 K16 x d/16) into one of the
+//                 TMEM score buffers of its row tile, one PV issuer warp sends O += P V (M128 N=d K16 x 4, P read from
+//                 tensor memory) into each row tile's TMEM accumulator;
 //                 warp 1 owns the TMEM allocation
 //   then          one group of four warps per row tile, one thread per query row: tcgen05.ld of the scores,
 //                 tree / tail masking from the row's ancestor bitmask (built from parent[] by the thread
