@@ -192,9 +192,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant_
         const int q = warp & 3;  // the tensor-memory lanes this warp may read: 32 q .. 32 q + 31
         const int grp = (warp - kLnRoleWarps) >> 2;
         griddep_wait();  // (the residual may be the result of the kernel in front, and nothing is written before that kernel has ended)
-        bool ok = true;
-        if (lane == 0) ok = mbar_wait(ACC_FULL, 0, dead);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        const bool ok = mbar_wait_warp(ACC_FULL, 0, dead);
         if (ok) tc_fence_after();
         const uint32_t stage = base + (uint32_t)(warp - kLnRoleWarps) * 4096u;  // 32 rows x 128 bytes, 16-byte pieces XOR-swizzled
         const int w_rows = prm.gate ? 2 * prm.N : prm.N;

@@ -188,8 +188,7 @@ lm_head_greedy_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_co
         bool ok = true;
         for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++it) {
             const int buf = it & 1;
-            if (lane == 0) ok = mbar_wait(ACC_FULL(buf), (it >> 1) & 1, dead);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            ok = mbar_wait_warp(ACC_FULL(buf), (it >> 1) & 1, dead);
             if (!ok) break;
             tc_fence_after();
             const int col0 = tile * bn, n_cols = min(bn, prm.V - col0);

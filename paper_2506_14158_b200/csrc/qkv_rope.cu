@@ -215,9 +215,7 @@ qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 }
             };
             fetch(0);
-            bool ok = true;
-            if (lane == 0) ok = mbar_wait(ACC_FULL, 0, dead);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            const bool ok = mbar_wait_warp(ACC_FULL, 0, dead);
             if (ok) {
                 tc_fence_after();
                 const uint32_t stage = base + (uint32_t)(warp - kQkRoleWarps) * 8192u;  // twice 32 rows x 128 bytes, 16-byte pieces XOR-swizzled

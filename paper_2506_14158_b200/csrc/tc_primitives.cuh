@@ -50,6 +50,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         }
     }
 }
+// The same for a warp that goes on together: every lane looks at the barrier itself and so has what lies behind it before its own next
+// access (one lane's answer, handed round by a shuffle or a vote, orders no memory for the others).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* dead) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, dead));
+}
 // Wait for something this CTA itself set in motion (a bulk copy, a committed product) on the way out of a CTA that has
 // given up: bounded like every wait, but not cut short by `dead`, so that nothing is still in flight into shared or
 // tensor memory when the CTA frees them.
