@@ -661,37 +661,42 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         // (one issuing warp per product and row tile: a single thread spends more time issuing a tile's
         //  instructions and polling its barriers than the tile takes to arrive; see kOneIssuer for who issues)
         const int t = warp - 1;
-        if constexpr (kOneIssuer) {
-            if (nt > 0 && t < nm_act && elect_one()) {
-                constexpr uint32_t idesc_qk = instr_desc_bf16(kBM, kBN, false);
-                constexpr uint64_t kStep = Cfg::kTileBytes >> 4;  // the start-address field counts 16-byte units
-                const uint64_t q_desc = smem_desc_sw128(sQ + t * Cfg::kQBytes, 16, 1024), k_first = smem_desc_sw128(sK, 16, 1024);
-                uint64_t k_desc = k_first;
-                uint32_t ph = 0;  // the ring pass's parity
-                int s = 0;
-                bool ok = mbar_wait(BAR(Q_FULL), 0, dead, limit);
-                for (int j = 0; j < nt && ok; ++j) {
-                    ok = mbar_wait(BAR(K_FULL + s), ph, dead, limit) && mbar_wait(S_EMPTY(t, j % NB), ((j / NB) & 1) ^ 1, dead, limit);
-                    if (!ok) break;
-                    tc_fence_after();
-    #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)  // 64-element halves along d, 32 bytes per K step inside a half
-                        tc_mma_bf16(TM_S(t, j % NB), q_desc + (uint64_t)(((kk >> 2) * (kBM * 128) + (kk & 3) * 32) >> 4),
-                                    k_desc + (uint64_t)(((kk >> 2) * (kBN * 128) + (kk & 3) * 32) >> 4), idesc_qk, kk > 0 ? 1u : 0u);
-                    tc_commit(S_FULL(t, j % NB));
-                    tc_commit(BAR(K_EMPTY + s));
-                    k_desc += kStep;
-                    if (++s == S) s = 0, ph ^= 1, k_desc = k_first;
+        constexpr uint32_t idesc_qk = instr_desc_bf16(kBM, kBN, false);
+        const uint64_t q_first = smem_desc_sw128(sQ + t * Cfg::kQBytes, 16, 1024);
+        // operand offset of K step kk: 64-element halves along d (rows * 128 bytes each), 32 bytes per step inside a half; the
+        // descriptor's address field counts 16 bytes
+        auto k_step = [](int kk, int rows) { return (uint64_t)(((kk >> 2) * (rows * 128) + (kk & 3) * 32) >> 4); };
+        // the products of tile j with the K tile in slot s, by one thread; q_desc(kk): the Q operand of K step kk
+        auto issue = [&](int j, int s, auto q_desc, uint64_t k_desc) {
+#pragma unroll
+            for (int kk = 0; kk < D / 16; ++kk)
+                tc_mma_bf16(TM_S(t, j % NB), q_desc(kk), k_desc + k_step(kk, kBN), idesc_qk, kk > 0 ? 1u : 0u);
+            tc_commit(S_FULL(t, j % NB));
+            tc_commit(BAR(K_EMPTY + s));
+        };
+        if (nt > 0 && t < nm_act) {
+            if constexpr (kOneIssuer) {
+                if (elect_one()) {
+                    constexpr uint64_t kStep = Cfg::kTileBytes >> 4;
+                    const uint64_t k_first = smem_desc_sw128(sK, 16, 1024);
+                    uint64_t k_desc = k_first;
+                    uint32_t ph = 0;  // the ring pass's parity
+                    int s = 0;
+                    bool ok = mbar_wait(BAR(Q_FULL), 0, dead, limit);
+                    for (int j = 0; j < nt && ok; ++j) {
+                        ok = mbar_wait(BAR(K_FULL + s), ph, dead, limit) && mbar_wait(S_EMPTY(t, j % NB), ((j / NB) & 1) ^ 1, dead, limit);
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue(j, s, [&](int kk) { return q_first + k_step(kk, kBM); }, k_desc);
+                        k_desc += kStep;
+                        if (++s == S) s = 0, ph ^= 1, k_desc = k_first;
+                    }
                 }
-            }
-            __syncwarp();
-        } else {
-            if (nt > 0 && t < nm_act) {
-                constexpr uint32_t idesc_qk = instr_desc_bf16(kBM, kBN, false);
-                uint64_t a_desc[D / 16];  // the Q operand never moves: one descriptor per K step, made once
-    #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk)  // 64-element halves along d, 32 bytes per K step inside a half
-                    a_desc[kk] = smem_desc_sw128(sQ + t * Cfg::kQBytes + (kk >> 2) * (kBM * 128) + (kk & 3) * 32, 16, 1024);
+                __syncwarp();
+            } else {
+                uint64_t q_desc[D / 16];  // the Q operand never moves: one descriptor per K step, made once
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk) q_desc[kk] = q_first + k_step(kk, kBM);
                 // `ok` is this lane's own record: once one of its waits has been given up it never issues again.  (The lanes
                 // poll on their own and need not agree at the moment of giving up; the elected lane acts on what it saw
                 // itself, and every later wait of every lane ends at once.)
@@ -702,14 +707,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     const uint64_t k_desc = smem_desc_sw128(sK + s * Cfg::kTileBytes, 16, 1024);
                     ok &= mbar_wait(S_EMPTY(t, j % NB), ((j / NB) & 1) ^ 1, dead, limit);
                     tc_fence_after();
-                    if (elect_one() && ok) {
-    #pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk)  // the start-address field counts 16-byte units
-                            tc_mma_bf16(TM_S(t, j % NB), a_desc[kk], k_desc + (uint64_t)(((kk >> 2) * (kBN * 128) + (kk & 3) * 32) >> 4),
-                                        idesc_qk, kk > 0 ? 1u : 0u);
-                        tc_commit(S_FULL(t, j % NB));
-                        tc_commit(BAR(K_EMPTY + s));
-                    }
+                    if (elect_one() && ok) issue(j, s, [&](int kk) { return q_desc[kk]; }, k_desc);
                     __syncwarp();
                 }
             }
@@ -717,25 +715,42 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     } else if (warp == NM + 1) {
         // ================= PV issuer: O += P V, for every row tile in turn =================
         // (the row tiles' softmax groups finish a tile one after the other, so one warp serves them in that order)
+        constexpr uint32_t idesc_pv = instr_desc_bf16(kBM, D, true);
+        // B = V [64 slots][d], MN-major: 16 slots (K step) = 2048 bytes; d halves kBN*128 bytes apart
+        auto v_tile = [&](int s) { return smem_desc_sw128(sV + s * Cfg::kTileBytes, kBN * 128, 1024); };
+        // row tile t's products of tile j with the V tile in slot s, by one thread
+        auto issue = [&](int t, int j, int s, uint64_t v_desc) {
+#pragma unroll
+            for (int kk = 0; kk < kBN / 16; ++kk)
+                // A = P in tensor memory, over the first 32 columns of the score buffer: 8 columns per K step
+                tc_mma_bf16_ts(TM_O(t, TC == 2 ? (j & 1) : 0), TM_S(t, j % NB) + kk * 8, v_desc + (uint64_t)((kk * 2048) >> 4), idesc_pv,
+                               (j >= TC || kk > 0) ? 1u : 0u);
+            tc_commit(PV_DONE(t, TC == 2 ? (j & 1) : 0));
+            tc_commit(S_EMPTY(t, j % NB));  // the score buffer (and the P inside it) may be overwritten
+            tc_commit(BAR(V_EMPTY + s));    // (one arrival per row tile)
+        };
+        // The sequence's last, partial tile: rows past the end may hold anything (even NaN); P is 0 there but 0 * NaN would poison O,
+        // so those V rows are cleared before the product reads them -- here, by the warp that waits for P anyway.  Every lane
+        // makes its own stores visible to the tensor core; the __syncwarp behind the call puts the issuing lane behind all of
+        // them (a vote or a shuffle would not: they order no memory).
+        auto clear_v_tail = [&](int j, int s) {
+            const int first = Ltot - (t0 + j) * kBN;  // 1..63
+            unsigned char* vt = base_ptr + (sV - base) + s * Cfg::kTileBytes;
+            constexpr int CPR = 8 * NH;  // 16-byte chunks per slot: a lane keeps its chunk and walks down the slots
+            for (int r = first + lane / CPR; r < kBN; r += 32 / CPR)
+                *reinterpret_cast<uint4*>(vt + ((lane % CPR) >> 3) * (kBN * 128) + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
+            fence_async_smem();  // generic-proxy stores, read by the tensor core through the async proxy
+        };
         if constexpr (kOneIssuer) {
-            constexpr uint32_t idesc_pv = instr_desc_bf16(kBM, D, true);
-            // the products of tile j with the V tile in slot s, by one thread; false: a wait was given up, nothing further is issued
-            auto issue = [&](int j, int s) -> bool {
-                // B = V [64 slots][d], MN-major: 16 slots (K step) = 2048 bytes; d halves kBN*128 bytes apart
-                const uint64_t v_desc = smem_desc_sw128(sV + s * Cfg::kTileBytes, kBN * 128, 1024);
-    #pragma unroll
+            // all row tiles' products of tile j, by one thread; false: a wait was given up, nothing further is issued
+            auto issue_tile = [&](int j, int s) -> bool {
+                const uint64_t v_desc = v_tile(s);
+#pragma unroll
                 for (int t = 0; t < NM; ++t) {
                     if (t >= nm_act) break;
                     if (!mbar_wait(P_FULL(t, j % NB), (j / NB) & 1, dead, limit)) return false;
                     tc_fence_after();
-    #pragma unroll
-                    for (int kk = 0; kk < kBN / 16; ++kk)
-                        // A = P in tensor memory, over the first 32 columns of the score buffer: 8 columns per K step
-                        tc_mma_bf16_ts(TM_O(t, TC == 2 ? (j & 1) : 0), TM_S(t, j % NB) + kk * 8, v_desc + (uint64_t)((kk * 2048) >> 4), idesc_pv,
-                                       (j >= TC || kk > 0) ? 1u : 0u);
-                    tc_commit(PV_DONE(t, TC == 2 ? (j & 1) : 0));
-                    tc_commit(S_EMPTY(t, j % NB));  // the score buffer (and the P inside it) may be overwritten
-                    tc_commit(BAR(V_EMPTY + s));    // (one arrival per row tile)
+                    issue(t, j, s, v_desc);
                 }
                 return true;
             };
@@ -746,7 +761,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 uint32_t ph = 0;
                 int s = 0;
                 for (int j = 0; j < n_whole && ok; ++j) {
-                    ok = mbar_wait(BAR(V_FULL + s), ph, dead, limit) && issue(j, s);
+                    ok = mbar_wait(BAR(V_FULL + s), ph, dead, limit) && issue_tile(j, s);
                     if (++s == S) s = 0, ph ^= 1;
                 }
             }
@@ -754,57 +769,29 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             if (short_end && ok) {
                 const int j = nt - 1, s = j % S;
                 ok = mbar_wait(BAR(V_FULL + s), (j / S) & 1, dead, limit);
-                // rows past the end may hold anything (even NaN); P is 0 there but 0 * NaN would poison O, so those V rows are cleared
-                // before the product reads them -- here, by the warp that waits for P anyway
-                const int first = Ltot - (t0 + j) * kBN;  // 1..63
-                unsigned char* vt = base_ptr + (sV - base) + s * Cfg::kTileBytes;
-                constexpr int CPR = 8 * NH;  // 16-byte chunks per slot: a lane keeps its chunk and walks down the slots
-                if (ok)
-                    for (int r = first + lane / CPR; r < kBN; r += 32 / CPR)
-                        *reinterpret_cast<uint4*>(vt + ((lane % CPR) >> 3) * (kBN * 128) + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
-                fence_async_smem();  // generic-proxy stores, read by the tensor core through the async proxy
+                if (ok) clear_v_tail(j, s);
+                __syncwarp();
                 ok = __all_sync(0xffffffffu, ok);
-                if (ok && elect_one()) issue(j, s);
+                if (ok && elect_one()) issue_tile(j, s);
             }
             __syncwarp();
         } else {
-            if (nt > 0) {
-                constexpr uint32_t idesc_pv = instr_desc_bf16(kBM, D, true);
-                bool ok = true;  // this lane's own record, as in the QK issuer
-                for (int j = 0; j < nt; ++j) {
-                    const int s = j % S, it = j / S;
-                    ok &= mbar_wait(BAR(V_FULL + s), it & 1, dead, limit);
-                    if ((t0 + j) * kBN + kBN > Ltot) {
-                        // last, partial tile of the sequence: rows past the end may hold anything (even NaN); P is 0 there
-                        // but 0 * NaN would poison O, so those V rows are cleared before the product reads them -- here, by
-                        // the warp that waits for P anyway
-                        const int first = Ltot - (t0 + j) * kBN;  // 1..63
-                        unsigned char* vt = base_ptr + (sV - base) + s * Cfg::kTileBytes;
-                        constexpr int CPR = 8 * NH;  // 16-byte chunks per slot: a lane keeps its chunk and walks down the slots
-                        for (int r = first + lane / CPR; r < kBN; r += 32 / CPR)
-                            *reinterpret_cast<uint4*>(vt + ((lane % CPR) >> 3) * (kBN * 128) + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
-                        fence_async_smem();  // generic-proxy stores, read by the tensor core through the async proxy
-                        __syncwarp();
-                    }
-                    // B = V [64 slots][d], MN-major: 16 slots (K step) = 2048 bytes; d halves kBN*128 bytes apart
-                    const uint64_t v_desc = smem_desc_sw128(sV + s * Cfg::kTileBytes, kBN * 128, 1024);
-    #pragma unroll
-                    for (int t = 0; t < NM; ++t) {
-                        if (t >= nm_act) break;
-                        ok &= mbar_wait(P_FULL(t, j % NB), (j / NB) & 1, dead, limit);
-                        tc_fence_after();
-                        if (elect_one() && ok) {
-    #pragma unroll
-                            for (int kk = 0; kk < kBN / 16; ++kk)
-                                // A = P in tensor memory, over the first 32 columns of the score buffer: 8 columns per K step
-                                tc_mma_bf16_ts(TM_O(t, TC == 2 ? (j & 1) : 0), TM_S(t, j % NB) + kk * 8, v_desc + (uint64_t)((kk * 2048) >> 4),
-                                               idesc_pv, (j >= TC || kk > 0) ? 1u : 0u);
-                            tc_commit(PV_DONE(t, TC == 2 ? (j & 1) : 0));
-                            tc_commit(S_EMPTY(t, j % NB));  // the score buffer (and the P inside it) may be overwritten
-                            tc_commit(BAR(V_EMPTY + s));    // (one arrival per row tile)
-                        }
-                        __syncwarp();
-                    }
+            bool ok = true;  // this lane's own record, as in the QK issuer
+            for (int j = 0; j < nt; ++j) {
+                const int s = j % S, it = j / S;
+                ok &= mbar_wait(BAR(V_FULL + s), it & 1, dead, limit);
+                if ((t0 + j) * kBN + kBN > Ltot) {
+                    clear_v_tail(j, s);
+                    __syncwarp();
+                }
+                const uint64_t v_desc = v_tile(s);
+#pragma unroll
+                for (int t = 0; t < NM; ++t) {
+                    if (t >= nm_act) break;
+                    ok &= mbar_wait(P_FULL(t, j % NB), (j / NB) & 1, dead, limit);
+                    tc_fence_after();
+                    if (elect_one() && ok) issue(t, j, s, v_desc);
+                    __syncwarp();
                 }
             }
         }

@@ -59,15 +59,21 @@ def test_extreme_tree_sizes(dtype):
     _case(B=1, Hq=4, Hkv=1, T=128, d=64, Ls=[0], dtype=dtype, seed=5, tree="chain")  # no prefix at all
 
 
-@pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("Hq,Hkv,T", [(4, 4, 26), (8, 2, 64)])
-def test_slots_past_the_sequence_end_may_hold_anything(dtype, Hq, Hkv, T):
+@pytest.mark.parametrize("dtype,Hq,Hkv,T,Ls,C", [
+    ("f32", 4, 4, 26, [1000, 70], 1152), ("f32", 8, 2, 64, [1000, 70], 1152),
+    ("bf16", 4, 4, 26, [1000, 70], 1152), ("bf16", 8, 2, 64, [1000, 70], 1152),  # row copies in splits; one row tile per CTA in splits
+    ("bf16", 32, 8, 26, [1000, 70, 998, 1001] * 3, 1152),  # turns, unsplit (998 + 26 slots: whole tiles)
+    ("bf16", 32, 8, 64, [1000, 70, 1024], 1152),           # two row tiles per CTA (1024 + 64: whole tiles)
+    ("bf16", 32, 8, 26, [300, 70, 294, 1] * 5, 384),       # half-SM CTAs, one issuing thread (294 + 26: whole tiles)
+    ("bf16", 8, 8, 26, [300, 70, 294, 1] * 5, 384),        # half-SM CTAs, row copies
+])
+def test_slots_past_the_sequence_end_may_hold_anything(dtype, Hq, Hkv, T, Ls, C):
     # K/V slots at and beyond L + n are not part of the sequence: NaN or Inf there must not reach the output
     # (their scores are masked by selection, their V rows never enter the product)
     from paper_2506_14158_b200 import s4c
     from parity import dev
 
-    B, d, Ls, C = 2, 128, [1000, 70], 1152
+    B, d = len(Ls), 128
     dt = {"f32": torch.float32, "bf16": torch.bfloat16}[dtype]
     rng = np.random.default_rng(11)
     g = torch.Generator().manual_seed(11)
