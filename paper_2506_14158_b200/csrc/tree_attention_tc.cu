@@ -256,9 +256,11 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
+__device__ __forceinline__ void cluster_arrive_started() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }  // (publishes nothing)
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_wait();
 }
 __device__ __forceinline__ void st_cluster_f2(uint32_t addr, float a, float b) {
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
@@ -518,6 +520,12 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     int nm_act = 0;  // row tiles with at least one row (they are the first ones)
 #pragma unroll
     for (int t = 0; t < NM; ++t) nm_act += rows_in(t) > 0 ? 1 : 0;
+
+    // A peer's shared memory may be written only once the peer has started: every thread says so first thing, the softmax warps wait for
+    // it where their first tile is on its way, the others in front of the merge.  (Said behind the prologue it
+    // cost 0.07 us of a launch of 9.04 us; here 0.01 to 0.03.)
+    const bool pushes = PUSH == 1 && prm.mode == kModeCluster && splits > 1;
+    if (pushes) cluster_arrive_started();
 
     // ---- prologue that touches no global memory: barriers (one per lane of warp 0), TMEM, descriptor prefetch
     if (warp == 0) {
@@ -841,6 +849,10 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             push_to = map_to_cta(base + (uint32_t)(Cfg::kQBytes + 2 * S * Cfg::kTileBytes) + (uint32_t)((o * splits + split) * XS),
                                  (uint32_t)(r - o * splits));
         }
+        if (pushes) {
+            __syncwarp();  // (the lanes may have left the loop above at different times; the wait is warp-wide)
+            cluster_wait();
+        }
         float m = -1e30f, l = 0.f;  // m: offset in use (scaled, log2 units); never -inf so that exp2(-inf - m) = 0
         const float sc = prm.scale_log2;
         bool alive = true;  // false once this warp has seen a wait of the CTA given up
@@ -1114,9 +1126,10 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         tc_fence_before();
     }
 
-    if (PUSH == 1 && prm.mode == kModeCluster && splits > 1) {
+    if (pushes) {
         // ---- every split's partial of this CTA's rows (rank, rank + splits, ...) has been stored into its receive area
         __syncwarp();
+        if (warp < Cfg::kRoleWarps) cluster_wait();  // (as the softmax warps have: the barrier's first phase is over for this thread)
         cluster_sync_all();
         const bool run = (flags | *bad_s) == 0;
         const int gave_up = *dead;  // (a CTA that gave up stores nothing; only the stores wait for this word)
