@@ -664,6 +664,10 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             }
             __syncwarp();
         }
+        // Splits that do not form a cluster end in any order, and the CTA that writes status[b] must not do so over a flag that another
+        // one has raised: it looks at all of the sequence's pages itself and raises the flag behind its own store.
+        if (NM == 2 && paged && prm.mode == kModeWorkspace && split == 0 && blockIdx.y == 0 && !flags)
+            for (int g = lane * prm.page_tiles; g * kBN < Ltot; g += 32 * prm.page_tiles) lookup_page(g);
     } else if (warp <= NM) {
         // ================= QK issuer of row tile t: S = Q K^T =================
         // (one issuing warp per product and row tile: a single thread spends more time issuing a tile's

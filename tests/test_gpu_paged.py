@@ -80,6 +80,26 @@ def test_a_page_outside_the_pool_flags_the_sequence_and_touches_nothing_else():
     assert np.abs(out[:1].double().cpu().numpy() - ref).max() <= ATTN_TOL["bf16"]
 
 
+@pytest.mark.parametrize("bad", [None, 0, 100, 194])
+def test_a_page_outside_the_pool_is_flagged_where_the_splits_are_no_cluster(bad):
+    # two row tiles of one sequence on more than 24k slots: the splits meet in a workspace, and end in any order
+    from paper_2506_14158_b200 import s4c
+
+    Hq, Hkv, T, d, ps, L = 32, 8, 64, 128, 128, 24890
+    nb = (L + T + ps - 1) // ps
+    assert s4c.tree_attention_workspace_bytes(1, T, Hq, Hkv, d, nb * ps, torch.bfloat16) > 0 and nb == 195
+    g = torch.Generator(device="cuda").manual_seed(9)
+    q = torch.randn((1, Hq, T, d), generator=g, device="cuda").bfloat16()
+    kp = torch.randn((nb, Hkv, ps, d), generator=g, device="cuda").bfloat16()
+    bt = np.arange(nb, dtype=np.int32)[None].copy()
+    if bad is not None:
+        bt[0, bad] = nb
+    for _ in range(20):
+        st = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        s4c.tree_attention_paged(q, kp, kp, dev(bt), dev(np.array([L], np.int32)), dev(W.chain_tree(T)[None].copy()), status=st)
+        assert st.cpu().tolist() == [0 if bad is None else s4c.SEQ_BAD_PAGE]
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("page_size", [64, 128])
 def test_paged_compaction_is_bit_exact(dtype, page_size):
