@@ -53,8 +53,9 @@ struct LnParams {
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
 
-// (at most half the registers of an SM, as if two CTAs were to share it: the finishing kernel of one product and the CTAs of the next
-// one, which request their weights meanwhile, are resident together)
+// (at most half the registers of an SM, as if two CTAs were to share it: the finishing kernel of one product and this kernel's CTAs of
+// the next one, which request their weights meanwhile, are resident together.  Behind a down projection the next product is the q/k/v
+// kernel, whose 64512 registers a CTA leave no room beside: it starts on an SM once the finishing CTAs there have left)
 __global__ void __launch_bounds__(kLnThreads, 2)
 linear_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
               const __grid_constant__ CUtensorMap map_w, const LnParams prm) {
@@ -542,19 +543,18 @@ static bool ln_make_map(CUtensorMap* map, const void* ptr, uint64_t rows, int H,
 // small model of this kernel on this GPU and the cheapest is launched:
 //   * one CTA per SM, so CTAs run in waves of 148; a second wave of a few CTAs costs as much as a full one
 //     (7B-shaped gate/up projection: 172 tiles of 64 columns took 50 us, 138 tiles of 80 take one wave);
-//   * per K slice of 64 elements a CTA needs the longest of: the issuing thread's fixed ~0.3 us (four tcgen05.mma, a
-//     commit, a wait -- whatever the tile's width, so narrow tiles move few bytes per issue); the tensor pipe's time for
-//     128 x bn x 64 products; its share of the weight stream from HBM (what one SM pulls, ~55 GB/s, or HBM divided
+//   * per K slice of 64 elements a CTA needs the longest of: 0.3 us whatever the tile's width, so narrow tiles move few bytes per
+//     slice (a fitted figure, not the issuing thread's time: its four tcgen05.mma and commit alone take 0.10 us up to 64 columns
+//     and 0.13 at 128); the tensor pipe's time for 128 x bn x 64 products; its share of the weight stream from HBM (what one SM pulls, ~55 GB/s, or HBM divided
 //     among the CTAs of the wave; row tiles of one column tile share the weights through L2 -- above 128 rows the next
 //     term is always the longer one); the stage's bytes over what an SM takes in from L2 (~100 GB/s); and the ring's
 //     turn-round (a slot is refilled ~1.3 us after its products retire, so few deep stages starve the issuer);
 //   * a shared-out K range writes and re-reads float32 partial sums and runs the finishing kernel.
-// The constants were fitted to 70 points of this kernel on 7B- and 8B-shaped projections (26 and 256 rows).  Against 2812
-// measured points -- eleven shapes from 2048 x 2560 to 13824 x 5120, plain and gated, 2 to 512 rows, the candidates that
-// the model holds for the best -- its choice takes 1.5 % longer than the best one on average up to 128 rows (12.7 % at worst:
-// 2048 x 2560 at 48 rows, 8.7 against 7.7 us; with 80 GB/s per SM 2.7 % on average), and 3.7 % above (24 % at worst:
-// 2048 x 2560 at 160 rows, 13.5 against 10.8 us; 13824 x 5120 at 256 rows 53.9 against 46.1 us: shares of 112 columns
-// and two row tiles are dearer in the model than on the GPU).
+// The constants were fitted to 70 points of an earlier form of this kernel on 7B- and 8B-shaped projections (26 and 256 rows).
+// Against 1848 measured points of the present one -- eleven shapes from 2048 x 2560 to 13824 x 5120, plain and gated, twelve
+// row counts from 2 to 512, the 14 candidates that the model holds for the best -- its choice takes 2.0 % longer than the best one on
+// average up to 128 rows (20 % at worst: 13824 x 5120 at 2 rows, 33.6 against 28.0 us), and 1.7 % above (8.4 % at worst: 8192 x
+// 4096 at 160 rows, 22.0 against 20.3 us).
 struct LnPlan {
     int bn, splits, x_rows, stages, cols_per_tile, m_tiles, n_tiles, nm;
 };

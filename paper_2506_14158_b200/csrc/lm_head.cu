@@ -39,8 +39,8 @@ constexpr int kLmMaxParts = 160;  // CTAs of a launch: one per SM, at most this 
 template <int NM>
 struct LmCfg {
     static constexpr int kMaxBN = NM == 2 ? 128 : 256;
-    // cut into stages at launch: a stage holds the rows and tokens that exist.  As large as fits (192 KB, five stages instead of six of
-    // 224 tokens: 128256 x 4096, 54 rows 162.3 against 157.8 us)
+    // cut into stages at launch: a stage holds the rows and tokens that exist.  As large as fits (head and merge, 192 against 216 KB: 128256 x 4096, 54
+    // rows, five against six stages of 224 tokens, 168.3 against 163.0 us; 32000 x 4096, 26 rows 45.4 both)
     static constexpr int kRingBytes = 216 * 1024;
     static constexpr int kMaxStages = 12;
     static constexpr int kTmemCols = 2 * NM * kMaxBN;  // two accumulator buffers: all 512 columns

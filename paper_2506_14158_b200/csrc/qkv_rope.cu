@@ -27,7 +27,8 @@ constexpr int kQkBM = 128;       // rows per CTA (tensor-memory lanes)
 constexpr int kQkBK = 64;        // hidden elements per stage (one 128-byte swizzled row)
 constexpr int kQkMaxStages = 12;
 // Cut into stages at launch: a stage holds the rows that exist and the head's d weight rows.  As large as fits: it is what the CTA has
-// requested of its weights before the kernel in front has ended (192 KB: 32 + 2 x 32 heads of 4096 x 128, 26 rows 18.8 against 18.4 us)
+// requested of its weights before the kernel in front has ended (a chain of such calls, 192 against 216 KB: 32 + 2 x 32 heads of 4096 x 128, 26 rows
+// 19.14 against 18.75 us; 40 + 2 x 40 of 5120 x 128 26.8 against 26.4; 256 rows of 32 + 2 x 8 heads 18.7 both)
 constexpr int kQkRingBytes = 216 * 1024;
 constexpr int kQkRoleWarps = 4;  // weight producer, issuer, state producer, one without a role: the epilogue warps start at a multiple of four
 constexpr int kQkThreads = 32 * (kQkRoleWarps + 8);  // two epilogue warps per tensor-memory quarter (32 rows)
@@ -82,6 +83,8 @@ qkv_prep_kernel(const int32_t* __restrict__ cache_len, const int32_t* __restrict
     }
 }
 
+// (168 registers a thread: the whole register file but a sliver, so a CTA starts only where no finishing CTA of the product in front runs
+// any more)
 __global__ void __launch_bounds__(kQkThreads, 1)
 qkv_rope_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const QkParams prm) {
     constexpr int SM = kQkMaxStages;

@@ -310,18 +310,22 @@ __device__ __forceinline__ void chain_eval(double p0, double q0, int v, int r, c
 }
 
 // ============================================================================= cluster path
-// The default path when V is a multiple of 4 and at most 8 * 1024 * 16: one thread-block cluster of 8 CTAs per
-// (sequence, node) row keeps the row's logits in registers, so every logit and every draft probability is read
-// from HBM exactly once and exponentiated exactly once; the row-wide maximum, sum and residual mass are merged
-// across the cluster through distributed shared memory in CTA-rank order (deterministic).  The walk then runs
-// as one cluster per sequence, its vocabulary-wide passes spread over the 8 CTAs.
+// Statistics, when V is a multiple of 4, above 4096 (shorter rows are one segment: see the launch) and at most 8 * 1024 * 16, and the
+// problem is small (kSegStatsMinElems): one thread-block cluster of 8 CTAs per (sequence, node) row keeps the row's logits
+// in registers, so every logit and every draft probability is read from HBM exactly once and exponentiated exactly once;
+// the row-wide maximum, sum and residual mass are merged across the cluster through distributed shared memory in CTA-rank
+// order (deterministic).  The walk runs as one cluster per sequence whichever statistics it has, its vocabulary-wide passes
+// spread over 8 CTAs, 16 where rows are long, or left to one where they are short.
 constexpr int kCl = 8;             // CTAs per cluster
 constexpr int kClEpt = 16;         // row elements per thread
 constexpr int kClMaxThreads = 1024;
 constexpr int kWalkMaxCl = 16;     // most CTAs of a walk (see the launch)
 constexpr int kWalkGroup = 128;    // vocabulary entries that a warp of the walk takes at once: four per lane
 constexpr int kClMaxV = kCl * kClMaxThreads * kClEpt;
-constexpr size_t kSegStatsMinElems = (size_t)8 << 20;  // B*T*V above which the segment kernels win (measured)
+// B*T*V above which the segment kernels win: drawn for the walk as it was when a pass took three times as long.  With today's walk the
+// line lies too high (cold L2, clusters against segments: 8 x 26 rows of 32000 80 against 45 us, 16 x 64 rows of 6144 270 against 49, 1 x 15 of
+// 16384 22.5 both).
+constexpr size_t kSegStatsMinElems = (size_t)8 << 20;
 
 __device__ __forceinline__ uint32_t cl_rank() {
     uint32_t r;
@@ -912,7 +916,7 @@ accept_walk_cluster_kernel(const float* __restrict__ logits, const float* __rest
     }
 }
 
-constexpr int kWalkWideV = 65536;  // rows from here on: 16 entries and more for each thread of 8 CTAs
+constexpr int kWalkWideV = 65536;  // rows from here on: eight entries and more for each thread of 8 CTAs (measured on both sides, see the launch)
 constexpr size_t kWalkState = ((sizeof(WalkClShared) + 15) / 16) * 16, kWalkSmemMax = 227 * 1024;
 
 // How many walks of 16 CTAs run at once (0: clusters of that size are not to be had here), asked of the device once: a cluster
@@ -975,8 +979,10 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
 
     // ---- per-node statistics: row-in-registers clusters for small problems (one launch, latency-bound), vocabulary
     //      segments of 4096 with many CTAs per SM for large ones (two launches, throughput-bound).  A row that is one segment goes
-    //      that way too: there is nothing to share out over a cluster, whose four barriers are most of the time (15 rows of 1000 with
-    //      the walk by one CTA as well, see below: 16.4 -> 12.3 us).
+    //      that way too: there is nothing to share out over a cluster, whose four barriers are most of the time.  With the walk by one CTA
+    //      as well (see below), both calls, cold L2, clusters against one segment: 1 x 15 rows of 1000 26.7 against 24.6 us, 30.7 both where
+    //      every test is rejected that can be; 1 x 64 of 4096 36.9 against 26.6; 8 x 26 of 4096 67.7 against 26.7; 16 x 64 of 64 to 4096
+    //      250-274 against 29-49; at 48 points (V from 64 to 4096, 1 to 64 sequences, few and many rejections) slower at none.
     const bool seg_stats = !(vec && V <= kClMaxV) || (size_t)B * T * V > kSegStatsMinElems || splits == 1;
     const int chunk = (int)round_up((size_t)ceil_div(V, kCl), 4);
     const float floor_span = kExpFloorSpan * (stoch ? temperature : 1.f);
@@ -1030,9 +1036,17 @@ extern "C" s4c_status s4c_tree_accept(const float* target_logits, const float* d
     const RowPartial* seg_row = seg_stats ? ws.row : nullptr;
     if (stoch) {
         // A pass over one row is what the walk consists of, so a long row goes to 16 CTAs where as many clusters of 16 run at once as
-        // there are sequences (4 x 64 rows of 128256, cold L2: the call 98 -> 88 us; 32000 entries are four for a thread of 8 CTAs
-        // already).
-        // Up to 4096 entries are four for a thread of one CTA, and then nothing has to be exchanged.
+        // there are sequences: 7 on the GPU measured.  The call, cold L2, 8 against 16 CTAs, every test rejected that can be:
+        //   V       1 x 26          4 x 64          7 x 32          8 x 32 (more than run at once: not taken)
+        //   32000   32.8 | 34.8     94.2 | 96.3     84.0 | 84.0     92.2 | 98.3
+        //   49152   30.7 | 30.7     65.5 | 59.4     63.5 | 57.4     69.6 | 63.5
+        //   65536   45.1 | 43.0     59.4 | 55.3     61.4 | 55.3     65.5 | 69.6
+        //   128256  69.6 | 61.4     86.0 | 77.9     92.2 | 82.0     94.2 | 98.3
+        //   256000  121 | 66        217 | 129 (39)  156 | 109 (22)  182 | 139 (19 rows)
+        // From 65536 on 16 are faster at every batch that takes them, rejections or not; at 32000 they are slower, in between it varies
+        // by 2 us either way where few tests are rejected.
+        // Up to 4096 entries are four for a thread of one CTA, and then nothing has to be exchanged.  (At 8192 one CTA is as fast as 8 on
+        // the same segments, 1 x 64 rows 32.8 both, at 16384 slower: 38.9 against 30.7.)
         const int n_cl = splits == 1 ? 1 : (V >= kWalkWideV && B <= walk_wide_clusters() ? kWalkMaxCl : kCl);
         const int chunk = (int)round_up((size_t)ceil_div(V, n_cl), 4);
         attr[0].val.clusterDim.x = n_cl;

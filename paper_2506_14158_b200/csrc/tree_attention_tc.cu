@@ -1179,7 +1179,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         //      lane, offsets and weights by shuffles: 2 us for every two to four rows of a warp, most of it instructions.)  The
         //      partials of this CTA come from its own shared memory, the others through distributed shared memory, whose path is
         //      slow: about a microsecond a read, 7 to 12 bytes per clock for an SM when all pull at once.  16 x 8 pairs of 104 rows in
-        //      two turns, L=2000: 34.3 -> 28.2 us per launch; 4 x 8 pairs of 256 rows, four splits, L=4096: 27.7 -> 26.8 us.
+        //      two turns, L=2000: 34.3 -> 28.4 us per launch; 4 x 8 pairs of 256 rows, four splits, L=4096: 27.7 -> 26.8 us.
         __syncwarp();
         if (splits > 1) {
             cluster_sync_all();
