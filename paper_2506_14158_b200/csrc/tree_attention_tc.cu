@@ -1036,12 +1036,13 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     // With no other split to merge it with, the merged partial is written as output (the steps of the merge below, with
                     // one partial; 192 pairs of one row, two CTAs per SM, L=1024: 25.5 -> 22.4 us per launch; 320 pairs of 26 rows:
                     // 49.9 -> 43.3); else it becomes one exchange row, pushed to the row's owner or left behind the parked copies, where
-                    // the peers will fetch it.  (A CTA that gave up a wait stores no output; every warp has passed its waits here.)
+                    // the peers will fetch it.  (A CTA that gave up a wait stores no output, nor does one that met a page outside the pool:
+                    // every tile has been consumed here, so every wait is over and every page was looked at -- `run` is older than that.)
                     const int gr = mt0 * kBM + r;
                     const bool valid = n == T || gr % T < n;
                     const float w1 = exp2f(M - M) * den, inv = (valid && w1 > 0.f) ? 1.f / w1 : 0.f;
                     __nv_bfloat16* out = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + col0;
-                    const bool store_out = run && !*dead;
+                    const bool store_out = run && !*reinterpret_cast<volatile int*>(bad_s) && !*dead;
                     const unsigned char* src = base_ptr + (size_t)r * XS + col0 * 2;
                     unsigned char* xo = base_ptr + Cfg::kXBytes + (size_t)r * XS;
 #pragma unroll 1

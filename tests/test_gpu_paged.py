@@ -80,6 +80,31 @@ def test_a_page_outside_the_pool_flags_the_sequence_and_touches_nothing_else():
     assert np.abs(out[:1].double().cpu().numpy() - ref).max() <= ATTN_TOL["bf16"]
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,T,L", [(2, 4, 4, 10, 100), (10, 32, 32, 20, 600), (20, 8, 8, 33, 600)])
+def test_rows_of_a_sequence_with_a_bad_page_are_left_untouched_in_unsplit_launches(B, Hq, Hkv, T, L):
+    # one CTA per head, four or two copies of its rows: it looks at every page of the sequence before it stores a row.  The bad page
+    # is the first one (met at once) or the last one (beyond the ring's first pass where the sequence has ten pages).
+    from paper_2506_14158_b200 import s4c
+
+    d, ps, nb = 128, 64, (L + T + 63) // 64
+    g = torch.Generator(device="cuda").manual_seed(10)
+    q = torch.randn((B, Hq, T, d), generator=g, device="cuda").bfloat16()
+    kp = torch.randn((B * nb, Hkv, ps, d), generator=g, device="cuda").bfloat16()
+    good = np.arange(B * nb, dtype=np.int32).reshape(B, nb)
+    args = dev(np.full(B, L, np.int32)), dev(np.tile(W.chain_tree(T), (B, 1)))
+    whole = s4c.tree_attention_paged(q, kp, kp, dev(good), *args)
+    for page in (0, nb - 1):
+        bt = good.copy()
+        bt[1, page] = B * nb
+        st = torch.full((B,), -1, dtype=torch.int32, device="cuda")
+        out = torch.full((B, Hq, T, d), 7.0, dtype=torch.bfloat16, device="cuda")
+        s4c.tree_attention_paged(q, kp, kp, dev(bt), *args, out=out, status=st)
+        assert st.cpu().tolist() == [s4c.SEQ_BAD_PAGE if b == 1 else 0 for b in range(B)]
+        assert bool((out[1] == 7.0).all()), page
+        rest = [b for b in range(B) if b != 1]
+        assert torch.equal(out[rest], whole[rest])
+
+
 @pytest.mark.parametrize("bad", [None, 0, 100, 194])
 def test_a_page_outside_the_pool_is_flagged_where_the_splits_are_no_cluster(bad):
     # two row tiles of one sequence on more than 24k slots: the splits meet in a workspace, and end in any order
