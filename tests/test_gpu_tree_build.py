@@ -12,7 +12,7 @@ from parity import Guarded, dev
 pytestmark = pytest.mark.gpu
 
 
-def _both(q, branching, root, L):
+def _both(q, branching, root, L, ranked=None):
     from paper_2506_14158_b200 import s4c
 
     B, T, V = q.shape
@@ -24,7 +24,7 @@ def _both(q, branching, root, L):
     torch.cuda.synchronize()
     for name, buf in g.items():
         buf.check("s4c_tree_build " + name)
-    ref = oracle.build_tree(q, branching, root, L)
+    ref = oracle.build_tree(q if ranked is None else ranked, branching, root, L)
     for key in ("tokens", "parent", "position", "n_nodes"):
         np.testing.assert_array_equal(r[key].cpu().numpy(), ref[key], err_msg=key)
     return ref
