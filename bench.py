@@ -114,8 +114,8 @@ def algorithmic_bytes(cfg, temperature, accept_lens):
     attn_layer = 2 * cfg.B * cfg.Hkv * (cfg.L + cfg.T) * cfg.d * s + 2 * cfg.B * cfg.Hq * cfg.T * cfg.d * s
     rows = sum(int(a) + 1 for a in accept_lens)
     accept = cfg.B * cfg.T * cfg.V * (8 if temperature > 0 else 4)
-    if temperature > 0 and (cfg.B * cfg.T * cfg.V > (8 << 20) or cfg.V % 4 or cfg.V > 131072):
-        # large problems: the residual masses are computed on the walked rows only, so the draft probabilities of the
+    if temperature > 0 and (cfg.B * cfg.T * cfg.V > (8 << 20) or cfg.V % 4 or cfg.V > 131072 or cfg.V <= 4096):
+        # large problems and rows of one segment: the residual masses are computed on the walked rows only, so the draft probabilities of the
         # other rows are never needed: every logits row once, logits and draft probabilities of the walked rows once more
         accept = cfg.B * cfg.T * cfg.V * 4 + rows * cfg.V * 8
     compact = cfg.n_layers * 2 * 2 * cfg.Hkv * rows * cfg.d * s + 2 * rows * cfg.hid * s
