@@ -1042,7 +1042,7 @@ tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     const bool valid = n == T || gr % T < n;
                     const float w1 = exp2f(M - M) * den, inv = (valid && w1 > 0.f) ? 1.f / w1 : 0.f;
                     __nv_bfloat16* out = prm.out + out_row_offset<ROWS>(prm, b, hk * G, gr, T, D) + col0;
-                    const bool store_out = run && !*reinterpret_cast<volatile int*>(bad_s) && !*dead;
+                    const bool store_out = splits == 1 && run && (*reinterpret_cast<volatile int*>(bad_s) | *dead) == 0;
                     const unsigned char* src = base_ptr + (size_t)r * XS + col0 * 2;
                     unsigned char* xo = base_ptr + Cfg::kXBytes + (size_t)r * XS;
 #pragma unroll 1
